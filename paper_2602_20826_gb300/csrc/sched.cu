@@ -7,11 +7,10 @@
 // of Alg.2 and the bound of Theorem 1. The schedule is written out as "plan rows" that the
 // candidate-bound kernel evaluates other allocations on.
 //
-// Alg.2 is sequential over the groups of a DAG. Groups with few members (the common case)
-// are scheduled by one thread of the team with plain loads and stores and no team-wide
-// barrier; large groups use the whole team.
+// Alg.2 is sequential over the groups of a DAG: one warp of the team runs it.
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "dagrt_internal.cuh"
@@ -20,9 +19,11 @@
 namespace dagrt {
 
 // node state bits
-enum : uint8_t { ST_ACTIVE = 1, ST_INT = 2, ST_SEL = 4, ST_DONE = 8, ST_LAUNCH = 16, ST_JOIN = 32 };
+enum : uint8_t { ST_ACTIVE = 1, ST_INT = 2, ST_SEL = 4, ST_JOIN = 32 };
 constexpr uint16_t NONE16 = 0xffff;
-constexpr int kSumWords = 8;  // released-set masks longer than this keep a summary of non-empty words
+constexpr int kRelWords = (DAGRT_MAX_V + 63) / 64;  // words of the largest released-set mask
+constexpr int kRelBytes = 8 * (kRelWords + kRelWords / 64);  // ... and of its summary
+constexpr int kSumWords = 16;  // released-set masks longer than this keep a summary of non-empty words
 
 // ------------------------------------------------------------------ workspace layout
 // Persistent arrays live for the whole DAG; the region after them is overlaid by the
@@ -58,9 +59,8 @@ struct Ws {
     uint16_t *gtmp;
     int32_t *gfill;
     // phase E
-    uint32_t *rem, *cfull;
-    uint16_t *mm;
-    int32_t *lst, *tmp;
+    uint4 *rc;  // node records and counters by rank (struct A2)
+    uint16_t *lst, *mm;
     // phase F (after Alg.2): the critical-path lower bound
     uint64_t *cpT, *cpM;
 };
@@ -136,11 +136,9 @@ __host__ __device__ inline int64_t ws_carve(unsigned char *base, int vc, int ec,
     w.gfill = (int32_t *)take(4ll * (vc + 1));
     mark();
     off = x0;
-    w.rem = (uint32_t *)take(4ll * vc);
-    w.cfull = (uint32_t *)take(4ll * vc);
+    w.rc = (uint4 *)take(16ll * vc);
+    w.lst = (uint16_t *)take(2ll * vc);
     w.mm = (uint16_t *)take(2ll * vc);
-    w.lst = (int32_t *)take(4ll * (vc + 1));
-    w.tmp = (int32_t *)take(4ll * vc);
     mark();
     off = x0;
     w.cpT = (uint64_t *)take(8ll * vc);
@@ -158,18 +156,14 @@ struct Dag {
     int V, W, variant;
     uint32_t M;
     bool want_edges;
-    const uint32_t *rp;  // staged CSR
-    const uint16_t *col;
 };
 
-// Alg.2 running totals, held by the team's first thread
+// Alg.2's totals, valid in the team's first warp
 struct Acc {
     uint64_t bound;
     int64_t nextra;
-    int nrows, nseg, nrel;  // plan rows, segments, released-and-unfinished nodes
+    int nrows, nseg, nrel;  // plan rows, segments; in: nodes released at the start
     bool err;
-    int lastr;       // the last plan row written by this thread (-1: unknown) ...
-    uint32_t lastz;  // ... and its packed m | k << 16, to mark it as the group's last row
 };
 
 __device__ inline void write_failure(const SchedArgs &a, int d, int code) {
@@ -203,437 +197,567 @@ __device__ __forceinline__ uint64_t sat_add(uint64_t a, uint64_t b) {
     return s > (uint64_t)INT64_MAX || s < a ? (uint64_t)INT64_MAX : s;
 }
 
-// plan row r: `id` is the node (< V) or segment (>= V) it runs, `owner` the node whose
-// allocation it uses (the segment's parent for a segment)
-__device__ inline uint32_t write_row(const SchedArgs &a, const Dag &g, int r, int id, int owner, int group,
-                                     uint32_t load, uint32_t k, uint32_t m, uint64_t c) {
-    const uint32_t z = m | (k << 16);
-    if (r >= 2 * g.V) return z;
-    const int64_t i = g.rbase + r;
-    if (a.plan) a.plan[i] = make_uint4(load, (uint32_t)c, z, (uint32_t)owner);
-    if (a.o.row_id) a.o.row_id[i] = id;
-    if (a.o.row_group) a.o.row_group[i] = group;
-    if (a.o.row_m0) a.o.row_m0[i] = (int32_t)m;
-    if (a.o.row_load) a.o.row_load[i] = load;
-    return z;
+// ------------------------------------------------------------------ Alg.2
+// Alg.2's working set in rank space: node r is the r-th in descending W^anc order (ties:
+// lower id), so the released set is a bit mask over r whose lowest bits come first, and an
+// edge leads from a rank to a smaller one.
+//
+// The arrays are 32-bit offsets, from the kernel's dynamic shared memory (SH) or from a
+// global workspace: the compiler then knows the memory space of every access in the chain,
+// and the whole set costs ten registers.
+template <bool SH>
+struct A2 {
+    unsigned char *base;  // !SH: the global workspace
+    uint32_t o_rc, o_col, o_cnt, o_gstart, o_gmem, o_byrank, o_lst, o_mm;
+    uint32_t o_rel, o_sum;  // always in shared memory
+
+    template <class T>
+    __device__ __forceinline__ T *at(uint32_t off) const {
+        extern __shared__ __align__(16) unsigned char smem[];
+        if constexpr (SH) return (T *)(smem + off);
+        else return (T *)(base + off);
+    }
+    // {load left (0: finished), C at min(load left, M) SMs (0: recompute), first edge,
+    //  out-degree | k << 16}
+    __device__ __forceinline__ uint4 &rc(uint32_t r) const { return at<uint4>(o_rc)[r]; }
+    __device__ __forceinline__ uint32_t &left(uint32_t r) const { return at<uint32_t>(o_rc)[4 * r]; }
+    __device__ __forceinline__ uint16_t &col(uint32_t e) const { return at<uint16_t>(o_col)[e]; }  // successors by edge, as ranks
+    __device__ __forceinline__ uint16_t &cnt(uint32_t r) const { return at<uint16_t>(o_cnt)[r]; }  // predecessors not yet finished
+    __device__ __forceinline__ uint16_t &gstart(int j) const { return at<uint16_t>(o_gstart)[j]; }
+    __device__ __forceinline__ uint16_t &gmem(int i) const { return at<uint16_t>(o_gmem)[i]; }  // members of each group, as ranks, in id order
+    __device__ __forceinline__ uint16_t &byrank(uint32_t r) const { return at<uint16_t>(o_byrank)[r]; }
+    __device__ __forceinline__ uint16_t &lst(int i) const { return at<uint16_t>(o_lst)[i]; }  // launched nodes of the group
+    __device__ __forceinline__ uint16_t &mm(int i) const { return at<uint16_t>(o_mm)[i]; }    // SMs of a large group's members
+    // released and unfinished nodes, 32 ranks a word; SUM: bit w of sum set: 64-bit word w of
+    // rel may be non-zero (cleared lazily by the scan)
+    __device__ __forceinline__ uint32_t *rel() const {
+        extern __shared__ __align__(16) unsigned char smem[];
+        return (uint32_t *)(smem + o_rel);
+    }
+    __device__ __forceinline__ uint32_t *sum() const {
+        extern __shared__ __align__(16) unsigned char smem[];
+        return (uint32_t *)(smem + o_sum);
+    }
+};
+
+// Arithmetic of one DAG: NARROW if 64 M max C^ fits 32 bits, so that every product and sum
+// over a group below does (loads below 453,000 ticks at M = 148): 64-bit products and the
+// branch on the size of a division are a third of the group step's instructions otherwise.
+template <bool NARROW>
+struct Arith {
+    using T = typename std::conditional<NARROW, uint32_t, uint64_t>::type;
+    static __device__ __forceinline__ T div(T n, T d) {
+        if constexpr (NARROW) return n / d;
+        else return udiv(n, d);
+    }
+    static __device__ __forceinline__ T sum(uint32_t x) {  // over the warp
+        if constexpr (NARROW) return __reduce_add_sync(FULL, x);
+        else return ((uint64_t)__reduce_add_sync(FULL, x >> 16) << 16) + __reduce_add_sync(FULL, x & 0xffffu);
+    }
+    // Eq.5 before the repair: round(x M / Wg) half up, at least 1, at most x
+    static __device__ __forceinline__ uint32_t eq5(uint32_t x, uint32_t M, T Wg) {
+        const T r = div((T)2 * x * M + Wg, (T)2 * Wg);
+        return r < 1 ? 1u : (r < x ? (uint32_t)r : x);
+    }
+    // Eq.1 on m <= M SMs
+    static __device__ __forceinline__ uint32_t time(uint32_t x, uint32_t k, uint32_t m) {
+        const T num = (T)x * (64u * m - k * (m - 1));
+        return (uint32_t)div((num - 1) >> 6, m) + 1u;
+    }
+    // does load x finish within R on S <= M SMs?
+    static __device__ __forceinline__ bool fits(uint32_t x, uint32_t k, uint32_t S, T R) {
+        return (T)x * (64u * S - k * (S - 1)) <= (T)(64u * S) * R;
+    }
+    // the largest load p in [1, x - 1] that finishes within R on min(p, S) SMs, for an x that
+    // does not: on S SMs if that leaves at least S ticks, else on p SMs (k < 64 then)
+    static __device__ __forceinline__ uint32_t split(uint32_t x, uint32_t k, uint32_t S, T R) {
+        T p = div((T)(64u * S) * R, 64u * S - k * (S - 1));
+        if (p < S) p = min(div((T)64 * R - k, 64u - k), (T)(S - 1));
+        return (uint32_t)min(p, (T)(x - 1));
+    }
+};
+
+template <bool SH>
+__device__ __forceinline__ void clear_released(const A2<SH> &w, uint32_t r) {
+    atomicAnd(w.rel() + (r >> 5), ~(1u << (r & 31)));
 }
 
-// ------------------------------------------------------------------ Alg.2 pieces
-// Launch parallel nodes for group j (Alg.2's parallel-launch and segmentation step): released, unfinished nodes outside
-// pi_j in descending W^anc order (lowest rank first). One thread. Returns the number of
-// launched parts (ids in ws.lst; a segment id is >= V) and of whole-node launches.
-template <bool SUM>
-__device__ __forceinline__ void launch_parallel(const Ws &ws, const SchedArgs &a, const Dag &g, int j, uint64_t R, uint32_t S0,
-                                Acc &acc, int *nl_out, int *nwhole_out) {
-    int nl = 0, nwhole = 0;
+// The 32 lanes decrement the open-predecessor counts of a finished node's successors (its
+// edges [eb, eb + deg), targets distinct; `s` holds the first 32 edges' targets) and mark
+// the ones that reach zero as released; with COUNT, returns how many did.
+template <bool SUM, bool COUNT, bool SH>
+__device__ __forceinline__ int release_succ(const A2<SH> &w, uint32_t eb, uint32_t deg, uint32_t s, int lane) {
+    int n = 0;
+    for (uint32_t e = lane; __any_sync(FULL, e < deg); e += 32) {
+        bool z = false;
+        if (e < deg) {
+            if (e >= 32) s = w.col(eb + e);
+            const uint32_t c = w.cnt(s) - 1u;
+            w.cnt(s) = (uint16_t)c;
+            z = c == 0;
+            if (z) {
+                atomicOr(w.rel() + (s >> 5), 1u << (s & 31));
+                if constexpr (SUM) atomicOr(w.sum() + (s >> 11), 1u << ((s >> 6) & 31));
+            }
+        }
+        if constexpr (COUNT) n += __popc(__ballot_sync(FULL, z));
+    }
+    __syncwarp();  // counts and released bits before the next release or scan
+    return n;
+}
+
+// Extra dependencies of group j (Alg.2's segmentation step): (v_n, succ(v_R)) for every
+// launched part in launch order (the ranks in w.lst, then segment `seg` if one was cut) and
+// (v_R, v_n) for every parallel node left in the released set, the split node's residual
+// included. Before any node of the group is released from. One lane.
+template <bool SH>
+__device__ __noinline__ void write_extra_edges(const A2<SH> w, int32_t *src, int32_t *dst, int64_t cap,
+                                               int V, uint32_t vR, int nwhole, int seg, int64_t idx) {
+    const uint4 q = w.rc(vR);
+    const uint32_t deg = q.w & 0xffffu;
+    const int id = w.byrank(vR);
+    for (int i = 0; i < nwhole + (seg >= 0); i++)
+        for (uint32_t e = q.z; e < q.z + deg; e++, idx++)
+            if (idx < cap) {
+                src[idx] = i < nwhole ? (int)w.byrank(w.lst(i)) : V + seg;
+                dst[idx] = w.byrank(w.col(e));
+            }
+    for (int i = 0; i < (V + 31) / 32; i++)
+        for (uint32_t bits = w.rel()[i]; bits; bits &= bits - 1, idx++)
+            if (idx < cap) {
+                src[idx] = id;
+                dst[idx] = w.byrank(i * 32 + __ffs(bits) - 1);
+            }
+}
+
+// Members of a group of more than 32: Eq.5 with the repair, Eq.1 and Lemma 1, 32 members at
+// a time. The SMs go to w.mm, C to the members' records; members leave the released set.
+// Returns the unfinished members; with one only, *vR is that member and nothing else is set.
+template <bool SH>
+__device__ __noinline__ int members_large(const A2<SH> w, int variant, uint32_t M, int gb, int n, int lane, uint64_t *R,
+                                          uint32_t *vR, uint32_t *sum_m) {
+    using Ar = Arith<false>;
+    int np = 0;
+    uint64_t Wg = 0;
+    uint32_t one = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const uint32_t r = i0 + lane < n ? w.gmem(gb + i0 + lane) : 0;
+        const uint32_t x = i0 + lane < n ? w.rc(r).x : 0;
+        const uint32_t live = __ballot_sync(FULL, x > 0);
+        if (live) one = __shfl_sync(FULL, r, __ffs(live) - 1);
+        np += __popc(live);
+        Wg += Ar::sum(x);
+    }
+    *vR = one;
+    if (np < 2) return np;
+    uint32_t sum = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const uint32_t r = i < n ? w.gmem(gb + i) : 0;
+        const uint32_t x = i < n ? w.rc(r).x : 0;
+        const uint32_t m = x ? Ar::eq5(x, M, Wg) : 0;
+        if (i < n) w.mm(i) = (uint16_t)m;
+        if (x) clear_released(w, r);
+        sum += __reduce_add_sync(FULL, m);
+    }
+    __syncwarp();
+    if (variant != DAGRT_VAR_NOREPAIR && sum > M) {
+        // taking one SM at a time from the largest m (ties: higher id) t times leaves every
+        // m at most L + 1, L the largest level with sum max(0, m - L) >= t, and then takes
+        // the rest from the members still at L + 1, highest id first
+        const uint32_t t = sum - M;
+        uint32_t lo = 0, hi = M;  // above(lo) >= t > above(hi)
+        auto above = [&](uint32_t L) {
+            uint32_t s = 0;
+            for (int i0 = 0; i0 < n; i0 += 32) {
+                const uint32_t m = i0 + lane < n ? w.mm(i0 + lane) : 0;
+                s += __reduce_add_sync(FULL, m > L ? m - L : 0);
+            }
+            return s;
+        };
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (above(mid) >= t) lo = mid;
+            else hi = mid;
+        }
+        uint32_t left = t - above(lo + 1);
+        __syncwarp();
+        for (int i0 = (n - 1) & ~31; i0 >= 0; i0 -= 32) {
+            const uint32_t m = i0 + lane < n ? w.mm(i0 + lane) : 0;
+            const uint32_t top = __ballot_sync(FULL, m > lo);
+            const uint32_t before = lane < 31 ? __popc(top >> (lane + 1)) : 0;
+            if (m > lo) w.mm(i0 + lane) = (uint16_t)(before < left ? lo : lo + 1);
+            left -= min(left, (uint32_t)__popc(top));
+        }
+        __syncwarp();
+        sum = M;
+    }
+    uint64_t csum = 0;
+    uint32_t Rm = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const uint32_t r = i < n ? w.gmem(gb + i) : 0;
+        const uint4 q = i < n ? w.rc(r) : make_uint4(0, 0, 0, 0);
+        uint32_t c = 0;
+        if (q.x) {
+            c = Ar::time(q.x, q.w >> 16, w.mm(i));
+            w.rc(r).y = c;
+        }
+        csum += Ar::sum(c);
+        const uint32_t cm = __reduce_max_sync(FULL, c);
+        const uint32_t at = __ballot_sync(FULL, c == cm);
+        if (cm > Rm) {
+            Rm = cm;
+            *vR = __shfl_sync(FULL, r, __ffs(at) - 1);
+        }
+    }
+    __syncwarp();
+    *sum_m = sum;
+    *R = sum > M ? csum : (uint64_t)Rm;  // over-full (no repair): members one after another
+    return np;
+}
+
+// Alg.2 over all groups of a DAG with Lemma 1 and Theorem 1, by one warp. The group step is
+// a serial chain, so it is written for latency: every lane runs the scalar part on the same
+// values (no divergence, no hand-over between lanes), a node's record is one 16-byte load,
+// the time of a whole launch comes precomputed (on x <= S SMs it is C at min(x, M) SMs), a
+// segment's time is R itself (below), and the successors of a finished node are counted
+// down by the 32 lanes with plain loads and stores while the first candidate's record is on
+// its way. Ranks instead of ids take the lookups out of the chain: the released set is one
+// 32-bit word per lane (up to 1,024 nodes) or a mask with a summary word per lane (SUM).
+//
+// A segment p is the largest load that finishes within R on min(p, S) SMs, and adding one
+// tick of load adds at most one tick of time: the part takes exactly R.
+//
+// What bounds it: the latency of one warp's dependent instructions (a third of the stalls are
+// shared-memory loads, the rest fixed-latency arithmetic). Against one lane walking id-indexed
+// arrays, a group went from 3,800 to 2,100-2,500 cycles and a call of 10,000 DAGs of 20-200
+// nodes from 1.80 to 1.42 ms; 300 DAGs of 100-1,000 nodes from 3.7 to 2.4 ms.
+//
+// FULL_OUT: some of the outputs that few callers ask for (rows, segments, group times, extra
+// dependencies) are wanted; without it the chain does not carry what only they need.
+template <bool SUM, bool SH, bool NARROW, bool FULL_OUT>
+__device__ __forceinline__ void alg2_warp(const A2<SH> &w, const SchedArgs &a, const Dag &g, int G, Acc &acc, int lane) {
+    using Ar = Arith<NARROW>;
+    using T = typename Ar::T;
     const uint32_t M = g.M;
-    // no SMs left (S = 0, so also WS = 0): every variant stops at its first candidate
-    if (g.variant != DAGRT_VAR_NOPARA && S0 > 0) {
-        uint32_t S = S0;
-        uint64_t WS = R * (uint64_t)S0;  // Eq.6
-        bool stop = false;
-        // the mask's words in order (lowest rank first); a long mask (SUM) is walked through
-        // its summary of possibly non-empty words
-        int w = -1, sw = -1;
-        uint64_t sbits = 0;
-        while (!stop) {
-            if constexpr (SUM) {
-                while (!sbits && ++sw < ((g.W + 63) >> 6)) sbits = ws.relsum[sw];
-                if (!sbits) break;
-                w = sw * 64 + __ffsll((long long)sbits) - 1;
-                sbits &= sbits - 1;
-            } else {
-                if (++w >= g.W) break;
-            }
-            uint64_t bits = ws.relmask[w];
-            if (SUM && !bits) {  // emptied since it was marked
-                ws.relsum[sw] &= ~(1ull << (w & 63));
-                continue;
-            }
-            while (bits) {
-                const int b = __ffsll((long long)bits) - 1;
-                bits &= bits - 1;
-                const int u = ws.byrank[w * 64 + b];
-                if (ws.group_of[u] == j) continue;  // a member of pi_j
-                const uint32_t load = ws.rem[u], k = ws.kk[u];
-                bool split = false;
-                uint32_t mu = 0;
-                uint64_t p = 0, c = 0;
-                if (g.variant == DAGRT_VAR_LITERAL) {
-                    if (WS == 0) { stop = true; break; }
-                    if (load > WS) {
-                        split = true;
-                        p = WS;
-                        mu = (uint32_t)(p < S ? p : S);
-                    } else {
-                        mu = load < S ? load : S;
-                        WS -= load;
-                        c = exec_time(load, k, mu, M);
-                    }
-                } else {
-                    if (S == 0) { stop = true; break; }
-                    mu = load < S ? load : S;
-                    // fits within R on mu <= M SMs: ceil(load (64mu - k(mu-1)) / (64mu)) <= R
-                    const uint64_t lhs = (uint64_t)load * (64ull * mu - (uint64_t)k * (mu - 1));
-                    if (lhs > 64ull * mu * R) {
-                        if (g.variant == DAGRT_VAR_NOSEG) continue;
-                        split = true;
-                        p = split_size(load, k, S, R);
-                        mu = (uint32_t)(p < S ? p : S);
-                    } else {
-                        c = exec_time(load, k, mu, M);
-                        S -= mu;
-                    }
-                }
-                if (split) {  // node segmentation: the parallel part runs now
-                    const int s = acc.nseg++;
-                    if (a.o.seg_parent) {
-                        a.o.seg_parent[g.n0 + s] = u;
-                        a.o.seg_load[g.n0 + s] = (int64_t)p;
-                        a.o.seg_m[g.n0 + s] = (int32_t)mu;
-                        a.o.seg_group[g.n0 + s] = j;
-                    }
-                    acc.lastr = acc.nrows;
-                    acc.lastz = write_row(a, g, acc.nrows++, g.V + s, u, j, (uint32_t)p, k, mu, exec_time(p, k, mu, M));
-                    ws.rem[u] = load - (uint32_t)p;
-                    ws.lst[nl++] = g.V + s;
-                    stop = true;
-                    break;
-                }
-                ws.st[u] |= ST_LAUNCH;
-                ws.mm[u] = (uint16_t)mu;
-                acc.lastr = acc.nrows;
-                acc.lastz = write_row(a, g, acc.nrows++, u, u, j, load, k, mu, c);
-                ws.lst[nl++] = u;
-                nwhole++;
-            }
+    const int variant = g.variant;
+    const bool node_out = a.o.m || a.o.exec_group;
+    const bool defer = FULL_OUT && g.want_edges;  // nothing is released before the extra edges are written
+    uint4 *plan = a.plan ? a.plan + g.rbase : nullptr;
+    uint64_t bound = 0;
+    int64_t nextra = 0;
+    int nrows = 0, nseg = 0, nrel = acc.nrel;
+    // plan row i runs `id` (a segment: >= V) of node `owner` with `load`; z = m | k << 16
+    auto write_row = [&](int i, int id, int owner, int j, uint32_t load, uint32_t z, uint32_t c, bool last) {
+        if (plan) plan[i] = make_uint4(load, c, z | (last ? 1u << 24 : 0u), (uint32_t)owner);
+        if constexpr (FULL_OUT) {
+            if (a.o.row_id) a.o.row_id[g.rbase + i] = id;
+            if (a.o.row_group) a.o.row_group[g.rbase + i] = j;
+            if (a.o.row_m0) a.o.row_m0[g.rbase + i] = (int32_t)(z & 0xffffu);
+            if (a.o.row_load) a.o.row_load[g.rbase + i] = load;
         }
-    }
-    if (a.plan && acc.nrows - 1 < 2 * g.V) {  // mark the last row of pi_j
-        if (acc.lastr == acc.nrows - 1)
-            a.plan[g.rbase + acc.nrows - 1].z = acc.lastz | (1u << 24);  // a plain store: no read back
-        else
-            a.plan[g.rbase + acc.nrows - 1].z |= 1u << 24;
-    }
-    if (acc.nrows > 2 * g.V || acc.nseg > g.V) acc.err = true;
-    *nl_out = nl;
-    *nwhole_out = nwhole;
-}
-
-// Extra dependencies (Alg.2's segmentation step): (v_n, succ(v_R)) for every launched part and
-// (v_R, v_n) for every unlaunched parallel node, the split node's residual included. The
-// count is always kept; the edges are written when requested. One thread.
-__device__ void extra_edges(const Ws &ws, const SchedArgs &a, const Dag &g, int j, int vR, int np, int nl,
-                            int nwhole, Acc &acc) {
-    if (g.variant == DAGRT_VAR_NOPARA) return;
-    const int outdeg = g.rp[vR + 1] - g.rp[vR];
-    if (g.want_edges) {
-        int64_t idx = acc.nextra;
-        for (int i = 0; i < nl; i++)
-            for (int e = g.rp[vR]; e < g.rp[vR + 1]; e++, idx++)
-                if (idx < g.ecap) {
-                    a.o.extra_src[g.ebase + idx] = ws.lst[i];
-                    a.o.extra_dst[g.ebase + idx] = g.col[e];
-                }
-        for (int w = 0; w < g.W; w++) {
-            uint64_t bits = ws.relmask[w];
-            while (bits) {
-                const int b = __ffsll((long long)bits) - 1;
-                bits &= bits - 1;
-                const int u = ws.byrank[w * 64 + b];
-                if (ws.group_of[u] == j || (ws.st[u] & ST_LAUNCH)) continue;
-                if (idx < g.ecap) {
-                    a.o.extra_src[g.ebase + idx] = vR;
-                    a.o.extra_dst[g.ebase + idx] = u;
-                }
-                idx++;
-            }
+    };
+    // node r finishes with group j on m SMs
+    auto finish = [&](uint32_t r, int id, int j, uint32_t m) {
+        w.left(r) = 0;
+        if (node_out) {
+            if (a.o.exec_group) a.o.exec_group[g.n0 + id] = j;
+            if (a.o.m) a.o.m[g.n0 + id] = (int32_t)m;
         }
-    }
-    acc.nextra += (int64_t)nl * outdeg + (int64_t)(acc.nrel - np - nwhole);
-}
-
-// Group j (any size in warp teams, at most 32 members in CTA teams): lane 0 of the team's
-// first warp runs Eq.5, Lemma 1, the parallel launches and the extra edges serially; the 32
-// lanes then release the finished nodes' successors together (the decrements commute).
-// `acc` is valid in lane 0 only.
-__device__ void group_serial(const Ws &ws, const SchedArgs &a, const Dag &g, int j, Acc &acc, int lane) {
-    int nf = 0;
-    uint64_t R = 0;
-    if (lane == 0) {
-        const uint32_t M = g.M;
-        const int gb = ws.gstart[j], ge = ws.gstart[j + 1];
-        int np = 0, vR = -1;
-        uint32_t sum_m = 0;
-        if (ge - gb == 1) {  // one member: Eq.5 gives m = min(C^, M)
-            const int v = ws.gmem[gb];
-            if (!(ws.st[v] & ST_DONE)) {
-                np = 1;
-                const uint32_t x = ws.rem[v], m = x < M ? x : M;
-                ws.mm[v] = (uint16_t)m;
-                sum_m = m;
-                const uint64_t c = x == ws.load[v] ? ws.cfull[v] : exec_time(x, ws.kk[v], m, M);
-                R = c;
-                vR = v;
-                acc.lastr = acc.nrows;
-                acc.lastz = write_row(a, g, acc.nrows++, v, v, j, x, ws.kk[v], m, c);
+    };
+    int gn = w.gstart(0);
+    int ge = w.gstart(1);
+    uint32_t rn = w.gmem(gn);
+    for (int j = 0; j < G; j++) {
+        const int gb = gn, n = ge - gb;
+        uint32_t r = rn;  // one member: its rank; up to 32: one per lane
+        gn = ge;          // the next group's bounds and first member
+        if (j + 1 < G) {
+            ge = w.gstart(j + 2);
+            rn = w.gmem(gn);
+        }
+        // ---- members: Eq.5, Eq.1, Lemma 1
+        int np;
+        T R = 0;
+        uint32_t sum_m = 0, vR = 0;
+        uint4 q = make_uint4(0, 0, 0, 0);
+        uint32_t m = 0, c = 0, live = 0;
+        if (n == 1) {
+            q = w.rc(r);
+            np = q.x > 0;
+        } else if (n <= 32) {
+            if (lane < n) {
+                r = w.gmem(gb + lane);
+                q = w.rc(r);
             }
-        } else {
-            uint64_t Wg = 0;
-            for (int i = gb; i < ge; i++) {
-                const int v = ws.gmem[i];
-                if (!(ws.st[v] & ST_DONE)) {
-                    np++;
-                    Wg += ws.rem[v];
+            live = __ballot_sync(FULL, q.x > 0);
+            np = __popc(live);
+            if (np > 1) {
+                const T Wg = Ar::sum(q.x);
+                if (q.x) {
+                    m = Ar::eq5(q.x, M, Wg);
+                    clear_released(w, r);
                 }
-            }
-            if (np > 0) {
-                // Eq.5; a single member gets round(C^ M / C^) = M, i.e. m = min(C^, M)
-                for (int i = gb; i < ge; i++) {
-                    const int v = ws.gmem[i];
-                    if (ws.st[v] & ST_DONE) continue;
-                    const uint32_t x = ws.rem[v];
-                    uint32_t m;
-                    if (np == 1) {
-                        m = x < M ? x : M;
-                    } else {
-                        const uint64_t num = 2ull * x * M + Wg, den = 2ull * Wg;
-                        uint64_t r = (num >> 32) == 0 && (den >> 32) == 0 ? (uint64_t)((uint32_t)num / (uint32_t)den)
-                                                                          : num / den;
-                        if (r < 1) r = 1;
-                        m = (uint32_t)(r < x ? r : x);
-                    }
-                    ws.mm[v] = (uint16_t)m;
-                    sum_m += m;
-                }
-                // keep sum m_i <= M: trim the largest m (ties: higher id); the no-repair
+                sum_m = __reduce_add_sync(FULL, m);
+                // keep sum m <= M: take from the largest m (ties: higher id); the no-repair
                 // variant leaves the rounded SMs as they are
-                while (g.variant != DAGRT_VAR_NOREPAIR && sum_m > M) {
-                    int best = -1;
-                    for (int i = gb; i < ge; i++) {
-                        const int v = ws.gmem[i];
-                        if (ws.st[v] & ST_DONE) continue;
-                        if (best < 0 || ws.mm[v] >= ws.mm[best]) best = v;
-                    }
-                    ws.mm[best]--;
+                while (sum_m > M && variant != DAGRT_VAR_NOREPAIR) {
+                    const uint32_t top = __reduce_max_sync(FULL, (m << 5) | (uint32_t)lane);
+                    m -= (top & 31u) == (uint32_t)lane;
                     sum_m--;
                 }
-                // Eq.1 per member and Lemma 1: R(pi_j) = max C_i, v_R = lowest id with C_i = R
-                uint64_t csum = 0;
-                for (int i = gb; i < ge; i++) {
-                    const int v = ws.gmem[i];
-                    if (ws.st[v] & ST_DONE) continue;
-                    const uint32_t x = ws.rem[v], m = ws.mm[v];
-                    const uint64_t c =
-                        (x == ws.load[v] && m == (x < M ? x : M)) ? ws.cfull[v] : exec_time(x, ws.kk[v], m, M);
-                    csum += c;
-                    if (c > R) {
-                        R = c;
-                        vR = v;
-                    }
-                    acc.lastr = acc.nrows;
-                    acc.lastz = write_row(a, g, acc.nrows++, v, v, j, x, ws.kk[v], m, c);
-                }
-                if (sum_m > M) R = csum;  // over-full (no repair): members one after another
+                if (q.x) c = q.y && m == min(q.x, M) ? q.y : Ar::time(q.x, q.w >> 16, m);
+                const uint32_t Rm = __reduce_max_sync(FULL, c);
+                if constexpr (FULL_OUT) vR = __shfl_sync(FULL, r, __ffs(__ballot_sync(FULL, c == Rm)) - 1);
+                R = Rm;
+                if (sum_m > M) R = Ar::sum(c);  // over-full (no repair): members one after another
+                __syncwarp();
+            } else if (np == 1) {
+                r = __shfl_sync(FULL, r, __ffs(live) - 1);
+                q = w.rc(r);
+            }
+        } else {
+            uint64_t RL;
+            np = members_large(w, variant, M, gb, n, lane, &RL, &vR, &sum_m);
+            if (np == 1) {
+                r = vR;
+                q = w.rc(r);
+            } else {
+                R = (T)RL;
             }
         }
         if (np == 0) {  // every member already ran as a parallel node: the group is dropped
-            if (a.o.group_R) a.o.group_R[g.n0 + j] = 0;
-        } else {
-            int nl, nwhole;
-            const uint32_t S0 = sum_m < M ? M - sum_m : 0u;
-            if (g.W > kSumWords)
-                launch_parallel<true>(ws, a, g, j, R, S0, acc, &nl, &nwhole);
-            else
-                launch_parallel<false>(ws, a, g, j, R, S0, acc, &nl, &nwhole);
-            extra_edges(ws, a, g, j, vR, np, nl, nwhole, acc);
-            nf = ge - gb + nl;  // candidates to finish: the members, then the launched parts
-            if (a.o.group_R) a.o.group_R[g.n0 + j] = (int64_t)R;
-            acc.bound += R;
+            if constexpr (FULL_OUT)
+                if (a.o.group_R && lane == 0) a.o.group_R[g.n0 + j] = 0;
+            continue;
         }
-    }
-    __syncwarp();  // lane 0's shared-memory writes (launch list, states) become visible
-    // members (not finished before) and whole launches finish with pi_j: one lane each
-    const int gb = __shfl_sync(FULL, lane == 0 ? (int)ws.gstart[j] : 0, 0);
-    const int ncand = __shfl_sync(FULL, nf, 0);
-    int nfin = 0;
-    for (int base = 0; base < ncand; base += 32) {
-        const int i = base + lane;
-        int v = -1;
-        if (i < ncand) {
-            const int ge = ws.gstart[j + 1];
-            if (gb + i < ge) {
-                v = ws.gmem[gb + i];
-                if (ws.st[v] & ST_DONE) v = -1;
+        const uint32_t deg = q.w & 0xffffu;
+        uint32_t s0 = 0, mw = 0;
+        if (np == 1) {  // Eq.5 gives m = min(C^, M)
+            if ((uint32_t)lane < deg) s0 = w.col(q.z + lane);
+            m = min(q.x, M);
+            c = q.y;
+            if (c == 0) c = Ar::time(q.x, q.w >> 16, m);  // the rest of a split node
+            sum_m = m;
+            R = c;
+            vR = r;
+        }
+        // ---- parallel launches and node segmentation: released, unfinished nodes outside
+        //      pi_j in rank order
+        const int nrel0 = nrel;
+        int nwhole = 0, seg = -1;
+        const bool early = !SUM && np == 1 && !defer;
+        uint32_t S = sum_m < M && variant != DAGRT_VAR_NOPARA ? M - sum_m : 0u;
+        if (S > 0) {
+            uint32_t lastz = 0;
+            int row = nrows + np, id = 0;
+            // next candidate of the scan, -1 at the end; mw (!SUM): the lane's candidates
+            int cw = -1, sl = -1;
+            uint64_t bits = 0, sbits = 0, sums = 0;
+            if constexpr (SUM) {
+                if (np == 1 && lane == 0) clear_released(w, r);
+                __syncwarp();
+                if (lane < ((g.W + 63) >> 6)) sums = ((const uint64_t *)w.sum())[lane];
             } else {
-                v = ws.lst[gb + i - ge];
-                if (v >= g.V) v = -1;  // a segment: its node is not finished
+                if (lane < 2 * g.W) mw = w.rel()[lane];
+                if (np == 1 && (uint32_t)lane == r >> 5) mw &= ~(1u << (r & 31));
+            }
+            auto next = [&]() -> int {
+                if constexpr (!SUM) {
+                    const uint32_t bal = __ballot_sync(FULL, mw != 0);
+                    if (!bal) return -1;
+                    const int l = __ffs(bal) - 1;
+                    const int u = __shfl_sync(FULL, 32 * lane + __ffs(mw) - 1, l);
+                    if (lane == l) mw &= mw - 1;
+                    return u;
+                } else {
+                    while (!bits) {
+                        if (!sbits) {
+                            const uint32_t bal = __ballot_sync(FULL, sums != 0) & (sl < 0 ? ~0u : ~0u << sl << 1);
+                            if (!bal) return -1;
+                            sl = __ffs(bal) - 1;
+                            sbits = __shfl_sync(FULL, sums, sl);
+                        }
+                        const int b = __ffsll((long long)sbits) - 1;
+                        sbits &= sbits - 1;
+                        cw = sl * 64 + b;
+                        bits = ((const uint64_t *)w.rel())[cw];
+                        if (!bits && lane == 0)  // emptied since it was marked
+                            atomicAnd(w.sum() + 2 * sl + (b >> 5), ~(1u << (b & 31)));
+                    }
+                    const int b = __ffsll((long long)bits) - 1;
+                    bits &= bits - 1;
+                    return cw * 64 + b;
+                }
+            };
+            int u = next();
+            uint4 qu = make_uint4(0, 0, 0, 0);
+            if (u >= 0) qu = w.rc(u);
+            if (early) {  // every lane has its copy of the released set
+                __syncwarp();
+                if (lane == 0) clear_released(w, r);
+                nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
+            }
+            T WS = R * (T)S;  // Eq.6 (literal variant)
+            while (u >= 0) {
+                const uint32_t x = qu.x, k = qu.w >> 16;
+                uint32_t mu = min(x, S), p = 0, cu;
+                bool fits;
+                id = w.byrank(u);
+                if (variant == DAGRT_VAR_LITERAL) {
+                    if (WS == 0) break;
+                    fits = x <= WS;
+                    p = (uint32_t)WS;
+                    if (fits) WS -= x;
+                    else mu = min(p, S);
+                    cu = Ar::time(fits ? x : p, k, mu);
+                } else {
+                    cu = qu.y;
+                    if (x <= S) {
+                        if (cu == 0) cu = Ar::time(x, k, x);
+                        fits = cu <= R;
+                    } else {
+                        fits = Ar::fits(x, k, S, R);
+                        if (fits) cu = Ar::time(x, k, S);
+                    }
+                    if (fits) {
+                        S -= mu;
+                    } else if (variant == DAGRT_VAR_NOSEG) {
+                        u = next();
+                        if (u >= 0) qu = w.rc(u);
+                        continue;
+                    } else {
+                        p = Ar::split(x, k, S, R);
+                        mu = min(p, S);
+                        cu = (uint32_t)R;
+                    }
+                }
+                lastz = mu | (k << 16);
+                if (!fits) {  // node segmentation: the parallel part runs now
+                    seg = nseg++;
+                    if (lane == 0) {
+                        *(uint2 *)&w.rc(u) = make_uint2(x - p, 0u);
+                        write_row(row, g.V + seg, id, j, p, lastz, cu, true);
+                        if constexpr (FULL_OUT)
+                            if (a.o.seg_parent) {
+                                a.o.seg_parent[g.n0 + seg] = id;
+                                a.o.seg_load[g.n0 + seg] = (int64_t)p;
+                                a.o.seg_m[g.n0 + seg] = (int32_t)mu;
+                                a.o.seg_group[g.n0 + seg] = j;
+                            }
+                    }
+                    break;
+                }
+                const uint32_t ub = qu.z, ud = qu.w & 0xffffu;
+                uint32_t su = 0;
+                if ((uint32_t)lane < ud) su = w.col(ub + lane);
+                if (lane == 0) {
+                    w.lst(nwhole) = (uint16_t)u;
+                    write_row(row, id, id, j, x, lastz, cu, false);
+                    finish((uint32_t)u, id, j, mu);
+                    clear_released(w, (uint32_t)u);
+                }
+                row++;
+                nwhole++;
+                const int u1 = S == 0 ? -1 : next();
+                if (u1 >= 0) qu = w.rc(u1);
+                // the scan has passed every rank below u, so u's successors, released now,
+                // are not seen before the next group
+                if (!defer) nrel += release_succ<SUM, FULL_OUT>(w, ub, ud, su, lane);
+                u = u1;
+            }
+            // the last launch ends the group
+            if (lane == 0 && nwhole && seg < 0 && plan) plan[row - 1].z = lastz | (1u << 24);
+        } else if (early) {
+            if (lane == 0) clear_released(w, r);
+            nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
+        }
+        const int nl = nwhole + (seg >= 0);
+        if constexpr (FULL_OUT) {
+            __syncwarp();
+            if (variant != DAGRT_VAR_NOPARA) {  // extra dependencies: counted, and written on request
+                if (defer) {
+                    if (np == 1 && lane == 0) clear_released(w, r);
+                    __syncwarp();
+                    if (lane == 0)
+                        write_extra_edges(w, a.o.extra_src + g.ebase, a.o.extra_dst + g.ebase, g.ecap, g.V, vR, nwhole,
+                                          seg, nextra);
+                    __syncwarp();
+                }
+                nextra += (int64_t)nl * (w.rc(vR).w & 0xffffu) + (int64_t)(nrel0 - np - nwhole);
             }
         }
-        const uint32_t fin = __ballot_sync(FULL, v >= 0);
-        if (v >= 0) {
-            ws.st[v] = ST_DONE;
-            ws.rem[v] = 0;
-            if (a.o.exec_group) a.o.exec_group[g.n0 + v] = j;
-            atomicAnd((unsigned long long *)&ws.relmask[ws.rank[v] >> 6], ~(1ull << (ws.rank[v] & 63)));
-            ws.tmp[nfin + __popc(fin & ((1u << lane) - 1))] = v;
-        }
-        nfin += __popc(fin);
-    }
-    if (lane == 0) acc.nrel -= nfin;
-    nf = nfin;
-    __syncwarp();
-    // ... and release their successors
-    int released = 0;
-    for (int f = 0; f < nf; f++) {
-        const int v = ws.tmp[f];
-        for (int e = g.rp[v] + lane; e < g.rp[v + 1]; e += 32) {
-            const int s = g.col[e];
-            if (atomicSub(&ws.cnt[s], 1) == 1) {
-                atomicOr((unsigned long long *)&ws.relmask[ws.rank[s] >> 6], 1ull << (ws.rank[s] & 63));
-                if (g.W > kSumWords)
-                    atomicOr((unsigned long long *)&ws.relsum[ws.rank[s] >> 12], 1ull << ((ws.rank[s] >> 6) & 63));
-                released++;
+        // ---- the members' rows; members finish with pi_j and release their successors
+        auto release_lanes = [&]() {  // lane by lane: targets of different members may coincide
+            for (uint32_t b = live; b; b &= b - 1) {
+                const int l = __ffs(b) - 1;
+                const uint32_t eb = __shfl_sync(FULL, q.z, l), dl = __shfl_sync(FULL, q.w, l) & 0xffffu;
+                const uint32_t s = (uint32_t)lane < dl ? w.col(eb + lane) : 0u;
+                nrel += release_succ<SUM, FULL_OUT>(w, eb, dl, s, lane);
             }
-        }
-    }
-    released = __reduce_add_sync(FULL, released);
-    if (lane == 0) acc.nrel += released;
-    __syncwarp();
-}
-
-// Group j scheduled by the whole CTA team (groups of more than 32 members). `acc` is only valid in
-// the team's first thread; sc[8] carries acc.nrows to the others.
-template <int NT>
-__device__ void group_team(const Team<NT> &tm, const Ws &ws, const SchedArgs &a, const Dag &g, int j, Acc &acc) {
-    const uint32_t M = g.M;
-    const bool lead = tm.t == 0;
-    volatile int32_t *sc = ws.sc;
-    const int gb = ws.gstart[j], ge = ws.gstart[j + 1];
-    uint32_t cm = 0;
-    uint64_t wl = 0;
-    for (int i = gb + tm.t; i < ge; i += NT) {
-        const int v = ws.gmem[i];
-        if (!(ws.st[v] & ST_DONE)) {
-            cm++;
-            wl += ws.rem[v];
-        }
-    }
-    const uint32_t np = (uint32_t)tm.sum(cm);
-    if (np == 0) {
-        if (lead && a.o.group_R) a.o.group_R[g.n0 + j] = 0;
-        return;
-    }
-    const uint64_t Wg = tm.sum(wl);
-    uint64_t sml = 0;
-    for (int i = gb + tm.t; i < ge; i += NT) {
-        const int v = ws.gmem[i];
-        if (ws.st[v] & ST_DONE) continue;
-        const uint64_t num = 2ull * ws.rem[v] * M + Wg, den = 2ull * Wg;
-        uint64_t r = (num >> 32) == 0 && (den >> 32) == 0 ? (uint64_t)((uint32_t)num / (uint32_t)den) : num / den;
-        if (r < 1) r = 1;
-        const uint32_t m = (uint32_t)(r < ws.rem[v] ? r : ws.rem[v]);
-        ws.mm[v] = (uint16_t)m;
-        sml += m;
-    }
-    uint64_t sum_m = tm.sum(sml);
-    tm.sync();
-    while (g.variant != DAGRT_VAR_NOREPAIR && sum_m > M) {
-        uint64_t key = 0;
-        for (int i = gb + tm.t; i < ge; i += NT) {
-            const int v = ws.gmem[i];
-            if (ws.st[v] & ST_DONE) continue;
-            const uint64_t kv = ((uint64_t)ws.mm[v] << 16) | (uint64_t)v;
-            key = kv > key ? kv : key;
-        }
-        key = tm.maxu(key);
-        if (lead) ws.mm[key & 0xffff]--;
-        sum_m--;
-        tm.sync();
-    }
-    uint64_t ckey = 0, csum = 0;  // (C, 0xffff - id): the max is the largest C, then the lowest id
-    for (int i = gb + tm.t; i < ge; i += NT) {
-        const int v = ws.gmem[i];
-        if (ws.st[v] & ST_DONE) continue;
-        const uint64_t c = exec_time(ws.rem[v], ws.kk[v], ws.mm[v], M);
-        const uint64_t kv = (c << 16) | (uint64_t)(0xffff - v);
-        ckey = kv > ckey ? kv : ckey;
-        csum += c;
-    }
-    ckey = tm.maxu(ckey);
-    csum = tm.sum(csum);
-    // over-full (no repair only): the members run one after another
-    const uint64_t R = sum_m > M ? csum : ckey >> 16;
-    const int vR = 0xffff - (int)(ckey & 0xffff);
-    int nrows = sc[8];
-    for (int base = gb; base < ge; base += NT) {
-        const int i = base + tm.t;
-        const bool mem = i < ge && !(ws.st[ws.gmem[i]] & ST_DONE);
-        uint32_t tot;
-        const uint32_t off = tm.excl_sum(mem ? 1u : 0u, &tot);
-        if (mem) {
-            const int v = ws.gmem[i];
-            write_row(a, g, nrows + (int)off, v, v, j, ws.rem[v], ws.kk[v], ws.mm[v],
-                      exec_time(ws.rem[v], ws.kk[v], ws.mm[v], M));
-        }
-        nrows += (int)tot;
-    }
-    tm.sync();
-    if (lead) {
-        acc.nrows = nrows;
-        acc.lastr = -1;  // the members' rows were written by the team
-        int nl, nwhole;
-        const uint32_t S0 = sum_m < M ? M - (uint32_t)sum_m : 0u;
-        if (g.W > kSumWords)
-            launch_parallel<true>(ws, a, g, j, R, S0, acc, &nl, &nwhole);
-        else
-            launch_parallel<false>(ws, a, g, j, R, S0, acc, &nl, &nwhole);
-        extra_edges(ws, a, g, j, vR, (int)np, nl, nwhole, acc);
-        sc[1] = nl;
-        sc[6] = 0;
-        sc[7] = 0;
-    }
-    tm.sync();
-    const int nl = sc[1];
-    for (int i = gb + tm.t; i < ge + nl; i += NT) {
-        int v;
-        if (i < ge) {
-            v = ws.gmem[i];
-            if (ws.st[v] & ST_DONE) continue;
+        };
+        if (np == 1) {
+            if (lane == 0) {
+                const int idm = w.byrank(r);
+                write_row(nrows, idm, idm, j, q.x, m | (q.w & 0xffff0000u), c, nl == 0);
+                finish(r, idm, j, m);
+            }
+            if (!early) {
+                if (lane == 0) clear_released(w, r);
+                nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
+            }
+        } else if (n <= 32) {
+            if (q.x) {
+                const int i = __popc(live & ((1u << lane) - 1)), idm = w.byrank(r);
+                write_row(nrows + i, idm, idm, j, q.x, m | (q.w & 0xffff0000u), c, nl == 0 && i == np - 1);
+                finish(r, idm, j, m);
+            }
+            release_lanes();
         } else {
-            v = ws.lst[i - ge];
-            if (v >= g.V) continue;
-        }
-        ws.st[v] = ST_DONE;
-        ws.rem[v] = 0;
-        if (a.o.exec_group) a.o.exec_group[g.n0 + v] = j;
-        atomicAnd((unsigned long long *)&ws.relmask[ws.rank[v] >> 6], ~(1ull << (ws.rank[v] & 63)));
-        ws.tmp[atomicAdd((int *)&sc[6], 1)] = v;
-    }
-    tm.sync();
-    const int nf = sc[6];
-    for (int f = 0; f < nf; f++) {
-        const int v = ws.tmp[f];
-        for (int e = g.rp[v] + tm.t; e < g.rp[v + 1]; e += NT) {
-            const int s = g.col[e];
-            if (atomicSub(&ws.cnt[s], 1) == 1) {
-                atomicOr((unsigned long long *)&ws.relmask[ws.rank[s] >> 6], 1ull << (ws.rank[s] & 63));
-                if (g.W > kSumWords)
-                    atomicOr((unsigned long long *)&ws.relsum[ws.rank[s] >> 12], 1ull << ((ws.rank[s] >> 6) & 63));
-                atomicAdd((int *)&sc[7], 1);
+            int i = 0;  // rows written
+            for (int i0 = 0; i0 < n; i0 += 32) {
+                q = make_uint4(0, 0, 0, 0);
+                if (i0 + lane < n) {
+                    r = w.gmem(gb + i0 + lane);
+                    q = w.rc(r);
+                }
+                live = __ballot_sync(FULL, q.x > 0);
+                if (q.x) {
+                    const int x = i + __popc(live & ((1u << lane) - 1)), idm = w.byrank(r);
+                    const uint32_t mr = w.mm(i0 + lane);
+                    write_row(nrows + x, idm, idm, j, q.x, mr | (q.w & 0xffff0000u), q.y, nl == 0 && x == np - 1);
+                    finish(r, idm, j, mr);
+                }
+                i += __popc(live);
+                release_lanes();
             }
         }
+        if constexpr (FULL_OUT) {
+            if (defer)  // whole launches, whose release waited for the extra edges
+                for (int i = 0; i < nwhole; i++) {
+                    const uint4 x = w.rc(w.lst(i));
+                    const uint32_t dl = x.w & 0xffffu;
+                    const uint32_t s = (uint32_t)lane < dl ? w.col(x.z + lane) : 0u;
+                    nrel += release_succ<SUM, FULL_OUT>(w, x.z, dl, s, lane);
+                }
+            nrel -= np + nwhole;
+            if (a.o.group_R && lane == 0) a.o.group_R[g.n0 + j] = (int64_t)R;
+        }
+        nrows += np + nl;
+        bound += R;
+        __syncwarp();
     }
-    tm.sync();
-    if (lead) {
-        acc.nrel += sc[7] - nf;
-        if (a.o.group_R) a.o.group_R[g.n0 + j] = (int64_t)R;
-        acc.bound += R;
-    }
+    acc.bound = bound;
+    acc.nextra = nextra;
+    acc.nrows = nrows;
+    acc.nseg = nseg;
+    acc.err = nrows > 2 * g.V || nseg > g.V;
 }
 
 // ------------------------------------------------------------------ one DAG
-template <int NT>
+// SH: the workspace is in the kernel's dynamic shared memory
+template <int NT, bool SH, bool FULL_OUT>
 __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &a, int d, int vc, int ec) {
     const int64_t n0 = a.node_off[d];
     const int V = (int)(a.node_off[d + 1] - n0);
@@ -1124,7 +1248,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     }
     tm.sync();
 
-    // ---- member lists of each group, ordered by id
+    // ---- member lists of each group, ordered by id, as ranks
     for (int q = tm.t; q <= G; q += NT) ws.gfill[q] = 0;
     tm.sync();
     for (int v = tm.t; v < V; v += NT) atomicAdd(&ws.gfill[ws.group_of[v]], 1);
@@ -1145,7 +1269,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
         const int q = ws.group_of[v];
         int pos = 0;
         for (int x = ws.gstart[q]; x < ws.gstart[q + 1]; x++) pos += ws.gtmp[x] < v;
-        ws.gmem[ws.gstart[q] + pos] = (uint16_t)v;
+        ws.gmem[ws.gstart[q] + pos] = ws.rank[v];
     }
     tm.sync();
 
@@ -1153,20 +1277,20 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     int nsrc = 0;
     const bool want_base = a.o.greedy || a.o.greedy_unaware || a.o.graham_para;
     uint64_t b_greedy = 0, b_unaware = 0, b_vol = 0;  // baseline sums (Evaluation section)
+    uint16_t *cnt = (uint16_t *)ws.cnt;  // predecessors not yet finished, by rank
     for (int v = tm.t; v < V; v += NT) {
-        const uint32_t x = ws.load[v];
-        ws.rem[v] = x;
-        ws.cfull[v] = (uint32_t)exec_time(x, ws.kk[v], x < M ? x : M, M);
+        const uint32_t x = ws.load[v], k = ws.kk[v], r = ws.rank[v];
+        const uint32_t cf = (uint32_t)exec_time(x, k, x < M ? x : M, M);
         if (want_base) {
-            b_greedy += ws.cfull[v];
-            b_unaware = sat_add(b_unaware, exec_time_unaware(x, ws.kk[v], M));
+            b_greedy += cf;
+            b_unaware = sat_add(b_unaware, exec_time_unaware(x, k, M));
             b_vol += x;
         }
-        ws.cnt[v] = ws.indeg[v];  // predecessors not yet finished
-        ws.st[v] = 0;
-        ws.mm[v] = 0;
+        ws.rc[r] = make_uint4(x, cf, rp[v], (rp[v + 1] - rp[v]) | (k << 16));
+        cnt[r] = ws.indeg[v];
         nsrc += ws.indeg[v] == 0;
     }
+    for (int e = tm.t; e < (int)E; e += NT) ws.scol[e] = ws.rank[ws.scol[e]];
     nsrc = (int)tm.sum(nsrc);
     if (want_base) {
         b_greedy = tm.sum(b_greedy);
@@ -1176,14 +1300,12 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     for (int w = tm.t; w < W; w += NT) ws.relmask[w] = 0;
     for (int w = tm.t; w < (W + 63) / 64; w += NT) ws.relsum[w] = 0;
     tm.sync();
-    // released set as a bit mask over ranks (W^anc descending), so the next parallel
-    // node to consider is always the lowest set bit; relsum marks its possibly non-empty
-    // words
+    // the released set; relsum marks its possibly non-empty words
     for (int v = tm.t; v < V; v += NT)
         if (ws.indeg[v] == 0) {
-            atomicOr((unsigned long long *)&ws.relmask[ws.rank[v] >> 6], 1ull << (ws.rank[v] & 63));
-            if (W > kSumWords)
-                atomicOr((unsigned long long *)&ws.relsum[ws.rank[v] >> 12], 1ull << ((ws.rank[v] >> 6) & 63));
+            const uint32_t r = ws.rank[v];
+            atomicOr((uint32_t *)ws.relmask + (r >> 5), 1u << (r & 31));
+            if (W > kSumWords) atomicOr((uint32_t *)ws.relsum + (r >> 11), 1u << ((r >> 6) & 31));
         }
     tm.sync();
 
@@ -1194,38 +1316,41 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     g.W = W;
     g.M = M;
     g.variant = a.variant;
-    g.rp = rp;
-    g.col = col;
     g.want_edges = a.o.extra_off != nullptr;
     g.ebase = g.want_edges ? a.o.extra_off[d] : 0;
     g.ecap = g.want_edges ? a.o.extra_off[d + 1] - g.ebase : 0;
     Acc acc;
-    acc.bound = 0;
-    acc.nextra = 0;
-    acc.nrows = 0;
-    acc.nseg = 0;
     acc.nrel = nsrc;
-    acc.err = false;
-    acc.lastr = -1;
-    acc.lastz = 0;
-    // Warp teams run every group on lane 0 (group_serial takes groups of any size; without
-    // the team path the warp kernel needs 96 instead of 127 registers, and measured 2.6%
-    // faster on the 10,000-DAG batch); CTA teams give groups of more than 32 members to the
-    // whole team.
-    constexpr int kSerialMax = NT == 32 ? 0x7fffffff : 32;
-    for (int j = 0; j < G;) {
-        int j1 = j;
-        while (j1 < G && ws.gstart[j1 + 1] - ws.gstart[j1] <= kSerialMax) j1++;
-        if (tm.t < 32)  // the team's first warp
-            for (int q = j; q < j1; q++) group_serial(ws, a, g, q, acc, tm.t);
-        if (j1 < G) {
-            if (lead) sc[8] = acc.nrows;
-            tm.sync();
-            if constexpr (NT > 32) group_team(tm, ws, a, g, j1, acc);
+    if (tm.t < 32) {  // the team's first warp
+        extern __shared__ __align__(16) unsigned char smem[];
+        A2<SH> w2;
+        unsigned char *b0 = SH ? smem : (unsigned char *)ws.load;
+        auto off = [&](const void *p) { return (uint32_t)((const unsigned char *)p - b0); };
+        w2.base = b0;
+        w2.o_rc = off(ws.rc);
+        w2.o_col = off(ws.scol);
+        w2.o_cnt = off(cnt);
+        w2.o_gstart = off(ws.gstart);
+        w2.o_gmem = off(ws.gmem);
+        w2.o_byrank = off(ws.byrank);
+        w2.o_lst = off(ws.lst);
+        w2.o_mm = off(ws.mm);
+        w2.o_rel = (uint32_t)((unsigned char *)ws.relmask - smem);
+        w2.o_sum = (uint32_t)((unsigned char *)ws.relsum - smem);
+        const bool narrow = 64ull * M * mx < (1ull << 32);
+        bool done = false;
+        if constexpr (NT > 32)
+            if (W > kSumWords) {
+                if (narrow) alg2_warp<true, SH, true, FULL_OUT>(w2, a, g, G, acc, tm.t);
+                else alg2_warp<true, SH, false, FULL_OUT>(w2, a, g, G, acc, tm.t);
+                done = true;
+            }
+        if (!done) {
+            if (narrow) alg2_warp<false, SH, true, FULL_OUT>(w2, a, g, G, acc, tm.t);
+            else alg2_warp<false, SH, false, FULL_OUT>(w2, a, g, G, acc, tm.t);
         }
-        tm.sync();
-        j = j1 + 1;
     }
+    tm.sync();
 
     // ---- per-DAG and per-node outputs
     if (lead) {
@@ -1256,7 +1381,6 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     for (int v = tm.t; v < V; v += NT) {
         if (a.o.block_of) a.o.block_of[n0 + v] = ws.blk[v];
         if (a.o.group_of) a.o.group_of[n0 + v] = ws.group_of[v];
-        if (a.o.m) a.o.m[n0 + v] = ws.mm[v];
     }
     tm.sync();
 
@@ -1268,7 +1392,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     //      or run in sequence). From the plan rows just written, level by level.
     uint64_t cp = 0;
     if (a.o.crit_path && a.plan) {  // uniform over the team
-        if (lead) sc[11] = acc.nrows;  // (after the outputs that read ws.mm: phase F overlays it)
+        if (lead) sc[11] = acc.nrows;  // (Alg.2 is done with the region that phase F overlays)
         for (int v = tm.t; v < V; v += NT) {
             ws.cpT[v] = 0;
             ws.cpM[v] = 0;
@@ -1291,7 +1415,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                 const uint64_t dv = ws.cpT[v] + ws.cpM[v];
                 ws.cpT[v] = dv;
                 for (int e = rp[v]; e < (int)rp[v + 1]; e++)
-                    atomicMax((unsigned long long *)&ws.cpM[col[e]], (unsigned long long)dv);
+                    atomicMax((unsigned long long *)&ws.cpM[ws.byrank[col[e]]], (unsigned long long)dv);
             }
             tm.sync();
         }
@@ -1316,7 +1440,9 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
 // ------------------------------------------------------------------ kernels
 // Warp teams for small DAGs: kWarpsPerCta teams per CTA, each with a shared-memory workspace
 // sized for (a.vcap, a.ecap), the largest V and E of the launch's size class.
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_sched_warp(SchedArgs a) {
+// Five CTAs an SM (96 registers): at four (128) the 10,000-DAG batch is latency-bound on 16 warps.
+template <bool FULL_OUT>
+__global__ void __launch_bounds__(32 * kWarpsPerCta, 5) k_sched_warp(SchedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5;
     Ws ws;
@@ -1328,20 +1454,24 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) k_sched_warp(SchedArgs a) {
         if (tm.t == 0) idx = atomicAdd(a.counter, 1);
         idx = __shfl_sync(FULL, idx, 0);
         if (idx >= a.n_list) break;
-        schedule_one<32>(tm, ws, a, a.list[idx], a.vcap, a.ecap);
+        schedule_one<32, true, FULL_OUT>(tm, ws, a, a.list[idx], a.vcap, a.ecap);
         __syncwarp();
     }
 }
 
 // CTA teams for large DAGs: the workspace sized for (a.vcap, a.ecap) lives in dynamic shared
 // memory (SMEM) or in the global block a.gws + blockIdx.x * a.gws_stride.
-template <int NT, bool SMEM>
+template <int NT, bool SMEM, bool FULL_OUT>
 __global__ void __launch_bounds__(NT) k_sched_cta(SchedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t red[NT / 32];
     __shared__ int idx_s;
     Ws ws;
     ws_carve(SMEM ? smem : a.gws + (int64_t)blockIdx.x * a.gws_stride, a.vcap, a.ecap, &ws, true);
+    if constexpr (!SMEM) {  // the released set changes with every group: always in shared memory
+        ws.relmask = (uint64_t *)smem;
+        ws.relsum = ws.relmask + kRelWords;
+    }
     Team<NT> tm{(int)threadIdx.x, red};
     for (;;) {
         if (threadIdx.x == 0) idx_s = atomicAdd(a.counter, 1);
@@ -1349,12 +1479,17 @@ __global__ void __launch_bounds__(NT) k_sched_cta(SchedArgs a) {
         const int idx = idx_s;
         __syncthreads();
         if (idx >= a.n_list) break;
-        schedule_one<NT>(tm, ws, a, a.list ? a.list[idx] : idx, a.vcap, a.ecap);
+        schedule_one<NT, SMEM, FULL_OUT>(tm, ws, a, a.list ? a.list[idx] : idx, a.vcap, a.ecap);
         __syncthreads();
     }
 }
 
 // ------------------------------------------------------------------ launchers
+// Does the call ask for an output that only the FULL_OUT kernels write?
+static bool full_out(const dagrt_schedule_out &o) {
+    return o.n_extra || o.extra_off || o.group_R || o.seg_parent || o.row_id || o.row_group || o.row_m0 || o.row_load;
+}
+
 // Occupancy of the warp kernel per (device, dynamic shared memory), queried once per size
 // (a schedule call launches up to 16 classes; these host queries were a visible part of
 // its enqueue time).
@@ -1364,33 +1499,35 @@ struct WarpLaunchCache {
     std::map<std::pair<int, int64_t>, int> occ;  // (device, bytes) -> CTAs per SM
     std::map<int, int> max_smem;                 // device -> max_dynamic_smem(k_sched_warp)
 };
-WarpLaunchCache &warp_cache() {
-    static WarpLaunchCache c;
-    return c;
+WarpLaunchCache &warp_cache(bool full) {  // one per kernel
+    static WarpLaunchCache c[2];
+    return c[full];
 }
 }  // namespace
 
 cudaError_t sched_launch_warp(const SchedArgs &a, int n_sm, cudaStream_t st) {
     const int64_t bytes = ws_carve(nullptr, a.vcap, a.ecap, nullptr) * kWarpsPerCta;
+    const bool full = full_out(a.o);
+    const auto kern = full ? k_sched_warp<true> : k_sched_warp<false>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     {
-        WarpLaunchCache &c = warp_cache();
+        WarpLaunchCache &c = warp_cache(full);
         std::lock_guard<std::mutex> lock(c.mu);
         auto it = c.occ.find({dev, bytes});
         if (it == c.occ.end() && bytes > sched_smem_limit()) return cudaErrorInvalidValue;
         auto mx = c.max_smem.find(dev);
-        if (mx == c.max_smem.end()) mx = c.max_smem.emplace(dev, max_dynamic_smem(k_sched_warp)).first;
+        if (mx == c.max_smem.end()) mx = c.max_smem.emplace(dev, max_dynamic_smem(kern)).first;
         if (bytes > mx->second) return cudaErrorInvalidValue;
         // the classes differ in size: the attribute allows the largest, whatever launched last
-        e = cudaFuncSetAttribute(k_sched_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, mx->second);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx->second);
         if (e != cudaSuccess) return e;
         if (it != c.occ.end()) {
             per_sm = it->second;
         } else {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sched_warp, 32 * kWarpsPerCta, bytes);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kWarpsPerCta, bytes);
             if (e != cudaSuccess) return e;
             c.occ[{dev, bytes}] = per_sm;
         }
@@ -1400,21 +1537,24 @@ cudaError_t sched_launch_warp(const SchedArgs &a, int n_sm, cudaStream_t st) {
     const int need = ceil_div(a.n_list, kWarpsPerCta);
     if (grid > need) grid = need;
     if (grid < 1) return cudaSuccess;
-    k_sched_warp<<<grid, 32 * kWarpsPerCta, bytes, st>>>(a);
+    kern<<<grid, 32 * kWarpsPerCta, bytes, st>>>(a);
     return cudaGetLastError();
 }
 
 int sched_cta_grid(int n_sm) {
-    int per_sm = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sched_cta<kCtaThreadsGlobal, false>,
-                                                                        kCtaThreadsGlobal, 0);
-    if (e != cudaSuccess || per_sm < 1) per_sm = 1;
-    return n_sm * per_sm;
+    int best = 1;  // CTAs of the variant with more of them: a grid may be larger than what is resident
+    for (auto kern : {k_sched_cta<kCtaThreadsGlobal, false, false>, k_sched_cta<kCtaThreadsGlobal, false, true>}) {
+        int per_sm = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCtaThreadsGlobal, kRelBytes);
+        if (e == cudaSuccess && per_sm > best) best = per_sm;
+    }
+    return n_sm * best;
 }
 
 cudaError_t sched_launch_cta(const SchedArgs &a, int grid, cudaStream_t st) {
     if (grid < 1 || a.n_list < 1) return cudaSuccess;
-    k_sched_cta<kCtaThreadsGlobal, false><<<grid, kCtaThreadsGlobal, 0, st>>>(a);
+    const auto kern = full_out(a.o) ? k_sched_cta<kCtaThreadsGlobal, false, true> : k_sched_cta<kCtaThreadsGlobal, false, false>;
+    kern<<<grid, kCtaThreadsGlobal, kRelBytes, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1429,17 +1569,18 @@ int64_t sched_smem_limit() {
 cudaError_t sched_launch_cta_smem(const SchedArgs &a, int n_sm, cudaStream_t st) {
     if (a.n_list < 1) return cudaSuccess;
     const int64_t bytes = sched_ws_bytes(a.vcap, a.ecap);
-    const int mx = max_dynamic_smem(k_sched_cta<kCtaThreads, true>);
+    const auto kern = full_out(a.o) ? k_sched_cta<kCtaThreads, true, true> : k_sched_cta<kCtaThreads, true, false>;
+    const int mx = max_dynamic_smem(kern);
     if (bytes > mx) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_sched_cta<kCtaThreads, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sched_cta<kCtaThreads, true>, kCtaThreads, bytes);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCtaThreads, bytes);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int grid = n_sm * per_sm;
     if (grid > a.n_list) grid = a.n_list;
-    k_sched_cta<kCtaThreads, true><<<grid, kCtaThreads, bytes, st>>>(a);
+    kern<<<grid, kCtaThreads, bytes, st>>>(a);
     return cudaGetLastError();
 }
 
