@@ -6,17 +6,13 @@
 // the bound is a max-plus sweep along the group chain (Theorem 1): F_j = F_{j-1} + R_j,
 // with R_j = max C_i over the group if its SMs fit in M (Lemma 1), else sum C_i.
 //
-// Two paths. Materialised candidates in blocks of 64 (n_alloc a multiple of 64) take the
+// Three paths. Materialised candidates in blocks of 64 (n_alloc a multiple of 64) take the
 // balanced work items (k_bound_items + k_bound_finish, below): chunks of whole groups of
 // every plan, one warp per (chunk, 64-candidate block), its rows staged by 2-D TMA tensor
-// copies, partial bounds added into per-candidate accumulators. Everything else (generated candidates, other n_alloc) takes
-// the tile kernel k_bound_tma: one CTA per DAG; row tiles of the DAG -- the candidate bytes
-// of T rows (one contiguous run of T * cand_stride bytes, or none when the candidates are
-// generated in the kernel) and the T plan rows of every variant in the call -- stream from
-// global to shared memory with TMA bulk copies into two stages that complete on mbarriers,
-// so the loads of tile i+1 overlap the evaluation of tile i. Each thread owns 1, 2 or 4
-// adjacent candidates of one variant and keeps their running group states; the argmin over
-// the DAG's candidates is reduced with warp shuffles and shared memory in the same kernel.
+// copies, partial bounds added into per-candidate accumulators. The exhaustive search
+// enumerates per DAG (k_bound_exhaustive). Everything else (random levels, perturbations,
+// other n_alloc) takes k_bound_rows: one CTA per DAG, its warps sharing windows of plan rows.
+#include <cooperative_groups.h>
 #include <cuda.h>  // CUtensorMap and its encoding enums (header only)
 
 #include <cstring>
@@ -27,7 +23,6 @@
 
 namespace dagrt {
 
-constexpr int kBoundMaxThreads = 256;
 constexpr uint32_t kSpinLimit = 1u << 24;  // bounded mbarrier wait
 
 // ------------------------------------------------------------------ TMA / mbarrier
@@ -97,21 +92,6 @@ __device__ __forceinline__ void better(int64_t &bb, int32_t &bc, int64_t ob, int
     }
 }
 
-// Shared-memory layout of one stage: T rows of candidate bytes, then T plan rows (16 B)
-// of each variant.
-struct TileLayout {
-    int T;
-    int64_t cand_bytes, stage_bytes;
-};
-
-__host__ __device__ inline TileLayout tile_layout(int T, int64_t stride, int nv) {
-    TileLayout t;
-    t.T = T;
-    t.cand_bytes = (int64_t)T * stride;
-    t.stage_bytes = t.cand_bytes + (int64_t)nv * T * 16;
-    return t;
-}
-
 // SMs of plan row `row` (owner node `owner`, scheduled on m0 SMs) for generated candidate c
 // of DAG d; 0 keeps the schedule's m.
 __device__ __forceinline__ uint32_t gen_alloc(const BoundArgs &a, int d, int c, int row, uint32_t owner, uint32_t m0,
@@ -127,219 +107,468 @@ __device__ __forceinline__ uint32_t gen_alloc(const BoundArgs &a, int d, int c, 
     return x == 0 ? 0u : perturb_m(m0, x);  // code 0 keeps the row's own m (even above 255)
 }
 
-// Candidate bytes of one row for a thread's CPT adjacent candidates (one shared load), or
-// the generated allocations of those candidates.
-template <int CPT, bool GEN>
-__device__ __forceinline__ uint32_t row_alloc(const BoundArgs &a, const unsigned char *cbuf, int64_t stride, int rr,
-                                              int d, int c, int row, uint32_t owner, uint32_t m0,
-                                              const uint8_t *s_lev) {
-    if (GEN) {
-        uint32_t m4 = 0;
-#pragma unroll
-        for (int q = 0; q < CPT; q++) m4 |= gen_alloc(a, d, c + q, row, owner, m0, s_lev) << (8 * q);
-        return m4;
-    }
-    if (CPT == 4) return *(const uint32_t *)(cbuf + rr * stride);
-    if (CPT == 2) return *(const uint16_t *)(cbuf + rr * stride);
-    return cbuf[rr * stride];
-}
+// ------------------------------------------------------------------ rows of one DAG per CTA
+// Candidates that the balanced work items below do not take: generated ones (random levels,
+// perturbations) and materialised ones whose count is not a multiple of 64. One CTA takes a
+// DAG; its warps share the DAG's (variant, window of kRowWindow plan rows, block of 32 CPT
+// candidates) tasks, so a DAG of 1,000 rows keeps 16 warps busy, where one thread per
+// candidate walked all rows of its variant alone. A window's groups are those that start in
+// it: no chunk index is needed, nor scratch in global memory, and partial bounds add up in
+// shared memory (Theorem 1's sum splits at group ends).
+//
+// What bounds it is instruction issue. Eq.1's division is out of the inner loop: generated
+// candidates look {C, m} up in a table of the row's few possible choices (built by one lane
+// per row), and a byte m <= M divides by 64 m with a multiply and a shift. Per candidate and
+// row that leaves SplitMix64 (two 64-bit multiplications) or ten instructions. Two candidates
+// a lane above 32 allocations (one: 359 us instead of 279 below). Windows of 32 rows: 64 and
+// 128 take 65 and 92 us instead of 58 on the second workload, the first does not care.
+// 500 DAGs of 100-1,000 nodes x 256 perturbations: 3.06 -> 0.28 ms; 1,000 DAGs of 20-200 nodes
+// x 74 allocations: 116 -> 63 us a call.
+constexpr int kRowWindow = 32;
+constexpr int kRowTile = 2048;   // candidates of one pass over the DAG (shared-memory sums)
+enum { SRC_BYTES = 0, SRC_RANDOM = 1, SRC_PERTURB = 2 };
+constexpr int kPerturbCodes = 5;
 
-// The tiles of DAG d for this thread's candidates c .. c+CPT-1 (variant vi, my_rows rows).
-// FIT (uniform over the DAG): every variant's plan keeps all sums below 2^31, so the
-// state is 32-bit and C for m = 2^l <= M takes the shift form
-//   ceil(x (64m - k(m-1)) / 64m) = ((x(64-k) + 64) << l + x k - 1) >> (l + 6);
-// other allocations (not a power of two, or above M) take exec_time. Group ends are
-// applied without branches, so threads of different variants may share a warp.
-// Returns false when a tile copy stalled (the CTA aborts).
-template <int CPT, bool GEN, bool FIT>
-__device__ __forceinline__ bool eval_tiles(const BoundArgs &a, int d, int c, int vi, int my_rows, int rows_max,
-                                           const TileLayout &L, int64_t stride, unsigned char *const *stage,
-                                           uint64_t *bar, uint32_t *uses, uint32_t *issued, uint32_t *landed,
-                                           int *s_abort, const uint8_t *s_lev, uint64_t *bound_out) {
-    using S = typename std::conditional<FIT, uint32_t, uint64_t>::type;
-    const int T = L.T, nv = a.n_variants, tid = threadIdx.x;
-    const uint32_t M = (uint32_t)a.M;
-    const int64_t rbase = 2 * a.node_off[d];
-    const int ntile = (rows_max + T - 1) / T;
-    S bound[CPT], gmax[CPT], gsum[CPT];
-    uint32_t gm[CPT];
-#pragma unroll
-    for (int q = 0; q < CPT; q++) bound[q] = gmax[q] = gsum[q] = 0, gm[q] = 0;
-
-    auto issue = [&](int i) {  // tile i of the DAG into stage i & 1 (thread 0)
-        const int s = i & 1;
-        const int r0 = i * T;
-        const int rn = min(T, rows_max - r0);
-        const uint32_t cb = (uint32_t)(rn * stride);
-        issued[s]++;
-        mbar_expect_tx(&bar[s], cb + (uint32_t)(nv * rn * 16));
-        if (!GEN) bulk_g2s(stage[s], a.m_alloc + (rbase + r0) * stride, cb, &bar[s]);
-        for (int v = 0; v < nv; v++)
-            bulk_g2s(stage[s] + L.cand_bytes + (int64_t)v * T * 16, a.plan[v] + rbase + r0, (uint32_t)(rn * 16),
-                     &bar[s]);
-    };
-    if (tid == 0) {
-        fence_proxy_async();
-        for (int i = 0; i < 2 && i < ntile; i++) issue(i);
-    }
-    for (int i = 0; i < ntile; i++) {
-        const int s = i & 1;
-        const bool ok = mbar_wait(&bar[s], uses[s] & 1);
-        uses[s]++;
-        landed[s] += ok;
-        if (!ok) atomicExch(s_abort, 1);
-        __syncthreads();
-        if (*s_abort) return false;
-        const int r0 = i * T;
-        const int rn = min(T, my_rows - r0);
-        const unsigned char *cbuf = stage[s] + c;  // candidate column c of row r0
-        const uint4 *pl = (const uint4 *)(stage[s] + L.cand_bytes) + (int64_t)vi * T;
-        for (int rr = 0; rr < rn; rr++) {
-            const uint4 x = pl[rr];
-            const uint32_t k = (x.z >> 16) & 0xffu, m0 = x.z & 0xffffu;
-            const bool last = (x.z >> 24) != 0;
-            const uint32_t m4 = row_alloc<CPT, GEN>(a, cbuf, stride, rr, d, c, r0 + rr, x.w, m0, s_lev);
-            S cc[CPT];
-            if (FIT) {
-                const uint32_t A1 = x.x * (64u - k) + 64u, B1 = x.x * k - 1u;
-#pragma unroll
-                for (int q = 0; q < CPT; q++) {
-                    const uint32_t m = (m4 >> (8 * q)) & 0xffu;
-                    const uint32_t ms = m ? m : 1u;
-                    const int l = 31 - __clz(ms);
-                    uint32_t v = ((A1 << l) + B1) >> (l + 6);
-                    if ((ms != (1u << l)) | (ms > M)) v = (uint32_t)exec_time(x.x, k, ms, M);
-                    cc[q] = m ? v : x.y;
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < CPT; q++) {
-                    const uint32_t m = (m4 >> (8 * q)) & 0xffu;
-                    cc[q] = m ? exec_time(x.x, k, m, M) : (uint64_t)x.y;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < CPT; q++) {
-                const uint32_t m = (m4 >> (8 * q)) & 0xffu;
-                gmax[q] = cc[q] > gmax[q] ? cc[q] : gmax[q];
-                gsum[q] += cc[q];
-                gm[q] += m ? m : m0;
-                const S r = gm[q] <= M ? gmax[q] : gsum[q];
-                bound[q] += last ? r : (S)0;
-                gmax[q] = last ? (S)0 : gmax[q];
-                gsum[q] = last ? (S)0 : gsum[q];
-                gm[q] = last ? 0u : gm[q];
-            }
-        }
-        __syncthreads();  // every thread is done with stage s
-        if (tid == 0 && i + 2 < ntile) {
-            fence_proxy_async();
-            issue(i + 2);
+// n / (64 m) for n < 2^31 as (n * x >> 32) >> y: x = ceil(2^(32+y) / 64 m), exact while
+// n (64 m x - 2^(32+y)) < 2^(32+y). Not a power of two: 2^y > 32 m, the bracket is below
+// 64 m <= 16320 and n < 2^17 * 64 m, so the product stays below 2^(32+y). A power of two:
+// the bracket is 0.
+struct Div64m {
+    uint32_t x[256], y[256];
+    constexpr Div64m() : x(), y() {
+        for (uint32_t m = 0; m < 256; m++) {
+            const uint64_t D = 64ull * (m ? m : 1);
+            int l = 0;
+            while ((D >> (l + 1)) != 0) l++;
+            y[m] = (uint32_t)((D & (D - 1)) ? l : l - 1);
+            x[m] = (uint32_t)(((1ull << (32 + y[m])) + D - 1) / D);
         }
     }
-#pragma unroll
-    for (int q = 0; q < CPT; q++) bound_out[q] = (uint64_t)bound[q];
-    return true;
-}
+};
+__device__ constexpr Div64m kDiv64m;
 
-// FIT selects the DAGs this instance evaluates (the 32-bit form exact for every variant, or
-// not); the host launches both instances over the batch, each skipping the other's DAGs,
-// so each keeps only its own state in registers.
-template <int CPT, bool GEN, bool FIT>
-__global__ void __launch_bounds__(kBoundMaxThreads) k_bound_tma(BoundArgs a, int T) {
-    extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ __align__(8) uint64_t bar[2];
-    __shared__ int s_abort;
-    __shared__ int64_t s_bb[kBoundMaxThreads / 32];
-    __shared__ int32_t s_bc[kBoundMaxThreads / 32];
+template <int CPT, int SRC>
+__global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
+    extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint8_t s_lev[16];
-    const int nv = a.n_variants;
-    const int n_cand = nv * a.n_alloc;
-    const int64_t stride = GEN ? 0 : a.stride;  // generated candidates stream plan rows only
-    const TileLayout L = tile_layout(T, stride, nv);
-    if (GEN && threadIdx.x < 16) s_lev[threadIdx.x] = a.levels[threadIdx.x];
-    unsigned char *stage[2] = {sm, sm + L.stage_bytes};
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        mbar_fence_init();
-        s_abort = 0;
-    }
-    __syncthreads();
-    uint32_t uses[2] = {0, 0};    // waits per stage so far (identical in every thread)
-    uint32_t issued[2] = {0, 0};  // copies issued per stage (thread 0)
-    uint32_t landed[2] = {0, 0};  // waits that saw their copy land (thread 0)
+    __shared__ int64_t s_bb[16];
+    __shared__ int32_t s_bc[16];
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int rank = (int)cl.block_rank(), nct = (int)cl.num_blocks(), NW = nct * (int)(blockDim.x >> 5);
+    const int nv = a.n_variants, n_cand = nv * a.n_alloc;
+    const int tile = min(n_cand, kRowTile);
+    const uint32_t M = (uint32_t)a.M;
+    unsigned long long *s_acc = (unsigned long long *)sm;
+    uint2 *s_div = (uint2 *)(s_acc + tile);  // SRC_BYTES: n / (64 m)
+    // per warp, 32 rows: {C, m} by choice, or (SRC_BYTES) {x (64 - k), x k - 1, C, m}
+    uint2 *tab = s_div + (SRC == SRC_BYTES ? 256 : 0) + (tile & 1) + w * 32 * entries;
+    if (SRC != SRC_BYTES && tid < 16) s_lev[tid] = a.levels[tid];
+    if (SRC == SRC_BYTES)
+        for (int m = tid; m < 256; m += blockDim.x) s_div[m] = make_uint2(kDiv64m.x[m], kDiv64m.y[m]);
 
-    for (int d = blockIdx.x; d < a.n_dags; d += gridDim.x) {
+    for (int d = blockIdx.x / nct; d < a.n_dags; d += gridDim.x / nct) {  // the same in a cluster's CTAs
         const int64_t rbase = 2 * a.node_off[d];
-        int rows_max = 0;
-        bool fit = true;  // the 32-bit form is exact for every variant
-        for (int v = 0; v < nv; v++)
-            if (a.status[v][d] == DAGRT_OK) {
-                rows_max = max(rows_max, a.nrows[v][d]);
-                fit = fit && (a.pflag[v][d] & 1);
-            }
-        if (fit != FIT) continue;  // uniform over the CTA
         int64_t best_b = 0;
         int32_t best_c = -1;
-
-        for (int c0 = 0; c0 < n_cand; c0 += blockDim.x * CPT) {
-            const int c = c0 + tid * CPT;
-            const bool active = c < n_cand;
-            const int vi = active ? c / a.n_alloc : 0;
-            const bool valid = active && a.status[vi][d] == DAGRT_OK;
-            const int my_rows = valid ? a.nrows[vi][d] : 0;
-            uint64_t bound[CPT];
-            const bool ok = eval_tiles<CPT, GEN, FIT>(a, d, c, vi, my_rows, rows_max, L, stride, stage, bar, uses,
-                                                      issued, landed, &s_abort, s_lev, bound);
-            if (!ok) break;
+        for (int t0 = 0; t0 < n_cand; t0 += tile) {
+            const int t1 = min(n_cand, t0 + tile);
+            for (int i = tid; i < tile; i += blockDim.x) s_acc[i] = 0;
+            __syncthreads();
+            int task = rank * (int)(blockDim.x >> 5) + w;  // tasks are numbered variant by variant; a warp takes every NW-th
+            for (int vi = t0 / a.n_alloc; vi * a.n_alloc < t1; vi++) {
+                // allocations of this variant in this pass
+                const int a0 = max(t0 - vi * a.n_alloc, 0), a1 = min(t1 - vi * a.n_alloc, a.n_alloc);
+                const int rows = a.status[vi][d] == DAGRT_OK ? a.nrows[vi][d] : 0;
+                const bool fit = rows && (a.pflag[vi][d] & 1);
+                const int nwin = (rows + kRowWindow - 1) / kRowWindow;
+                const int nblk = (a1 - a0 + 32 * CPT - 1) / (32 * CPT);
+                const uint4 *plan = a.plan[vi] + rbase;
+                for (; task < nwin * nblk; task += NW) {
+                    const int win = task / nblk, al0 = a0 + (task - win * nblk) * 32 * CPT + lane;
+                    const int wend = (win + 1) * kRowWindow;  // groups that start before it
+                    bool on[CPT];
 #pragma unroll
-            for (int q = 0; q < CPT; q++) {
-                const int cq = c + q;
-                if (!active || cq >= n_cand) break;
-                const int64_t b = valid ? (int64_t)bound[q] : -1;
-                if (a.out) a.out[(int64_t)d * n_cand + cq] = b;
-                if (valid) better(best_b, best_c, b, cq);
+                    for (int q = 0; q < CPT; q++) on[q] = al0 + 32 * q < a1;
+                    uint64_t total[CPT];
+                    uint32_t b[CPT], gmax[CPT], gsum[CPT], gm[CPT];
+                    uint64_t wmax[CPT], wsum[CPT];  // 64-bit sums
+#pragma unroll
+                    for (int q = 0; q < CPT; q++)
+                        total[q] = 0, b[q] = gmax[q] = gsum[q] = gm[q] = 0, wmax[q] = wsum[q] = 0;
+                    // is row `base` the start of a group?
+                    bool prev = win == 0 || (plan[win * kRowWindow - 1].z >> 24) != 0, open = false;
+                    for (int base = win * kRowWindow; base < rows && (open || base < wend); base += 32) {
+                        const int rn = min(32, rows - base);
+                        uint4 x = make_uint4(0, 0, 0, 0);
+                        if (lane < rn) x = plan[base + lane];
+                        const uint32_t k = (x.z >> 16) & 0xffu, m0 = x.z & 0xffffu;
+                        const uint32_t endm = __ballot_sync(FULL, (x.z >> 24) != 0);
+                        uint32_t startm = (endm << 1) | (prev ? 1u : 0u);
+                        if (rn < 32) startm &= (1u << rn) - 1;
+                        prev = (endm >> 31) != 0;
+                        // rows [ra, rb): from the first start (an open group: from 0) to the end
+                        // of the last group that starts before wend
+                        const int inwin = wend - base;  // rows of the window from here on
+                        const uint32_t mine = inwin >= 32 ? startm : (inwin > 0 ? startm & ((1u << inwin) - 1) : 0u);
+                        if (!open && !mine) continue;
+                        const int ra = open ? 0 : __ffs(mine) - 1;
+                        int rb = rn;
+                        const uint32_t later = startm & ~mine;  // groups of the next window
+                        if (later && inwin < 32) rb = __ffs(later) - 1;
+                        open = rb == 32 && !(endm >> 31);
+                        __syncwarp();
+                        if (SRC == SRC_BYTES) {
+                            ((uint4 *)tab)[lane] = make_uint4(x.x * (64u - k), x.x * k - 1u, x.y, m0);
+                        } else if (fit && lane < rn) {
+                            uint2 *t = tab + lane * entries;
+                            t[0] = make_uint2(x.y, m0);  // keep
+                            for (int e = 1; e < entries; e++) {
+                                const uint32_t m = SRC == SRC_PERTURB ? perturb_m(m0, e) : s_lev[e - 1];
+                                t[e] = make_uint2((uint32_t)exec_time(x.x, k, m, M), m);
+                            }
+                        }
+                        __syncwarp();
+                        if (fit) {
+                            const uint8_t *src = a.m_alloc + (rbase + base) * a.stride + vi * a.n_alloc + al0;
+                            constexpr int U = SRC == SRC_BYTES ? 8 : 2;  // rows in flight together
+                            for (int rr = ra; rr < rb; rr += U) {
+                                uint32_t mb[U][CPT];
+                                if constexpr (SRC == SRC_BYTES) {
+#pragma unroll
+                                    for (int i = 0; i < U; i++)
+#pragma unroll
+                                        for (int q = 0; q < CPT; q++)
+                                            mb[i][q] = on[q] && rr + i < rb ? src[(int64_t)(rr + i) * a.stride + 32 * q] : 0u;
+                                }
+#pragma unroll
+                                for (int i = 0; i < U; i++) {
+                                    const int r = rr + i;
+                                    if (r >= rb) break;
+                                    uint2 cm[CPT];
+                                    if constexpr (SRC == SRC_BYTES) {
+                                        const uint4 y = ((const uint4 *)tab)[r];
+#pragma unroll
+                                        for (int q = 0; q < CPT; q++) {
+                                            const uint32_t m = mb[i][q];
+                                            const uint2 dv = s_div[m];
+                                            cm[q].x = (__umulhi(y.x * m + y.y, dv.x) >> dv.y) + 1u;
+                                            cm[q].y = m;
+                                            if (m > M) {
+                                                const uint4 z = plan[base + r];
+                                                cm[q].x = (uint32_t)exec_time(z.x, (z.z >> 16) & 0xffu, m, M);
+                                            }
+                                            if (m == 0) cm[q] = make_uint2(y.z, y.w);
+                                        }
+                                    } else {
+#pragma unroll
+                                        for (int q = 0; q < CPT; q++) {
+                                            const int al = al0 + 32 * q;
+                                            const int lv = gen_level(a.seed, d, vi * a.n_alloc + al, base + r, a.n_levels);
+                                            const int e = al == 0 ? 0 : (SRC == SRC_PERTURB ? (int)s_lev[lv] : lv + 1);
+                                            cm[q] = tab[r * entries + e];
+                                        }
+                                    }
+                                    const bool first = (startm >> r) & 1u, last = (endm >> r) & 1u;
+                                    if (first && last) {
+#pragma unroll
+                                        for (int q = 0; q < CPT; q++) b[q] += cm[q].x;
+                                        continue;
+                                    }
+#pragma unroll
+                                    for (int q = 0; q < CPT; q++) {
+                                        gmax[q] = first ? cm[q].x : max(gmax[q], cm[q].x);
+                                        gsum[q] = first ? cm[q].x : gsum[q] + cm[q].x;
+                                        gm[q] = first ? cm[q].y : gm[q] + cm[q].y;
+                                        if (last) b[q] += gm[q] <= M ? gmax[q] : gsum[q];
+                                    }
+                                }
+                            }
+                        } else {  // 64-bit sums: Eq.1 for every candidate
+                            for (int r = ra; r < rb; r++) {
+                                const uint4 y = plan[base + r];
+                                const uint32_t ky = (y.z >> 16) & 0xffu, my = y.z & 0xffffu;
+                                const bool first = (startm >> r) & 1u, last = (endm >> r) & 1u;
+#pragma unroll
+                                for (int q = 0; q < CPT; q++) {
+                                    const int al = al0 + 32 * q;
+                                    uint32_t m = 0;
+                                    if (SRC != SRC_BYTES) m = gen_alloc(a, d, vi * a.n_alloc + al, base + r, y.w, my, s_lev);
+                                    else if (on[q]) m = a.m_alloc[(rbase + base + r) * a.stride + vi * a.n_alloc + al];
+                                    const uint64_t c = m ? exec_time(y.x, ky, m, M) : (uint64_t)y.y;
+                                    wmax[q] = first || c > wmax[q] ? c : wmax[q];
+                                    wsum[q] = first ? c : wsum[q] + c;
+                                    gm[q] = (first ? 0u : gm[q]) + (m ? m : my);
+                                    if (last) total[q] += gm[q] <= M ? wmax[q] : wsum[q];
+                                }
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < CPT; q++)
+                        if (on[q] && rows)
+                            atomicAdd(&s_acc[vi * a.n_alloc + al0 + 32 * q - t0], (unsigned long long)(total[q] + b[q]));
+                }
+                task -= nwin * nblk;
             }
+            if (nct > 1) {  // the cluster's sums to its first CTA
+                cl.sync();
+                if (rank > 0) {
+                    unsigned long long *acc0 = cl.map_shared_rank(s_acc, 0);
+                    for (int i = tid; t0 + i < t1; i += blockDim.x) atomicAdd(&acc0[i], s_acc[i]);
+                }
+                cl.sync();
+            } else {
+                __syncthreads();
+            }
+            for (int i = tid; rank == 0 && t0 + i < t1; i += blockDim.x) {
+                const int c = t0 + i;
+                const bool ok = a.status[c / a.n_alloc][d] == DAGRT_OK;
+                const int64_t v = ok ? (int64_t)s_acc[i] : -1;
+                if (a.out) a.out[(int64_t)d * n_cand + c] = v;
+                if (ok) better(best_b, best_c, v, c);
+            }
+            __syncthreads();
         }
-        if (s_abort) break;
-        if (a.best_bound || a.best_cand) {
+        if (rank == 0 && (a.best_bound || a.best_cand || a.best_m)) {
             for (int o = 16; o > 0; o >>= 1) {
                 const int64_t ob = __shfl_xor_sync(FULL, best_b, o);
                 const int32_t oc = __shfl_xor_sync(FULL, best_c, o);
                 better(best_b, best_c, ob, oc);
             }
-            if ((tid & 31) == 0) {
-                s_bb[tid >> 5] = best_b;
-                s_bc[tid >> 5] = best_c;
+            if (lane == 0) {
+                s_bb[w] = best_b;
+                s_bc[w] = best_c;
             }
             __syncthreads();
+            best_c = -1;
+            for (int i = 0; i < (int)(blockDim.x >> 5); i++) better(best_b, best_c, s_bb[i], s_bc[i]);
             if (tid == 0) {
-                for (int w = 1; w < (int)(blockDim.x >> 5); w++) better(best_b, best_c, s_bb[w], s_bc[w]);
                 if (a.best_bound) a.best_bound[d] = best_c < 0 ? -1 : best_b;
                 if (a.best_cand) a.best_cand[d] = best_c;
-                s_bc[0] = best_c;
             }
-            __syncthreads();
-            if (GEN && a.best_m && s_bc[0] >= 0) {  // the winning allocation, row by row
-                const int wc = s_bc[0], wv = wc / a.n_alloc;
-                const int rows = a.nrows[wv][d];
-                for (int r = tid; r < rows; r += blockDim.x) {
+            if (SRC != SRC_BYTES && a.best_m && best_c >= 0) {  // the winning allocation, row by row
+                const int wv = best_c / a.n_alloc;
+                for (int r = tid; r < a.nrows[wv][d]; r += blockDim.x) {
                     const uint4 x = a.plan[wv][rbase + r];
-                    a.best_m[rbase + r] = (uint8_t)gen_alloc(a, d, wc, r, x.w, x.z & 0xffffu, s_lev);
+                    a.best_m[rbase + r] = (uint8_t)gen_alloc(a, d, best_c, r, x.w, x.z & 0xffffu, s_lev);
                 }
             }
             __syncthreads();
         }
     }
-    if (s_abort && tid == 0) {
-        // a copy stalled: report it, and give the copies already issued a bounded chance to
-        // land before the CTA's shared memory is released
-        if (a.err) atomicExch(a.err, DAGRT_E_TIMEOUT);
-        for (int s = 0; s < 2; s++)
-            for (uint32_t k = landed[s]; k < issued[s]; k++) mbar_wait(&bar[s], k & 1);
+}
+
+// ------------------------------------------------------------------ exhaustive enumeration
+// Allocation a gives node u the level of digit (a / B^u) mod B, B = n_levels + 1. A cluster
+// of CTAs takes a DAG and shares its allocations; candidates beyond B^V repeat earlier ones
+// (the digits of the DAG's own nodes repeat) and cannot win, so they are only evaluated when
+// every bound is asked for. Each thread fixes the digits of nodes 1.. and runs through node
+// 0's B levels: only the groups that hold a row of node 0 (mostly one) change, the sum of
+// the others is kept. {C, m} of every row and digit come from a table in shared memory.
+// Ties go to the smaller allocation, as everywhere.
+// Bound by instruction issue (76% of the issue slots); 2,000 DAGs of 3-6 nodes x 9^6
+// allocations: 41.9 -> 0.51 ms (the duplicates are 72% of the candidates; the rest was a
+// division per digit and per C). One CTA per DAG takes 0.96 ms there, two 0.67, eight 0.60.
+constexpr int kExhThreads = 256;
+constexpr int kExhMaxRows = 64;  // rows of a plan that the table and the row records hold
+
+// a row in the kernel's shared memory: first table entry | shift of its node's digit in the
+// packed digits << 16 (0xff: node 0) | last row of its group << 24
+constexpr uint32_t kExhNode0 = 0xffu << 16, kExhLast = 1u << 24;
+
+__global__ void __launch_bounds__(kExhThreads) k_bound_exhaustive(BoundArgs a, int bits) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    __shared__ uint32_t s_row[kExhMaxRows];  // groups without a row of node 0, then the others
+    __shared__ uint2 s_tab[kExhMaxRows * 16];  // {C, m} by digit
+    __shared__ int64_t s_bb[kExhThreads / 32 + 1];
+    __shared__ int32_t s_bc[kExhThreads / 32 + 1];
+    __shared__ uint8_t s_lev[16];
+    __shared__ int s_split;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t rank = cl.block_rank(), nct = cl.num_blocks();
+    const int d = blockIdx.x / nct;
+    const uint32_t B = (uint32_t)a.n_levels + 1u, M = (uint32_t)a.M, msk = (1u << bits) - 1;
+    const uint32_t rcpB = (uint32_t)(((1ull << 32) + B - 1) / B);  // t / B = t * rcpB >> 32 for t < 2^20
+    if (tid < 16) s_lev[tid] = a.levels[tid];
+    const int64_t n0 = a.node_off[d], rbase = 2 * n0;
+    const int V = (int)(a.node_off[d + 1] - n0), n_cand = a.n_variants * a.n_alloc;
+    uint32_t T = (uint32_t)a.n_alloc;  // allocations to evaluate
+    int digits = 0;                    // nodes whose digit can be other than 0
+    for (uint64_t p = 1; digits < V; digits++, p *= B)
+        if (p >= T) break;
+    if (!a.out) {
+        uint64_t p = 1;
+        for (int u = 0; u < digits; u++) p *= B;
+        if (p < T) T = (uint32_t)p;
     }
+    int64_t best_b = 0;
+    int32_t best_c = -1;
+    for (int v = 0; v < a.n_variants; v++) {
+        const bool ok = a.status[v][d] == DAGRT_OK;
+        const int rows = ok ? a.nrows[v][d] : 0;
+        const uint4 *plan = a.plan[v] + rbase;
+        const int c0 = v * a.n_alloc;
+        if (!ok || (a.pflag[v][d] & 1) == 0 || rows > kExhMaxRows) {
+            // failed, 64-bit sums or a long plan: candidate by candidate
+            for (uint32_t al = rank * kExhThreads + tid; al < T; al += nct * kExhThreads) {
+                uint64_t b = 0, mx = 0, sum = 0;
+                uint32_t ms = 0;
+                for (int r = 0; r < rows; r++) {
+                    const uint4 x = plan[r];
+                    const uint32_t m = gen_alloc(a, d, (int)al, r, x.w, x.z & 0xffffu, s_lev);
+                    const uint64_t c = m ? exec_time(x.x, (x.z >> 16) & 0xffu, m, M) : (uint64_t)x.y;
+                    mx = c > mx ? c : mx;
+                    sum += c;
+                    ms += m ? m : x.z & 0xffffu;
+                    if (x.z >> 24) {
+                        b += ms <= M ? mx : sum;
+                        mx = sum = 0;
+                        ms = 0;
+                    }
+                }
+                if (a.out) a.out[(int64_t)d * n_cand + c0 + al] = ok ? (int64_t)b : -1;
+                if (ok) better(best_b, best_c, (int64_t)b, c0 + (int)al);
+            }
+            continue;
+        }
+        __syncthreads();  // the table of the variant before is read
+        if (w < 2) {      // 64 rows, one per thread: which groups hold a row of node 0
+            __shared__ uint32_t s_end[2], s_zero[2];
+            const int r = tid;
+            const uint4 x = r < rows ? plan[r] : make_uint4(0, 0, 0, 0);
+            const uint32_t eb = __ballot_sync(FULL, (x.z >> 24) != 0);
+            const uint32_t zb = __ballot_sync(FULL, r < rows && x.w == 0);
+            if (lane == 0) {
+                s_end[w] = eb;
+                s_zero[w] = zb;
+            }
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            const uint64_t end = s_end[0] | ((uint64_t)s_end[1] << 32), zero = s_zero[0] | ((uint64_t)s_zero[1] << 32);
+            // rows of r's group: after the last end before r, up to the first end at or after r
+            const uint64_t below = r ? end & ((1ull << r) - 1) : 0ull;
+            const int first = below ? 64 - __clzll((long long)below) : 0;
+            const uint64_t from = end >> r << r;
+            const int lastr = from ? __ffsll((long long)from) - 1 : 63;
+            const uint64_t grp = (lastr == 63 ? ~0ull : (1ull << (lastr + 1)) - 1) & ~((1ull << first) - 1);
+            const bool hot = r < rows && (zero & grp) != 0;
+            const uint32_t hb = __ballot_sync(FULL, hot);
+            asm volatile("bar.sync 1, 64;" ::: "memory");  // both warps have read s_zero
+            if (lane == 0) s_zero[w] = hb;
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            const uint64_t hots = s_zero[0] | ((uint64_t)s_zero[1] << 32);
+            const int cold = rows - __popcll(hots), hbef = __popcll(hots & ((1ull << r) - 1));
+            if (r < rows) {
+                const int at = hot ? cold + hbef : r - hbef;
+                // node 0's digit is the innermost loop's: digits are packed from node 1 on
+                const uint32_t sh = x.w == 0 ? 0xffu : (int)x.w < digits ? (x.w - 1) * bits : 31u;
+                s_row[at] = (uint32_t)(r * 16) | (sh << 16) | (x.z >> 24 ? kExhLast : 0u);
+            }
+            if (r == 0) s_split = cold;
+        }
+        for (int i = tid; i < rows * (int)B; i += kExhThreads) {
+            const int r = i / (int)B, dg = i - r * (int)B;
+            const uint4 x = plan[r];
+            const uint32_t m = dg ? s_lev[dg - 1] : 0u;
+            s_tab[r * 16 + dg] = m ? make_uint2((uint32_t)exec_time(x.x, (x.z >> 16) & 0xffu, m, M), m)
+                                   : make_uint2(x.y, x.z & 0xffffu);
+        }
+        __syncthreads();
+        const int cold = s_split;
+        const uint32_t H = (T + B - 1) / B;
+        uint32_t lb = ~0u, la = 0;  // this variant's best; a later allocation wins only if smaller
+        for (uint32_t h = rank * kExhThreads + tid; h < H; h += nct * kExhThreads) {
+            uint32_t pk = 0;
+            for (uint32_t u = 1, t = h; u < (uint32_t)digits; u++) {
+                const uint32_t q = __umulhi(t, rcpB);
+                pk |= (t - q * B) << ((u - 1) * bits);
+                t = q;
+            }
+            auto entry = [&](uint32_t x) { return s_tab[(x & 0xffffu) + ((pk >> ((x >> 16) & 31u)) & msk)]; };
+            uint32_t fixed = 0, mx = 0, sum = 0, ms = 0;
+            for (int r = 0; r < cold; r++) {
+                const uint32_t x = s_row[r];
+                const uint2 e = entry(x);
+                mx = max(mx, e.x);
+                sum += e.x;
+                ms += e.y;
+                if (x & kExhLast) {
+                    fixed += ms <= M ? mx : sum;
+                    mx = sum = ms = 0;
+                }
+            }
+            uint32_t tot[16];  // by node 0's digit
+#pragma unroll
+            for (int dg = 0; dg < 16; dg++) tot[dg] = fixed;
+            for (int r = cold, z = 0; r < rows; r++) {
+                const uint32_t x = s_row[r];
+                if ((x & kExhNode0) == kExhNode0) {  // the group's row of node 0
+                    z = (int)(x & 0xffffu);
+                } else {
+                    const uint2 e = entry(x);
+                    mx = max(mx, e.x);
+                    sum += e.x;
+                    ms += e.y;
+                }
+                if (x & kExhLast) {
+#pragma unroll
+                    for (int dg = 0; dg < 16; dg++) {
+                        if (dg >= (int)B) break;
+                        const uint2 e = s_tab[z + dg];
+                        tot[dg] += ms + e.y <= M ? max(mx, e.x) : sum + e.x;
+                    }
+                    mx = sum = ms = 0;
+                }
+            }
+#pragma unroll
+            for (int dg = 0; dg < 16; dg++) {
+                const uint32_t al = h * B + dg;
+                if (dg >= (int)B || al >= T) break;
+                if (a.out) a.out[(int64_t)d * n_cand + c0 + al] = (int64_t)tot[dg];
+                if (tot[dg] < lb) {
+                    lb = tot[dg];
+                    la = al;
+                }
+            }
+        }
+        if (lb != ~0u) better(best_b, best_c, (int64_t)lb, c0 + (int)la);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const int64_t ob = __shfl_xor_sync(FULL, best_b, o);
+        const int32_t oc = __shfl_xor_sync(FULL, best_c, o);
+        better(best_b, best_c, ob, oc);
+    }
+    if (lane == 0) {
+        s_bb[w] = best_b;
+        s_bc[w] = best_c;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int i = 1; i < kExhThreads / 32; i++) better(best_b, best_c, s_bb[i], s_bc[i]);
+        s_bb[kExhThreads / 32] = best_b;
+        s_bc[kExhThreads / 32] = best_c;
+    }
+    cl.sync();
+    if (rank == 0) {
+        best_c = -1;
+        for (uint32_t i = 0; i < nct; i++)
+            better(best_b, best_c, *cl.map_shared_rank(&s_bb[kExhThreads / 32], i),
+                   *cl.map_shared_rank(&s_bc[kExhThreads / 32], i));
+        if (tid == 0) {
+            if (a.best_bound) a.best_bound[d] = best_c < 0 ? -1 : best_b;
+            if (a.best_cand) a.best_cand[d] = best_c;
+        }
+        if (a.best_m && best_c >= 0) {  // the winning allocation, row by row
+            const int wv = best_c / a.n_alloc;
+            for (int r = tid; r < a.nrows[wv][d]; r += kExhThreads) {
+                const uint4 x = a.plan[wv][rbase + r];
+                a.best_m[rbase + r] = (uint8_t)gen_alloc(a, d, best_c, r, x.w, x.z & 0xffffu, s_lev);
+            }
+        }
+    }
+    cl.sync();  // the CTAs' shared memory is read until here
 }
 
 // ------------------------------------------------------------------ balanced work items
@@ -893,43 +1122,61 @@ cudaError_t bound_launch(const BoundArgs &a, const ChunkArgs *ch, int n_sm, cuda
         *launches += 2;
         return cudaSuccess;  // k_bound_finish evaluated the DAGs that need 64-bit sums
     }
-    // candidates per thread: a thread's candidates must never straddle two variants
-    const int cpt = a.n_alloc % 4 == 0 ? 4 : (a.n_alloc % 2 == 0 ? 2 : 1);
-    int threads = (n_cand + cpt - 1) / cpt;
-    threads = (threads + 31) / 32 * 32;
-    if (threads > kBoundMaxThreads) threads = kBoundMaxThreads;
-    // rows per tile: about 8 KB of candidate bytes (plan rows when generating) per stage
-    int T = (int)(8192 / ((a.gen ? 0 : a.stride) + 16ll * a.n_variants));
-    if (T < 1) T = 1;
-    if (T > 128) T = 128;
-    const TileLayout L = tile_layout(T, a.gen ? 0 : a.stride, a.n_variants);
-    const int64_t smem = 2 * L.stage_bytes;
-    if (smem > 200 * 1024) return cudaErrorInvalidValue;
     using K = void (*)(BoundArgs, int);
-    const K fast = a.gen ? (cpt == 4 ? k_bound_tma<4, true, true> : cpt == 2 ? k_bound_tma<2, true, true>
-                                                                           : k_bound_tma<1, true, true>)
-                         : (cpt == 4 ? k_bound_tma<4, false, true> : cpt == 2 ? k_bound_tma<2, false, true>
-                                                                             : k_bound_tma<1, false, true>);
-    const K wide = a.gen ? (cpt == 4 ? k_bound_tma<4, true, false> : cpt == 2 ? k_bound_tma<2, true, false>
-                                                                            : k_bound_tma<1, true, false>)
-                         : (cpt == 4 ? k_bound_tma<4, false, false> : cpt == 2 ? k_bound_tma<2, false, false>
-                                                                              : k_bound_tma<1, false, false>);
-    for (K kern : {fast, wide}) {
-        int per_sm = 0;
-        const int mx = max_dynamic_smem(kern);
-        if (smem > mx) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        int grid = a.n_dags;
-        if (grid > per_sm * n_sm) grid = per_sm * n_sm;
-        if (kern == wide && grid > 2 * n_sm) grid = 2 * n_sm;  // few DAGs need the 64-bit form
-        kern<<<grid, threads, smem, st>>>(a, T);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (a.gen && a.gen_mode == DAGRT_SEARCH_EXHAUSTIVE) {
+        // CTAs per DAG: enough of them for every SM, while each thread keeps a run of node 0's levels
+        const int B = a.n_levels + 1;
+        int bits = 1;
+        while ((1 << bits) < B) bits++;
+        int cl = 1;
+        while (cl < 8 && (int64_t)a.n_dags * cl < 32ll * n_sm && a.n_alloc / B >= 2 * cl * kExhThreads) cl *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)a.n_dags * cl);
+        cfg.blockDim = dim3(kExhThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
         ++*launches;
+        return cudaLaunchKernelEx(&cfg, k_bound_exhaustive, a, bits);
     }
-    return cudaSuccess;
+    // warps per CTA, and CTAs per DAG when even 16 leave SMs without work: enough warps for
+    // every SM (500 DAGs: 16 warps 279 us, 8 315, 4 396; 1,000 small ones: 4 or 8 57-62 us, 16
+    // 76; clusters only cost where the DAGs fill the chip)
+    int warps = 4, cl = 1;
+    while (warps < 16 && (int64_t)a.n_dags * warps < 32ll * n_sm) warps *= 2;
+    while (cl < 8 && (int64_t)a.n_dags * cl * warps < 16ll * n_sm) cl *= 2;
+    const bool two = a.n_alloc > 32;
+    const int src = !a.gen ? SRC_BYTES : a.gen_mode == DAGRT_SEARCH_PERTURB ? SRC_PERTURB : SRC_RANDOM;
+    const K kern = src == SRC_BYTES    ? (two ? (K)k_bound_rows<2, SRC_BYTES> : (K)k_bound_rows<1, SRC_BYTES>)
+                   : src == SRC_RANDOM ? (two ? (K)k_bound_rows<2, SRC_RANDOM> : (K)k_bound_rows<1, SRC_RANDOM>)
+                                       : (two ? (K)k_bound_rows<2, SRC_PERTURB> : (K)k_bound_rows<1, SRC_PERTURB>);
+    const int entries = src == SRC_BYTES ? 2 : src == SRC_PERTURB ? kPerturbCodes : a.n_levels + 1;
+    const int tile = n_cand < kRowTile ? n_cand : kRowTile;
+    const int smem = 8 * (tile + (tile & 1) + (src == SRC_BYTES ? 256 : 0) + warps * 32 * entries);
+    const int mx = max_dynamic_smem(kern);
+    if (smem > mx) return cudaErrorInvalidValue;
+    int per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cl * (a.n_dags < 8 * per_sm * n_sm ? a.n_dags : 8 * per_sm * n_sm)));
+    cfg.blockDim = dim3(warps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ++*launches;
+    return cudaLaunchKernelEx(&cfg, kern, a, entries);
 }
 
 }  // namespace dagrt
