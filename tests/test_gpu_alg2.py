@@ -74,3 +74,21 @@ def test_released_set_width(ctx, V):
     rp, col, w, k = random_small_dag(rng, V, 3.0 / V, 3000)
     for variant in (0, 2, 3):
         _check(ctx, wl.from_dags([(rp, col, w, k)], 148), variant)
+
+
+@pytest.mark.parametrize("V", [2, 17, 33, 64, 100, 128, 129, 200, 256, 300])
+def test_ids_in_and_out_of_topological_order(ctx, V):
+    """The same graphs with ids in topological order (a path of its own in the warp teams) and
+    permuted, with many equal W^anc (equal loads) and with distinct ones."""
+    rng = np.random.default_rng(73 + V)
+    dags = []
+    for wmax in (2, 5000):
+        rp, col, w, k = random_small_dag(rng, V, min(0.5, 6.0 / V), wmax)
+        dags.append((rp, col, w, k))
+        src, perm = np.repeat(np.arange(V), np.diff(rp)), rng.permutation(V)
+        prp, pcol = wl.csr_from_edges(V, perm[src], perm[col])
+        pw, pk = np.empty_like(w), np.empty_like(k)
+        pw[perm], pk[perm] = w, k
+        dags.append((prp, pcol, pw, pk))
+    for M in (4, 148):
+        _check(ctx, wl.from_dags(dags, M), 0)
