@@ -177,7 +177,7 @@ struct dagrt_batch {
         bool graph = false, train = false;
         int32_t *pred_off, *pred_idx, *succ_off, *succ_idx, *cursor, *level, *m;
         int64_t *wanc;
-        uint16_t *x, *h[3];
+        uint16_t *x, *h[3], *agg[3];  // agg: the layers' aggregated inputs, kept for training
         float *logits, *dlogits, *dh[3], *da, *loss_part;
         int8_t *labels;
         uint8_t *best_level, *cand;
@@ -1082,7 +1082,7 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
         if (rc) return rc;
         const int32_t *st0 = b->plan[DAGRT_VAR_PAPER].status;
         CK(gnn_build_graph(b->n_dags, b->node_off, b->edge_off, b->row_ptr, b->col, st0, G.pred_off, G.pred_idx,
-                           G.succ_off, G.succ_idx, G.cursor, ctx->n_sm, ctx->stream), "build message-passing graph");
+                           G.succ_off, G.succ_idx, G.cursor, b->max_v, ctx->n_sm, ctx->stream), "build message-passing graph");
         CK(gnn_features(b->n_dags, b->node_off, b->wcet, b->k64, G.level, G.wanc, G.m, st0, graph_of(b), G.x,
                         ctx->n_sm, ctx->stream), "node features");
         ctx->launches += 3;
@@ -1092,6 +1092,9 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
         if ((e = batch_alloc(b, &G.dlogits, N * kMaxLevels)) != cudaSuccess ||
             (e = batch_alloc(b, &G.dh[0], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.dh[1], N * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.dh[2], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.da, N * 3 * kHidden)) != cudaSuccess ||
+            (e = batch_alloc(b, &G.agg[0], N * 2 * kFeat)) != cudaSuccess ||
+            (e = batch_alloc(b, &G.agg[1], N * 2 * kHidden)) != cudaSuccess ||
+            (e = batch_alloc(b, &G.agg[2], N * 2 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.labels, N)) != cudaSuccess || (e = batch_alloc(b, &G.loss_part, 1024)) != cudaSuccess)
             return cuda_fail(ctx, e, "allocate training state");
         G.train = true;
@@ -1099,14 +1102,14 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
     return DAGRT_OK;
 }
 
-static int gnn_forward(dagrt_batch *b, dagrt_model *md) {
+static int gnn_forward(dagrt_batch *b, dagrt_model *md, bool train = false) {
     dagrt_ctx *ctx = b->ctx;
     auto &G = b->gnn;
     const GnnGraph g = graph_of(b);
     const int64_t boff[3] = {ParamLayout::b1, ParamLayout::b2, ParamLayout::b3};
     const uint16_t *in = G.x;
     for (int l = 0; l < 3; l++) {
-        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], G.h[l], b->err, ctx->n_sm,
+        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], G.h[l], train ? G.agg[l] : nullptr, b->err, ctx->n_sm,
                          ctx->stream), "layer forward");
         in = G.h[l];
     }
@@ -1252,21 +1255,21 @@ static int gnn_grad(dagrt_batch *b, dagrt_model *md, const int8_t *labels, float
     const float scale = nl ? 1.f / (float)nl : 0.f;
     cudaStream_t st = ctx->stream;
     if (N) CK(cudaMemcpyAsync(G.labels, labels, N, cudaMemcpyHostToDevice, st), "copy labels");
-    if ((rc = gnn_forward(b, md))) return rc;
+    if ((rc = gnn_forward(b, md, true))) return rc;
     const GnnGraph g = graph_of(b);
     CK(gnn_head(g, G.h[2], md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, G.labels, scale, G.logits, G.dlogits,
                 G.dh[2], G.loss_part, ctx->n_sm, st), "head");
     CK(gnn_head_grad(g, G.h[2], G.dlogits, md->L, md->part, md->n_parts, st), "head gradient");
     // layer 3 and 2: weight gradients, then the gradient of the layer input
     for (int l = 2; l >= 1; l--) {
-        CK(gnn_layer_bwd_dw(kHidden, l, g, G.h[l - 1], G.h[l], G.dh[l], md->part, md->n_parts, b->err, st), "dW");
+        CK(gnn_layer_bwd_dw(kHidden, l, g, G.h[l - 1], G.agg[l], G.h[l], G.dh[l], md->part, md->n_parts, b->err, st), "dW");
         CK(gnn_layer_bwd_da(kHidden, g, G.h[l], G.dh[l], md->wb[l], G.da, b->err, ctx->n_sm, st), "dA");
         CK(gnn_agg_bwd(kHidden, g, G.da, G.dh[l - 1], ctx->n_sm, st), "aggregation backward");
     }
-    CK(gnn_layer_bwd_dw(kFeat, 0, g, G.x, G.h[0], G.dh[0], md->part, md->n_parts, b->err, st), "dW");
+    CK(gnn_layer_bwd_dw(kFeat, 0, g, G.x, G.agg[0], G.h[0], G.dh[0], md->part, md->n_parts, b->err, st), "dW");
     ctx->launches += 10;
-    std::vector<float> lp(ctx->n_sm);
-    CK(cudaMemcpyAsync(lp.data(), G.loss_part, 4 * ctx->n_sm, cudaMemcpyDeviceToHost, st), "copy loss");
+    std::vector<float> lp(N ? gnn_head_ctas(g.n_nodes, ctx->n_sm) : 0);
+    CK(cudaMemcpyAsync(lp.data(), G.loss_part, 4 * lp.size(), cudaMemcpyDeviceToHost, st), "copy loss");
     int32_t err = 0;
     CK(cudaMemcpyAsync(&err, b->err, sizeof err, cudaMemcpyDeviceToHost, st), "copy error word");
     CK(cudaStreamSynchronize(st), "synchronize");

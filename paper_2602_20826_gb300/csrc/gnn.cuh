@@ -47,15 +47,18 @@ struct GnnParams {
 // paper schedule failed (status != DAGRT_OK) get no edges
 cudaError_t gnn_build_graph(int32_t n_dags, const int64_t *node_off, const int64_t *edge_off, const int32_t *row_ptr,
                             const int32_t *col, const int32_t *status, int32_t *pred_off, int32_t *pred_idx,
-                            int32_t *succ_off, int32_t *succ_idx, int32_t *cursor, int n_sm, cudaStream_t st);
+                            int32_t *succ_off, int32_t *succ_idx, int32_t *cursor, int max_v, int n_sm,
+                            cudaStream_t st);
 // features from the batch and the paper schedule's outputs (zero for failed DAGs)
 cudaError_t gnn_features(int32_t n_dags, const int64_t *node_off, const int64_t *wcet, const uint8_t *k64,
                          const int32_t *level, const int64_t *wanc, const int32_t *m, const int32_t *status,
                          GnnGraph g, uint16_t *x, int n_sm, cudaStream_t st);
-// one layer: h_out = ReLU(agg(h_in) W + b); kin = 16 or 128
+// one layer: h_out = ReLU([h_in | mean_pred h_in | mean_succ h_in] W + b); kin = 16 or 128;
+// agg (or NULL): the two means, bf16 [N x 2 kin], kept for the weight gradients
 cudaError_t gnn_layer_fwd(int kin, GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,
-                          uint16_t *h_out, int32_t *err, int n_sm, cudaStream_t st);
+                          uint16_t *h_out, uint16_t *agg, int32_t *err, int n_sm, cudaStream_t st);
 // head: logits (and, with labels, loss pieces and dlogits)
+int gnn_head_ctas(int64_t n_nodes, int n_sm);  // partial losses that gnn_head writes (at most 1024)
 cudaError_t gnn_head(GnnGraph g, const uint16_t *h3, const float *wh, const float *bh, int n_levels,
                      const int8_t *labels, float scale, float *logits, float *dlogits, float *dh3,
                      float *loss_part, int n_sm, cudaStream_t st);
@@ -63,8 +66,9 @@ cudaError_t gnn_head_grad(GnnGraph g, const uint16_t *h3, const float *dlogits, 
                           int n_parts, cudaStream_t st);
 // backward of one layer
 // weight and bias gradients of layer `layer` (0..2) into the per-CTA partial rows
-cudaError_t gnn_layer_bwd_dw(int kin, int layer, GnnGraph g, const uint16_t *h_in, const uint16_t *h_out,
-                             const float *dh_out, float *part, int n_parts, int32_t *err, cudaStream_t st);
+cudaError_t gnn_layer_bwd_dw(int kin, int layer, GnnGraph g, const uint16_t *h_in, const uint16_t *agg,
+                             const uint16_t *h_out, const float *dh_out, float *part, int n_parts, int32_t *err,
+                             cudaStream_t st);
 cudaError_t gnn_layer_bwd_da(int kin, GnnGraph g, const uint16_t *h_out, const float *dh_out, const uint16_t *wb,
                              float *da, int32_t *err, int n_sm, cudaStream_t st);
 cudaError_t gnn_agg_bwd(int kin, GnnGraph g, const float *da, float *dh_in, int n_sm, cudaStream_t st);

@@ -58,6 +58,24 @@ __device__ __forceinline__ void umma_gemm(uint32_t tmem_d, const void *a_smem, c
     }
 }
 
+// instruction descriptor bits: A and B are MN-major (transposed) in shared memory
+constexpr uint32_t kUmmaMnMajor = (1u << 15) | (1u << 16);
+
+// D (+)= A^T B over 16 K rows, both operands tiles of [rows x columns] with the reduction
+// along the rows, in the layout of kmajor_off(row, column, columns): M and N run along the
+// tiles' columns (stride byte offset 128), K along their 8-row groups (leading byte offset
+// 16 * columns). M = 128 columns from a_smem, N from b_smem.
+__device__ __forceinline__ void umma_gemm_tn(uint32_t tmem_d, const void *a_smem, int a_cols, const void *b_smem,
+                                             int b_cols, int rows, int N, bool accumulate) {
+    const uint32_t a0 = smem_u32(a_smem), b0 = smem_u32(b_smem);
+    const uint32_t idesc = umma_idesc_bf16(128, N) | kUmmaMnMajor;
+    for (int ks = 0; ks < rows / 16; ks++) {
+        const uint64_t ad = umma_desc(a0 + ks * 32 * a_cols, (uint32_t)a_cols * 16, 128);
+        const uint64_t bd = umma_desc(b0 + ks * 32 * b_cols, (uint32_t)b_cols * 16, 128);
+        umma_bf16(tmem_d, ad, bd, idesc, (accumulate || ks > 0) ? 1u : 0u);
+    }
+}
+
 // all prior MMAs of this thread arrive on the mbarrier when they complete
 __device__ __forceinline__ void umma_commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar))
