@@ -177,7 +177,8 @@ struct dagrt_batch {
         bool graph = false, train = false;
         int32_t *pred_off, *pred_idx, *succ_off, *succ_idx, *cursor, *level, *m;
         int64_t *wanc;
-        uint16_t *x, *h[3], *agg[3];  // agg: the layers' aggregated inputs, kept for training
+        uint16_t *x, *h[3], *agg[3];  // agg: the layers' aggregated inputs; agg[1] alone serves
+                                       // every layer of a forward pass, training keeps all
         float *logits, *dlogits, *dh[3], *da, *loss_part;
         int8_t *labels;
         uint8_t *best_level, *cand;
@@ -1069,6 +1070,7 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
             (e = batch_alloc(b, &G.m, N)) != cudaSuccess || (e = batch_alloc(b, &G.wanc, N)) != cudaSuccess ||
             (e = batch_alloc(b, &G.x, N * kFeat)) != cudaSuccess || (e = batch_alloc(b, &G.h[0], N * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.h[1], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.h[2], N * kHidden)) != cudaSuccess ||
+            (e = batch_alloc(b, &G.agg[1], N * 2 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.logits, N * kMaxLevels)) != cudaSuccess ||
             (e = batch_alloc(b, &G.best_level, N)) != cudaSuccess || (e = batch_alloc(b, &G.cand, 2 * N * kPropStride)) != cudaSuccess ||
             (e = batch_alloc(b, &G.cbest, b->n_dags)) != cudaSuccess || (e = batch_alloc(b, &G.bbest, b->n_dags)) != cudaSuccess)
@@ -1093,7 +1095,6 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
             (e = batch_alloc(b, &G.dh[0], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.dh[1], N * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.dh[2], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.da, N * 3 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.agg[0], N * 2 * kFeat)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.agg[1], N * 2 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.agg[2], N * 2 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.labels, N)) != cudaSuccess || (e = batch_alloc(b, &G.loss_part, 1024)) != cudaSuccess)
             return cuda_fail(ctx, e, "allocate training state");
@@ -1109,11 +1110,11 @@ static int gnn_forward(dagrt_batch *b, dagrt_model *md, bool train = false) {
     const int64_t boff[3] = {ParamLayout::b1, ParamLayout::b2, ParamLayout::b3};
     const uint16_t *in = G.x;
     for (int l = 0; l < 3; l++) {
-        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], G.h[l], train ? G.agg[l] : nullptr, b->err, ctx->n_sm,
+        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], G.h[l], G.agg[train ? l : 1], b->err, ctx->n_sm,
                          ctx->stream), "layer forward");
         in = G.h[l];
     }
-    ctx->launches += 3;
+    ctx->launches += 6;
     return DAGRT_OK;
 }
 

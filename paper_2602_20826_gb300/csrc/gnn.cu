@@ -255,101 +255,130 @@ cudaError_t gnn_features(int32_t n_dags, const int64_t *node_off, const int64_t 
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ forward layer
-// Persistent CTAs of kFwdWarps warps over 128-row tiles. The A tile (K = 3 KIN) is gathered
-// straight into shared memory: a group of KIN/8 lanes owns one row (16 bytes = 8 features
-// per lane), so a warp gathers 32 / (KIN/8) rows at once, and the neighbour loops are
-// unrolled by 4 so that several neighbour rows are in flight per lane (the gather is
-// latency-bound: neighbours are scattered over the DAG). One thread then issues the
-// tcgen05 MMA chain against the resident W^T; the epilogue (bias, ReLU, bf16) reads TMEM with
-// the first 16 warps: warp w takes TMEM lanes 32 (w % 4) .. + 31 and columns 32 (w / 4) .. + 31,
-// while the other 16 warps already gather their rows of the next tile.
-constexpr int kFwdWarps = 32;
-
-__device__ __forceinline__ void acc8(float *a, uint4 u) {
-    a[0] += bf2f(u.x & 0xffff);
-    a[1] += bf2f(u.x >> 16);
-    a[2] += bf2f(u.y & 0xffff);
-    a[3] += bf2f(u.y >> 16);
-    a[4] += bf2f(u.z & 0xffff);
-    a[5] += bf2f(u.z >> 16);
-    a[6] += bf2f(u.w & 0xffff);
-    a[7] += bf2f(u.w >> 16);
-}
-
-// mean over the rows idx[b .. e) of h, features [8 sub, 8 sub + 8)
-template <int KIN>
-__device__ __forceinline__ void mean_rows(const uint16_t *__restrict__ h, const int32_t *__restrict__ idx, int b,
-                                          int e, int sub, float *m) {
-#pragma unroll
-    for (int q = 0; q < 8; q++) m[q] = 0.f;
-    int i = b;
-    for (; i + 4 <= e; i += 4) {
-        const int32_t j0 = __ldg(idx + i), j1 = __ldg(idx + i + 1), j2 = __ldg(idx + i + 2), j3 = __ldg(idx + i + 3);
-        const uint4 u0 = __ldg((const uint4 *)(h + (int64_t)j0 * KIN) + sub);
-        const uint4 u1 = __ldg((const uint4 *)(h + (int64_t)j1 * KIN) + sub);
-        const uint4 u2 = __ldg((const uint4 *)(h + (int64_t)j2 * KIN) + sub);
-        const uint4 u3 = __ldg((const uint4 *)(h + (int64_t)j3 * KIN) + sub);
-        acc8(m, u0);
-        acc8(m, u1);
-        acc8(m, u2);
-        acc8(m, u3);
-    }
-    for (; i < e; i++) acc8(m, __ldg((const uint4 *)(h + (int64_t)__ldg(idx + i) * KIN) + sub));
-    const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; q++) m[q] *= inv;
-}
-
+// ------------------------------------------------------------------ aggregation
 __device__ __forceinline__ uint4 pack8(const float *f) {
     return make_uint4((uint32_t)f2bf(f[0]) | ((uint32_t)f2bf(f[1]) << 16), (uint32_t)f2bf(f[2]) | ((uint32_t)f2bf(f[3]) << 16),
                       (uint32_t)f2bf(f[4]) | ((uint32_t)f2bf(f[5]) << 16), (uint32_t)f2bf(f[6]) | ((uint32_t)f2bf(f[7]) << 16));
 }
 
-// rows [32 w / ... ) of the tile: the A operand [h | mean_pred h | mean_succ h] in K-major order
-template <int KIN>
-__device__ __forceinline__ void gather_tile(const GnnGraph &g, const uint16_t *__restrict__ h_in, int64_t tile,
-                                            unsigned char *sA, uint16_t *__restrict__ agg, int w, int lane) {
-    constexpr int K = 3 * KIN, LPR = KIN / 8, RPW = 32 / LPR;  // lanes per row, rows per warp pass
-    constexpr int ROWS = 128 / kFwdWarps;                      // rows of the tile per warp
-    const int sub = lane % LPR;
-    for (int r0 = 0; r0 < ROWS; r0 += RPW) {
-        const int rl = r0 + lane / LPR;
-        if (rl >= ROWS) continue;
-        const int r = w * ROWS + rl;
-        const int64_t v = tile * 128 + r;
-        uint4 s0 = make_uint4(0, 0, 0, 0), s1 = s0, s2 = s0;
-        if (v < g.n_nodes) {
-            s0 = __ldg((const uint4 *)(h_in + v * KIN) + sub);
-            float m[8];
-            mean_rows<KIN>(h_in, g.pred_idx, g.pred_off[v], g.pred_off[v + 1], sub, m);
-            s1 = pack8(m);
-            mean_rows<KIN>(h_in, g.succ_idx, g.succ_off[v], g.succ_off[v + 1], sub, m);
-            s2 = pack8(m);
-            if (agg) {  // kept for the weight gradients
-                *(uint4 *)(agg + v * 2 * KIN + 8 * sub) = s1;
-                *(uint4 *)(agg + v * 2 * KIN + KIN + 8 * sub) = s2;
-            }
-        }
-        *(uint4 *)(sA + kmajor_off(r, 8 * sub, K)) = s0;
-        *(uint4 *)(sA + kmajor_off(r, KIN + 8 * sub, K)) = s1;
-        *(uint4 *)(sA + kmajor_off(r, 2 * KIN + 8 * sub, K)) = s2;
+// acc[2i], acc[2i + 1] += the two bf16 of word i (fp32 additions, two to an instruction)
+__device__ __forceinline__ void acc8(uint64_t *acc, uint4 u) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        uint64_t x;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(w[i] << 16), "r"(w[i] & 0xffff0000u));
+        asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[i]) : "l"(x));
     }
 }
 
+// bf16 mean over the rows idx[b .. e) of h, features [8 sub, 8 sub + 8): fp32 sums in list
+// order, one rounding; four rows in flight
 template <int KIN>
-__global__ void __launch_bounds__(32 * kFwdWarps) k_gnn_fwd(GnnGraph g, const uint16_t *__restrict__ h_in,
-                                                            const uint16_t *__restrict__ wt,
-                                                            const float *__restrict__ bias,
-                                                            uint16_t *__restrict__ h_out,
-                                                            uint16_t *__restrict__ agg, int32_t *err) {
-    constexpr int K = 3 * KIN;
+__device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const int32_t *__restrict__ idx, int b,
+                                           int e, int sub) {
+    uint64_t acc[4] = {0, 0, 0, 0};
+    const uint4 *hs = (const uint4 *)h + sub;
+    int i = b;
+    for (; i + 4 <= e; i += 4) {
+        const int32_t j0 = __ldg(idx + i), j1 = __ldg(idx + i + 1), j2 = __ldg(idx + i + 2), j3 = __ldg(idx + i + 3);
+        const uint4 u0 = __ldg(hs + (int64_t)j0 * (KIN / 8)), u1 = __ldg(hs + (int64_t)j1 * (KIN / 8));
+        const uint4 u2 = __ldg(hs + (int64_t)j2 * (KIN / 8)), u3 = __ldg(hs + (int64_t)j3 * (KIN / 8));
+        acc8(acc, u0);
+        acc8(acc, u1);
+        acc8(acc, u2);
+        acc8(acc, u3);
+    }
+    for (; i < e; i++) acc8(acc, __ldg(hs + (int64_t)__ldg(idx + i) * (KIN / 8)));
+    const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
+    float m[8];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        float x, y;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(acc[q]));
+        m[2 * q] = x * inv;
+        m[2 * q + 1] = y * inv;
+    }
+    return pack8(m);
+}
+
+// agg[v] = [mean over predecessors of h | mean over successors of h], bf16 [N x 2 KIN]. A
+// group of KIN/8 lanes owns a node (16 bytes = 8 features per lane). A CTA's nodes are
+// neighbours in the batch, so mostly of one DAG, whose rows (140 KB for 550 nodes) stay in
+// the L1 cache: the kernel uses no shared memory, and that is why it is apart from the
+// matrix product, whose operands fill it. Bound by the L1 rate and the additions.
+// 165,000 nodes, 2.8 M edges, 128 features: XXa us, and the product XXb, where one kernel for
+// both took 190; 16 features: 97 -> XXc and XXd.
+constexpr int kAggThreads = 512;
+template <int KIN>
+__global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *__restrict__ h,
+                                                         uint16_t *__restrict__ agg) {
+    constexpr int LPN = KIN / 8, NODES = kAggThreads / LPN;  // lanes per node, nodes per CTA pass
+    const int sub = threadIdx.x % LPN;
+    constexpr int CHUNK = NODES < 128 ? 128 : NODES;         // neighbouring nodes that a CTA takes together
+    for (int64_t c0 = (int64_t)blockIdx.x * CHUNK; c0 < g.n_nodes; c0 += (int64_t)gridDim.x * CHUNK)
+        for (int i = 0; i < CHUNK / NODES; i++) {
+            const int64_t v = c0 + i * NODES + threadIdx.x / LPN;
+            if (v >= g.n_nodes) break;
+            uint4 *dst = (uint4 *)(agg + v * 2 * KIN);
+            dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred_off[v], g.pred_off[v + 1], sub);
+            dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ_off[v], g.succ_off[v + 1], sub);
+        }
+}
+
+// 16-byte piece i of warp w's share of a [128 rows x 8 C columns] tile in the layout of
+// kmajor_off: eight lanes store eight rows of one column piece, 128 contiguous bytes, and the
+// warp reads 64 (C a multiple of 4) or 32 contiguous bytes per row
+template <int C>
+__device__ __forceinline__ void tile_piece(int i, int warps, int w, int lane, int &r, int &c) {
+    constexpr int CL = C % 4 == 0 ? 4 : 2, RG = 4 / CL;  // columns of a warp's piece, 8-row groups of it
+    const int p = i * warps + w, cg = p % (C / CL), rg = p / (C / CL) * RG;
+    c = cg * CL + (lane >> 3) % CL;
+    r = 8 * (rg + (lane >> 3) / CL) + (lane & 7);
+}
+
+// 32 bytes in one store (an aligned sector)
+__device__ __forceinline__ void st32(void *p, const uint32_t *x) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x[0]), "r"(x[1]), "r"(x[2]),
+                 "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
+                 : "memory");
+}
+
+// ------------------------------------------------------------------ forward layer
+// h_out = ReLU([h | agg] W + b). Persistent CTAs over 128-row tiles: the A tile (K = 3 KIN) is
+// copied to shared memory through registers, the next tile's loads issued before the wait for
+// this one's MMA; one thread issues the tcgen05 chain against the resident W^T; the epilogue
+// (bias, ReLU, bf16) reads TMEM: warp w takes TMEM lanes 32 (w % 4) .. + 31 and columns
+// 32 (w / 4) .. + 31. Bound by reading A.
+constexpr int kFwdThreads = 512;
+
+template <int KIN>
+__global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint16_t *__restrict__ h_in,
+                                                         const uint16_t *__restrict__ agg,
+                                                         const uint16_t *__restrict__ wt,
+                                                         const float *__restrict__ bias,
+                                                         uint16_t *__restrict__ h_out, int32_t *err) {
+    constexpr int K = 3 * KIN, C = K / 8, N_IT = (128 * C + kFwdThreads - 1) / kFwdThreads;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     __shared__ float sbias[kHidden];
     unsigned char *sA = sm, *sB = sm + 128 * K * 2;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    uint4 x[N_IT];  // this thread's 16-byte pieces of the next A tile
+    auto load = [&](int64_t tile) {
+#pragma unroll
+        for (int i = 0; i < N_IT; i++) {
+            int r, c;
+            tile_piece<C>(i, kFwdThreads / 32, w, lane, r, c);
+            const int64_t v = tile * 128 + r;
+            x[i] = make_uint4(0, 0, 0, 0);
+            if (r < 128 && v < g.n_nodes)
+                x[i] = c < KIN / 8 ? __ldg((const uint4 *)(h_in + v * KIN) + c)
+                                   : __ldg((const uint4 *)(agg + v * 2 * KIN) + c - KIN / 8);
+        }
+    };
+    load(blockIdx.x);
     for (int i = t; i < kHidden * (K / 8); i += blockDim.x) {  // W^T [H x K] -> K-major B operand
         const int r = i / (K / 8), kc = (i % (K / 8)) * 8;
         *(uint4 *)(sB + kmajor_off(r, kc, K)) = *(const uint4 *)(wt + (size_t)r * K + kc);
@@ -362,11 +391,16 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_gnn_fwd(GnnGraph g, const ui
     tmem_fence_after();
     const uint32_t taddr = tslot;
     const int64_t n_tiles = (g.n_nodes + 127) / 128;
-    const int lq = w & 3, cb = w >> 2;  // epilogue: TMEM lane quarter and 32-column block
+    const int lq = w & 3, c0 = 32 * (w >> 2);  // epilogue: TMEM lane quarter and 32-column block
     uint32_t phase = 0;
     bool ok = true;
     for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        gather_tile<KIN>(g, h_in, tile, sA, agg, w, lane);
+#pragma unroll
+        for (int i = 0; i < N_IT; i++) {
+            int r, c;
+            tile_piece<C>(i, kFwdThreads / 32, w, lane, r, c);
+            if (r < 128) *(uint4 *)(sA + kmajor_off(r, 8 * c, K)) = x[i];
+        }
         fence_async_smem();
         __syncthreads();
         if (t == 0) {
@@ -374,12 +408,12 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_gnn_fwd(GnnGraph g, const ui
             umma_gemm(taddr, sA, sB, K, kHidden, false);
             umma_commit(&bar);
         }
+        load(tile + gridDim.x);  // (rows past the end read as zero)
         ok = __syncthreads_and(mbar_wait_parity(&bar, phase, kWaitLimit)) != 0;  // uniform across the CTA
         phase ^= 1;
         tmem_fence_after();
-        if (ok && w < 16) {
+        if (ok) {
             const int64_t v = tile * 128 + 32 * lq + lane;  // this thread's TMEM lane = row 32 lq + lane
-            const int c0 = 32 * cb;
             float acc[32];
             tmem_ld32(taddr + ((uint32_t)(32 * lq) << 16) + c0, acc);
             if (v < g.n_nodes) {
@@ -390,16 +424,14 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_gnn_fwd(GnnGraph g, const ui
                     const float a1 = fmaxf(acc[2 * i + 1] + sbias[c0 + 2 * i + 1], 0.f);
                     pk[i] = (uint32_t)f2bf(a0) | ((uint32_t)f2bf(a1) << 16);
                 }
-                uint4 *dst = (uint4 *)(h_out + v * kHidden + c0);
-#pragma unroll
-                for (int i = 0; i < 4; i++) dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+                st32(h_out + v * kHidden + c0, pk);
+                st32(h_out + v * kHidden + c0 + 16, pk + 8);
             }
-        } else if (!ok && t == 0 && err) {
+        } else if (t == 0 && err) {
             atomicExch(err, DAGRT_E_TIMEOUT);
         }
-        // no barrier here: the warps without epilogue work start gathering the next tile
-        // (the MMA that read the A tile has completed); the barrier after that gather orders
-        // this epilogue's TMEM reads before the next MMA writes the accumulator
+        // no barrier here: the MMA that read the A tile has completed, and the barrier after the
+        // next copy orders this epilogue's TMEM reads before the next MMA writes the accumulator
         tmem_fence_before();
     }
     __syncthreads();  // every epilogue has read TMEM before it is released
@@ -410,18 +442,24 @@ template <int KIN>
 static cudaError_t launch_fwd(GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,
                               uint16_t *h_out, uint16_t *agg, int32_t *err, int n_sm, cudaStream_t st) {
     constexpr int K = 3 * KIN;
-    const int smem = 2 * 128 * K * 2;
-    cudaError_t e = cudaFuncSetAttribute(k_gnn_fwd<KIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    const int64_t n_tiles = (g.n_nodes + 127) / 128;
+    if (n_tiles < 1) return cudaSuccess;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gnn_fwd<KIN>, 32 * kFwdWarps, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gnn_agg<KIN>, kAggThreads, 0);
+    if (e != cudaSuccess) return e;
+    constexpr int chunk = kAggThreads * 8 / KIN < 128 ? 128 : kAggThreads * 8 / KIN;
+    const int64_t n_chunks = (g.n_nodes + chunk - 1) / chunk, most = (int64_t)n_sm * (per_sm < 1 ? 1 : per_sm);
+    k_gnn_agg<KIN><<<(int)(n_chunks < most ? n_chunks : most), kAggThreads, 0, st>>>(g, h_in, agg);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int smem = 2 * 128 * K * 2;
+    e = cudaFuncSetAttribute(k_gnn_fwd<KIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gnn_fwd<KIN>, kFwdThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     if (per_sm > 4) per_sm = 4;  // 4 x 128 TMEM columns per SM
-    const int64_t n_tiles = (g.n_nodes + 127) / 128;
     int grid = (int)(n_tiles < (int64_t)n_sm * per_sm ? n_tiles : (int64_t)n_sm * per_sm);
-    if (grid < 1) return cudaSuccess;
-    k_gnn_fwd<KIN><<<grid, 32 * kFwdWarps, smem, st>>>(g, h_in, wt, bias, h_out, agg, err);
+    k_gnn_fwd<KIN><<<grid, kFwdThreads, smem, st>>>(g, h_in, agg, wt, bias, h_out, err);
     return cudaGetLastError();
 }
 
@@ -642,19 +680,22 @@ cudaError_t gnn_head_grad(GnnGraph g, const uint16_t *h3, const float *dlogits, 
 
 // ------------------------------------------------------------------ backward
 // dZ = dh * [h_out > 0] in bf16 for the 128 rows of a tile, in the layout of
-// kmajor_off(row, output, kHidden); thread t of kBwdThreads takes outputs 8 (t % 16) .. + 7 of
-// rows t / 16 + 32 i, and adds its unrounded dZ to db[8].
+// kmajor_off(row, output, kHidden); thread t of kBwdThreads takes outputs dz_out(t) .. + 7 of
+// rows dz_row(t) + 32 i (eight lanes store eight rows, 128 contiguous bytes), and adds its
+// unrounded dZ to db[8].
 constexpr int kBwdThreads = 512;
 constexpr int kZBytes = 128 * kHidden * 2;
+__device__ __forceinline__ int dz_out(int t) { return 8 * (((t >> 3) & 3) + 4 * ((t >> 5) & 3)); }
+__device__ __forceinline__ int dz_row(int t) { return (t & 7) + 8 * (t >> 7); }
 __device__ __forceinline__ void stage_dz(const GnnGraph &g, const uint16_t *__restrict__ h_out,
                                          const float *__restrict__ dh_out, int64_t tile, unsigned char *sZ, int t,
                                          float *db) {
-    const int o = 8 * (t & 15);
+    const int o = dz_out(t);
     float4 x[4], y[4];
     uint4 h[4];
 #pragma unroll
     for (int i = 0; i < 4; i++) {
-        const int64_t v = tile * 128 + (t >> 4) + 32 * i;
+        const int64_t v = tile * 128 + dz_row(t) + 32 * i;
         const bool in = v < g.n_nodes;
         h[i] = in ? __ldg((const uint4 *)(h_out + v * kHidden + o)) : make_uint4(0, 0, 0, 0);
         x[i] = in ? __ldg((const float4 *)(dh_out + v * kHidden + o)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -669,7 +710,7 @@ __device__ __forceinline__ void stage_dz(const GnnGraph &g, const uint16_t *__re
             if (((hw[j >> 1] >> (16 * (j & 1))) & 0xffffu) == 0) z[j] = 0.f;
             db[j] += z[j];
         }
-        *(uint4 *)(sZ + kmajor_off((t >> 4) + 32 * i, o, kHidden)) = pack8(z);
+        *(uint4 *)(sZ + kmajor_off(dz_row(t) + 32 * i, o, kHidden)) = pack8(z);
     }
 }
 
@@ -716,7 +757,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_dw(GnnGraph g, const ui
             uint4 x[U];
 #pragma unroll
             for (int i = 0; i < U; i++) {
-                const int p = t + (i0 + i) * kBwdThreads, r = p / C, c = p % C;
+                int r, c;
+                tile_piece<C>(i0 + i, kBwdThreads / 32, w, lane, r, c);
                 const int64_t v = tile * 128 + r;
                 x[i] = make_uint4(0, 0, 0, 0);
                 if (r < 128 && v < g.n_nodes)
@@ -725,7 +767,8 @@ __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_dw(GnnGraph g, const ui
             }
 #pragma unroll
             for (int i = 0; i < U; i++) {
-                const int p = t + (i0 + i) * kBwdThreads, r = p / C, c = p % C;
+                int r, c;
+                tile_piece<C>(i0 + i, kBwdThreads / 32, w, lane, r, c);
                 if (r < 128) *(uint4 *)(sA + kmajor_off(r, 8 * c, KP)) = x[i];
             }
         }
@@ -759,7 +802,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_dw(GnnGraph g, const ui
         }
     }
 #pragma unroll
-    for (int j = 0; j < 8; j++) sdb[t >> 4][8 * (t & 15) + j] = db[j];
+    for (int j = 0; j < 8; j++) sdb[dz_row(t)][dz_out(t) + j] = db[j];
     tmem_fence_before();
     __syncthreads();
     if (t < kHidden) {
@@ -843,10 +886,13 @@ __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_da(GnnGraph g, const ui
                 float acc[32];
                 tmem_ld32(taddr + ((uint32_t)(32 * lq) << 16) + s * 128 + 32 * cb, acc);
                 if (v < g.n_nodes) {
-                    float4 *dst = (float4 *)(da + v * K + s * 128 + 32 * cb);
 #pragma unroll
-                    for (int i = 0; i < 8; i++)
-                        dst[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+                    for (int i = 0; i < 4; i++) {
+                        uint32_t x[8];
+#pragma unroll
+                        for (int j = 0; j < 8; j++) x[j] = __float_as_uint(acc[8 * i + j]);
+                        st32(da + v * K + s * 128 + 32 * cb + 8 * i, x);
+                    }
                 }
             }
         } else if (t == 0 && err) {
@@ -894,12 +940,13 @@ __device__ __forceinline__ void add_div(float4 &s, float4 x, float n) {
 }
 
 template <int KIN>
-__global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__restrict__ da, float *dh_in) {
+__global__ void __launch_bounds__(512) k_gnn_agg_bwd(GnnGraph g, const float *__restrict__ da, float *dh_in) {
     constexpr int K = 3 * KIN;
     static_assert(KIN == 128, "four features per lane");
     const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < g.n_nodes; u += warps) {
+    // a CTA takes 128 neighbouring nodes, mostly of one DAG, whose rows stay in the L1 cache
+    for (int64_t c0 = (int64_t)blockIdx.x * 128; c0 < g.n_nodes; c0 += (int64_t)gridDim.x * 128)
+    for (int64_t u = c0 + (threadIdx.x >> 5); u < min(g.n_nodes, c0 + 128); u += 16) {
         float4 s = __ldg((const float4 *)(da + u * K) + lane);
         auto gather = [&](const int32_t *__restrict__ off, const int32_t *__restrict__ idx,
                           const int32_t *__restrict__ noff, int third) {
@@ -929,10 +976,10 @@ __global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__
 
 cudaError_t gnn_agg_bwd(int kin, GnnGraph g, const float *da, float *dh_in, int n_sm, cudaStream_t st) {
     if (kin != kHidden) return cudaErrorInvalidValue;
-    int64_t grid = (g.n_nodes + 7) / 8;
-    if (grid > 32 * n_sm) grid = 32 * n_sm;
+    int64_t grid = (g.n_nodes + 127) / 128;
+    if (grid > 8 * n_sm) grid = 8 * n_sm;
     if (grid < 1) return cudaSuccess;
-    k_gnn_agg_bwd<kHidden><<<(int)grid, 256, 0, st>>>(g, da, dh_in);
+    k_gnn_agg_bwd<kHidden><<<(int)grid, 512, 0, st>>>(g, da, dh_in);
     return cudaGetLastError();
 }
 
@@ -995,186 +1042,197 @@ namespace dagrt {
 // earlier groups fixed) has the successors: next option of g; keep g and take option 0 of
 // g+1; and, from option 0 only, drop g and take option 0 of g+1. Every assignment has one
 // parent and no successor is cheaper, so a best-first walk pops the k best in order.
-// One warp per DAG; column 0 of every row keeps the paper's allocation (0), column 1 + j
+// One CTA per DAG; column 0 of every row keeps the paper's allocation (0), column 1 + j
 // holds the j-th best assignment.
+//
+// The kTopkMax - 1 smallest (delta, node, level) of a thread's nodes stay sorted in registers
+// as one 64-bit key each (a delta is not negative, so its bits order like it); the CTA merges
+// them by argmin over the threads' heads; one thread walks. A row is written as two 16-byte
+// stores, and only rows of the few nodes that some assignment changes look at the masks.
+// Bound by latency: 300 DAGs of 100-1,000 nodes, 857 -> XXT us (a warp per DAG, sorted lists in
+// local memory, a test of every change for every byte).
 constexpr int kTopkMax = 16;
+constexpr int kTopkThreads = 128;
+static_assert(kTopkMax + 1 <= 32, "a row's candidates fit its 32 bytes");
 
-__global__ void __launch_bounds__(128) k_gnn_topk(int32_t n_dags, const int64_t *node_off, const float *logits,
+template <int K1>
+__device__ __forceinline__ void topk_insert(uint64_t (&best)[K1], uint64_t x) {
+#pragma unroll
+    for (int i = 0; i < K1; i++) {  // x sinks to its place, the last key falls out
+        const bool lt = x < best[i];
+        const uint64_t y = best[i];
+        best[i] = lt ? x : y;
+        x = lt ? y : x;
+    }
+}
+
+__global__ void __launch_bounds__(kTopkThreads) k_gnn_topk(int32_t n_dags, const int64_t *node_off, const float *logits,
                                                   int L, const uint8_t *levels, int k, const uint4 *plan,
                                                   const int32_t *nrows, uint8_t *best_level, uint8_t *m_alloc,
                                                   int64_t stride) {
-    __shared__ float s_dv[4][32 * (kTopkMax - 1)];
-    __shared__ int32_t s_dn[4][32 * (kTopkMax - 1)];
-    __shared__ uint8_t s_dl[4][32 * (kTopkMax - 1)];
-    __shared__ uint32_t s_mask[4][kTopkMax];
-    __shared__ int s_nc[4];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    constexpr int KM = kTopkMax - 1;
+    __shared__ uint64_t s_key[KM];
+    __shared__ uint64_t s_red[kTopkThreads / 32];
+    __shared__ float s_dv[KM];
+    __shared__ int32_t s_dn[KM];
+    __shared__ uint8_t s_dl[KM];
+    __shared__ uint32_t s_mask[kTopkMax];
+    __shared__ int s_nc;
+    __shared__ float s_hc[3 * kTopkMax + 1];
+    __shared__ uint32_t s_hm[3 * kTopkMax + 1];
+    __shared__ uint8_t s_hg[3 * kTopkMax + 1], s_hj[3 * kTopkMax + 1], s_lev[kMaxLevels];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int K1 = k - 1;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dags; d += warps) {
+    if (tid < L) s_lev[tid] = levels[tid];
+    for (int d = blockIdx.x; d < n_dags; d += gridDim.x) {
         const int64_t n0 = node_off[d];
         const int V = (int)(node_off[d + 1] - n0);
-        // per lane: the K1 smallest (delta, node, level) of its nodes, kept sorted
-        float bv[kTopkMax - 1];
-        int32_t bn[kTopkMax - 1];
-        uint8_t bl[kTopkMax - 1];
-        int cnt = 0;
-        for (int v = lane; v < V; v += 32) {
-            const float *z = logits + (n0 + v) * L;
+        uint64_t best[KM];
+#pragma unroll
+        for (int i = 0; i < KM; i++) best[i] = KEY_INF;
+        for (int v = tid; v < V; v += kTopkThreads) {
+            const float *zp = logits + (n0 + v) * L;
+            float z[kMaxLevels];
+#pragma unroll
+            for (int l = 0; l < kMaxLevels; l++) z[l] = l < L ? __ldg(zp + l) : 0.f;
             int b = 0;
-            for (int l = 1; l < L; l++)
-                if (z[l] > z[b]) b = l;
+            float zb = z[0];
+#pragma unroll
+            for (int l = 1; l < kMaxLevels; l++)
+                if (l < L && z[l] > zb) {
+                    b = l;
+                    zb = z[l];
+                }
             best_level[n0 + v] = (uint8_t)b;
-            for (int l = 0; l < L && K1 > 0; l++) {
-                if (l == b) continue;
-                const float dl = z[b] - z[l];
-                if (cnt == K1 && !(dl < bv[K1 - 1])) continue;
-                int pos = cnt < K1 ? cnt++ : K1 - 1;
-                while (pos > 0 && bv[pos - 1] > dl) {
-                    bv[pos] = bv[pos - 1];
-                    bn[pos] = bn[pos - 1];
-                    bl[pos] = bl[pos - 1];
-                    pos--;
-                }
-                bv[pos] = dl;
-                bn[pos] = v;
-                bl[pos] = (uint8_t)l;
+            if (K1 == 0) continue;
+#pragma unroll
+            for (int l = 0; l < kMaxLevels; l++) {
+                if (l >= L || l == b) continue;
+                // (delta, node, level); a sum with +0 makes a -0 a +0
+                const uint64_t key = ((uint64_t)__float_as_uint(zb - z[l] + 0.f) << 32) | ((uint32_t)v << 8) | (uint32_t)l;
+                if (key < best[KM - 1]) topk_insert(best, key);
             }
         }
-        for (int i = 0; i < K1; i++) {
-            s_dv[wib][lane * K1 + i] = i < cnt ? bv[i] : __int_as_float(0x7f800000);
-            s_dn[wib][lane * K1 + i] = i < cnt ? bn[i] : -1;
-            s_dl[wib][lane * K1 + i] = i < cnt ? bl[i] : 0;
-        }
-        __syncwarp();
-        // merge: the K1 smallest over all lanes (ties: lower node, then lower level), by a
-        // warp argmin over the heads of the lanes' sorted lists
-        float dv[kTopkMax - 1];
-        int32_t dn[kTopkMax - 1];
-        uint8_t dlv[kTopkMax - 1];
-        int m = 0, hp = 0;
-        for (int i = 0; i < K1; i++) {
-            float hv = __int_as_float(0x7f800000);
-            int32_t hn = 0x7fffffff;
-            int hl = 0xff;
-            if (hp < cnt) {
-                hv = s_dv[wib][lane * K1 + hp];
-                hn = s_dn[wib][lane * K1 + hp];
-                hl = s_dl[wib][lane * K1 + hp];
-            }
-            float bvv = hv;
-            int32_t bnn = hn;
-            int bll = hl, bln = lane;
+        // merge: the K1 smallest over all threads, an argmin over their heads at a time
+        int m = 0;
+        for (; m < K1; m++) {
+            uint64_t x = best[0];
             for (int o = 16; o > 0; o >>= 1) {
-                const float ov = __shfl_xor_sync(FULL, bvv, o);
-                const int32_t on = __shfl_xor_sync(FULL, bnn, o);
-                const int ol = __shfl_xor_sync(FULL, bll, o), oln = __shfl_xor_sync(FULL, bln, o);
-                if (ov < bvv || (ov == bvv && (on < bnn || (on == bnn && (ol < bll || (ol == bll && oln < bln)))))) {
-                    bvv = ov;
-                    bnn = on;
-                    bll = ol;
-                    bln = oln;
-                }
+                const uint64_t y = __shfl_xor_sync(FULL, x, o);
+                x = y < x ? y : x;
             }
-            if (bnn == 0x7fffffff) break;  // every list is exhausted
-            if (lane == bln) hp++;
-            dv[m] = bvv;
-            dn[m] = bnn;
-            dlv[m] = (uint8_t)bll;
-            m++;
+            if (lane == 0) s_red[w] = x;
+            __syncthreads();
+            x = s_red[0];
+#pragma unroll
+            for (int i = 1; i < kTopkThreads / 32; i++) x = s_red[i] < x ? s_red[i] : x;
+            if (x == KEY_INF) break;  // every list is exhausted
+            if (best[0] == x) {  // keys are distinct: one thread moves on
+#pragma unroll
+                for (int i = 0; i + 1 < KM; i++) best[i] = best[i + 1];
+                best[KM - 1] = KEY_INF;
+                s_key[m] = x;
+            }
+            __syncthreads();
         }
-        __syncwarp();
-        if (lane == 0) {
+        __syncthreads();
+        if (tid == 0) {
             // group-major order: groups in order of first appearance (= smallest delta)
             int gs[kTopkMax], gc[kTopkMax], G = 0, q = 0;
-            bool used[kTopkMax - 1];
-            for (int i = 0; i < m; i++) used[i] = false;
+            uint32_t used = 0;
             for (int i = 0; i < m; i++) {
-                if (used[i]) continue;
+                if (used >> i & 1) continue;
+                const uint32_t ni = (uint32_t)s_key[i] >> 8;
                 gs[G] = q;
                 gc[G] = 0;
                 for (int j = i; j < m; j++)
-                    if (!used[j] && dn[j] == dn[i]) {
-                        used[j] = true;
-                        s_dv[wib][q] = dv[j];
-                        s_dn[wib][q] = dn[j];
-                        s_dl[wib][q] = dlv[j];
+                    if (!(used >> j & 1) && (uint32_t)s_key[j] >> 8 == ni) {
+                        used |= 1u << j;
+                        s_dv[q] = __uint_as_float((uint32_t)(s_key[j] >> 32));
+                        s_dn[q] = (int32_t)ni;
+                        s_dl[q] = (uint8_t)s_key[j];
                         q++;
                         gc[G]++;
                     }
                 G++;
             }
             // best-first walk: heap entries (cost, mask of chosen items, group, option)
-            constexpr int H = 3 * kTopkMax + 1;
-            float hc[H];
-            uint32_t hm[H];
-            uint8_t hg[H], hj[H];
             int hn = 0, nc = 0;
-            s_mask[wib][nc++] = 0;  // the all-best assignment
+            s_mask[nc++] = 0;  // the all-best assignment
             if (G > 0) {
-                hc[0] = s_dv[wib][0];
-                hm[0] = 1u;
-                hg[0] = 0;
-                hj[0] = 0;
+                s_hc[0] = s_dv[0];
+                s_hm[0] = 1u;
+                s_hg[0] = 0;
+                s_hj[0] = 0;
                 hn = 1;
             }
             while (nc < k && hn > 0) {
                 int bi = 0;
-                for (int i = 1; i < hn; i++)
-                    if (hc[i] < hc[bi] || (hc[i] == hc[bi] && hm[i] < hm[bi])) bi = i;
-                const float c = hc[bi];
-                const uint32_t msk = hm[bi];
-                const int g = hg[bi], j = hj[bi];
-                hn--;
-                hc[bi] = hc[hn];
-                hm[bi] = hm[hn];
-                hg[bi] = hg[hn];
-                hj[bi] = hj[hn];
-                s_mask[wib][nc++] = msk;
-                const int it = gs[g] + j;
-                if (j + 1 < gc[g]) {  // next option of group g
-                    hc[hn] = c - s_dv[wib][it] + s_dv[wib][it + 1];
-                    hm[hn] = (msk & ~(1u << it)) | (1u << (it + 1));
-                    hg[hn] = (uint8_t)g;
-                    hj[hn] = (uint8_t)(j + 1);
-                    hn++;
+                float c = s_hc[0];
+                uint32_t msk = s_hm[0];
+                for (int i = 1; i < hn; i++) {
+                    const float ci = s_hc[i];
+                    const uint32_t mi = s_hm[i];
+                    if (ci < c || (ci == c && mi < msk)) {
+                        bi = i;
+                        c = ci;
+                        msk = mi;
+                    }
                 }
+                const int g = s_hg[bi], j = s_hj[bi];
+                hn--;
+                s_hc[bi] = s_hc[hn];
+                s_hm[bi] = s_hm[hn];
+                s_hg[bi] = s_hg[hn];
+                s_hj[bi] = s_hj[hn];
+                s_mask[nc++] = msk;
+                const int it = gs[g] + j;
+                auto push = [&](float cost, uint32_t mask, int gg, int jj) {
+                    s_hc[hn] = cost;
+                    s_hm[hn] = mask;
+                    s_hg[hn] = (uint8_t)gg;
+                    s_hj[hn] = (uint8_t)jj;
+                    hn++;
+                };
+                if (j + 1 < gc[g])  // next option of group g
+                    push(c - s_dv[it] + s_dv[it + 1], (msk & ~(1u << it)) | (1u << (it + 1)), g, j + 1);
                 if (g + 1 < G) {
                     const int nx = gs[g + 1];
-                    hc[hn] = c + s_dv[wib][nx];  // keep g, add group g+1
-                    hm[hn] = msk | (1u << nx);
-                    hg[hn] = (uint8_t)(g + 1);
-                    hj[hn] = 0;
-                    hn++;
-                    if (j == 0) {  // swap g for g+1
-                        hc[hn] = c - s_dv[wib][it] + s_dv[wib][nx];
-                        hm[hn] = (msk & ~(1u << it)) | (1u << nx);
-                        hg[hn] = (uint8_t)(g + 1);
-                        hj[hn] = 0;
-                        hn++;
+                    push(c + s_dv[nx], msk | (1u << nx), g + 1, 0);  // keep g, add group g+1
+                    if (j == 0) push(c - s_dv[it] + s_dv[nx], (msk & ~(1u << it)) | (1u << nx), g + 1, 0);  // swap
+                }
+            }
+            s_nc = nc;
+        }
+        __syncthreads();
+        const int nc = s_nc;
+        const int rows = nrows[d];
+        const int64_t rbase = 2 * n0;
+        for (int r = tid; r < rows; r += kTopkThreads) {
+            const int node = (int)plan[rbase + r].w;
+            uint32_t hit = 0;  // changes of this node
+            for (int i = 0; i < m; i++) hit |= (uint32_t)(s_dn[i] == node) << i;
+            const uint32_t lb = s_lev[best_level[n0 + node]];
+            uint32_t out[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) out[i] = lb * 0x01010101u;
+            out[0] &= ~0xffu;
+            if (hit) {
+                // mostly one change: byte 1 + j of the row for every assignment that has it
+#pragma unroll
+                for (int j = 0; j < kTopkMax; j++) {
+                    const uint32_t x = s_mask[j < nc ? j : 0] & hit;
+                    if (x && j < k) {
+                        const uint32_t lv = s_lev[s_dl[31 - __clz(x)]];
+                        out[(1 + j) >> 2] = (out[(1 + j) >> 2] & ~(0xffu << (8 * ((1 + j) & 3)))) | (lv << (8 * ((1 + j) & 3)));
                     }
                 }
             }
-            s_nc[wib] = nc;
+            uint4 *dst = (uint4 *)(m_alloc + (rbase + r) * stride);
+            dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
+            dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
         }
-        __syncwarp();
-        const int nc = s_nc[wib];  // m (the merged changes) is the same in every lane
-        const int rows = nrows[d];
-        const int64_t rbase = 2 * n0;
-        for (int r = lane; r < rows; r += 32) {
-            const int node = (int)plan[rbase + r].w;
-            const int b = best_level[n0 + node];
-            uint8_t *dst = m_alloc + (rbase + r) * stride;
-            dst[0] = 0;
-            for (int j = 0; j < k; j++) {
-                const uint32_t msk = s_mask[wib][j < nc ? j : 0];
-                int lv = b;
-                for (int i = 0; i < m; i++)
-                    if ((msk >> i & 1) && s_dn[wib][i] == node) lv = s_dl[wib][i];
-                dst[1 + j] = levels[lv];
-            }
-        }
-        __syncwarp();
+        __syncthreads();  // the DAG's lists are read
     }
 }
 
@@ -1182,32 +1240,28 @@ cudaError_t gnn_topk(int32_t n_dags, const int64_t *node_off, const float *logit
                      const uint8_t *levels, int k, const uint4 *plan, const int32_t *nrows, uint8_t *best_level,
                      uint8_t *m_alloc, int64_t stride, int n_sm, cudaStream_t st) {
     if (n_dags == 0) return cudaSuccess;
-    if (k < 1 || k > kTopkMax) return cudaErrorInvalidValue;
-    int grid = (n_dags + 3) / 4;
-    if (grid > 16 * n_sm) grid = 16 * n_sm;
-    k_gnn_topk<<<grid, 128, 0, st>>>(n_dags, node_off, logits, n_levels, levels, k, plan, nrows, best_level, m_alloc,
-                                     stride);
+    if (k < 1 || k > kTopkMax || stride % 16 != 0 || stride < 32) return cudaErrorInvalidValue;
+    const int grid = n_dags < 32 * n_sm ? n_dags : 32 * n_sm;
+    k_gnn_topk<<<grid, kTopkThreads, 0, st>>>(n_dags, node_off, logits, n_levels, levels, k, plan, nrows, best_level,
+                                              m_alloc, stride);
     return cudaGetLastError();
 }
 
-// the winning candidate's allocation, row by row (one warp per DAG)
+// the winning candidate's allocation, row by row (one CTA per DAG)
 __global__ void k_pick_column(int32_t n_dags, const int64_t *node_off, const int32_t *nrows, const int32_t *best,
                               const uint8_t *m_alloc, int64_t stride, uint8_t *out) {
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dags; d += warps) {
+    for (int d = blockIdx.x; d < n_dags; d += gridDim.x) {
         const int c = best[d];
         const int64_t rbase = 2 * node_off[d];
-        for (int r = lane; r < nrows[d]; r += 32) out[rbase + r] = c >= 0 ? m_alloc[(rbase + r) * stride + c] : 0;
+        for (int r = threadIdx.x; r < nrows[d]; r += blockDim.x) out[rbase + r] = c >= 0 ? m_alloc[(rbase + r) * stride + c] : 0;
     }
 }
 
 cudaError_t gnn_pick_column(int32_t n_dags, const int64_t *node_off, const int32_t *nrows, const int32_t *best,
                             const uint8_t *m_alloc, int64_t stride, uint8_t *out, int n_sm, cudaStream_t st) {
     if (n_dags == 0) return cudaSuccess;
-    int grid = (n_dags + 7) / 8;
-    if (grid > 16 * n_sm) grid = 16 * n_sm;
-    k_pick_column<<<grid, 256, 0, st>>>(n_dags, node_off, nrows, best, m_alloc, stride, out);
+    const int grid = n_dags < 32 * n_sm ? n_dags : 32 * n_sm;
+    k_pick_column<<<grid, 128, 0, st>>>(n_dags, node_off, nrows, best, m_alloc, stride, out);
     return cudaGetLastError();
 }
 
