@@ -38,7 +38,7 @@ static int graph_smem(int v) { return 4 * ((kGraphWarps + 2) * v + 1); }
 // its cursors, and it fills 32 edges at a time; lanes with the same target rank themselves
 // with a match. Larger DAGs: counts and fill in global memory with atomics, then an insertion
 // sort per list. Bound by the latency of a DAG's passes: eight warps a DAG instead of one
-// take 300 DAGs of 100-1,000 nodes from 725 to XXG us.
+// take 300 DAGs of 100-1,000 nodes from 725 to 110 us.
 __global__ void __launch_bounds__(kGraphThreads)
     k_gnn_graph(int32_t n_dags, const int64_t *node_off, const int64_t *edge_off, const int32_t *row_ptr,
                 const int32_t *col, const int32_t *status, int32_t *pred_off, int32_t *pred_idx, int32_t *succ_off,
@@ -307,8 +307,9 @@ __device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const
 // neighbours in the batch, so mostly of one DAG, whose rows (140 KB for 550 nodes) stay in
 // the L1 cache: the kernel uses no shared memory, and that is why it is apart from the
 // matrix product, whose operands fill it. Bound by the L1 rate and the additions.
-// 165,000 nodes, 2.8 M edges, 128 features: XXa us, and the product XXb, where one kernel for
-// both took 190; 16 features: 97 -> XXc and XXd.
+// 165,000 nodes, 2.8 M edges, 128 features: 116 us, and the product 52, where one kernel for
+// both took 190 (the rows of a CTA's nodes from a chunk next to its SM's other CTAs: 127, the
+// chunks' degrees then differ by SM); 16 features: 97 -> 31 and 24.
 constexpr int kAggThreads = 512;
 template <int KIN>
 __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *__restrict__ h,
@@ -327,14 +328,14 @@ __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const ui
 }
 
 // 16-byte piece i of warp w's share of a [128 rows x 8 C columns] tile in the layout of
-// kmajor_off: eight lanes store eight rows of one column piece, 128 contiguous bytes, and the
-// warp reads 64 (C a multiple of 4) or 32 contiguous bytes per row
+// kmajor_off. A warp takes RW rows of CL pieces: whole 128-byte lines of four rows (C a
+// multiple of 8; two lanes then store to the same banks) or 32 bytes of 16 rows.
 template <int C>
 __device__ __forceinline__ void tile_piece(int i, int warps, int w, int lane, int &r, int &c) {
-    constexpr int CL = C % 4 == 0 ? 4 : 2, RG = 4 / CL;  // columns of a warp's piece, 8-row groups of it
-    const int p = i * warps + w, cg = p % (C / CL), rg = p / (C / CL) * RG;
-    c = cg * CL + (lane >> 3) % CL;
-    r = 8 * (rg + (lane >> 3) / CL) + (lane & 7);
+    constexpr int CL = C % 8 == 0 ? 8 : 2, RW = 32 / CL;
+    const int p = i * warps + w;
+    c = p % (C / CL) * CL + lane / RW;
+    r = p / (C / CL) * RW + lane % RW;
 }
 
 // 32 bytes in one store (an aligned sector)
@@ -477,7 +478,7 @@ cudaError_t gnn_layer_fwd(int kin, GnnGraph g, const uint16_t *h_in, const uint1
 // shared memory, dh3 with four outputs per lane (their weights in registers), so every store
 // is a whole line. The loss is reduced per CTA in a fixed order. Bound by the FMAs of the two
 // products; with one node's row per thread for the stores too, and one CTA an SM, 110,000
-// nodes took 285 us (now XXH), 165,000 without labels 77 (now XXI).
+// nodes took 285 us (now 89), 165,000 without labels 77 (now 39).
 constexpr int kHeadThreads = 128;
 constexpr int kHeadMaxCtas = 1024;  // partial losses
 __global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uint16_t *__restrict__ h3,
@@ -611,7 +612,7 @@ cudaError_t gnn_head(GnnGraph g, const uint16_t *h3, const float *wh, const floa
 // dWh = h3^T dlogits, dbh = sum dlogits: CTA c reduces a fixed node range in tiles of
 // kHgTile nodes whose dlogits are staged; thread (o, p) adds output row o over every 8th
 // node from p, and the parts are added in order. Bound by the loads of h3 (one line per node
-// and warp); with one node after another per CTA it took 395 us for 110,000 nodes (now XXD).
+// and warp); with one node after another per CTA it took 395 us for 110,000 nodes (now 44).
 constexpr int kHgParts = 8, kHgTile = 64;
 __global__ void __launch_bounds__(kHidden * kHgParts) k_gnn_head_grad(GnnGraph g, const uint16_t *__restrict__ h3,
                                                                      const float *__restrict__ dlogits, int L,
@@ -719,8 +720,8 @@ __device__ __forceinline__ void stage_dz(const GnnGraph &g, const uint16_t *__re
 // mean_pred h | mean_succ h] comes from h and from the means the forward pass kept. The
 // accumulators stay in TMEM across tiles (128 columns per 128 features); db_part = column
 // sums of dZ in a fixed order. Bound by reading A, dh and h_out once: 512 threads keep 24
-// 16-byte loads each in flight. 110,000 nodes: 636 -> XXW us a 128-wide layer (128 threads
-// gathered the means again and transposed through 2-byte stores), the first 518 -> XX1.
+// 16-byte loads each in flight. 110,000 nodes: 636 -> 62 us a 128-wide layer (128 threads
+// gathered the means again and transposed through 2-byte stores), the first 518 -> 35.
 template <int KIN>
 __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_dw(GnnGraph g, const uint16_t *__restrict__ h_in,
                                                             const uint16_t *__restrict__ agg,
@@ -836,7 +837,7 @@ cudaError_t gnn_layer_bwd_dw(int kin, int layer, GnnGraph g, const uint16_t *h_i
 // dA = dZ W^T per 128-row tile: A operand dZ [rows x H], B operand W [K x H] (resident),
 // three 128-column TMEM blocks for K = 384. Bound by writing dA (1.5 KB a node): every thread
 // writes 128 contiguous bytes of its row per 32 columns, and 512 threads stage the next dZ
-// while others still write. 110,000 nodes: 380 -> XXA us (128 threads, 4-byte stores).
+// while others still write. 110,000 nodes: 380 -> 70 us (128 threads, 4-byte stores).
 template <int KIN>
 __global__ void __launch_bounds__(kBwdThreads) k_gnn_bwd_da(GnnGraph g, const uint16_t *__restrict__ h_out,
                                                             const float *__restrict__ dh_out,
@@ -926,7 +927,7 @@ cudaError_t gnn_layer_bwd_da(int kin, GnnGraph g, const uint16_t *h_out, const f
 // sum keeps its order. x / n is x (1/n) with one Newton step on the remainder, which rounds
 // like the division (Markstein, "Computation of elementary functions on the IBM RISC
 // System/6000", 1990) as long as nothing is subnormal. Bound by the rows it gathers from L2
-// (512 bytes per edge and direction). 110,000 nodes, 740,000 edges: 277 -> XXB us.
+// (512 bytes per edge and direction). 110,000 nodes, 740,000 edges: 277 -> 105 us.
 __device__ __forceinline__ void add_div(float4 &s, float4 x, float n) {
     const float r = __frcp_rn(n);
     auto div = [&](float a) {
@@ -940,13 +941,12 @@ __device__ __forceinline__ void add_div(float4 &s, float4 x, float n) {
 }
 
 template <int KIN>
-__global__ void __launch_bounds__(512) k_gnn_agg_bwd(GnnGraph g, const float *__restrict__ da, float *dh_in) {
+__global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__restrict__ da, float *dh_in) {
     constexpr int K = 3 * KIN;
     static_assert(KIN == 128, "four features per lane");
     const int lane = threadIdx.x & 31;
-    // a CTA takes 128 neighbouring nodes, mostly of one DAG, whose rows stay in the L1 cache
-    for (int64_t c0 = (int64_t)blockIdx.x * 128; c0 < g.n_nodes; c0 += (int64_t)gridDim.x * 128)
-    for (int64_t u = c0 + (threadIdx.x >> 5); u < min(g.n_nodes, c0 + 128); u += 16) {
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < g.n_nodes; u += warps) {
         float4 s = __ldg((const float4 *)(da + u * K) + lane);
         auto gather = [&](const int32_t *__restrict__ off, const int32_t *__restrict__ idx,
                           const int32_t *__restrict__ noff, int third) {
@@ -976,10 +976,10 @@ __global__ void __launch_bounds__(512) k_gnn_agg_bwd(GnnGraph g, const float *__
 
 cudaError_t gnn_agg_bwd(int kin, GnnGraph g, const float *da, float *dh_in, int n_sm, cudaStream_t st) {
     if (kin != kHidden) return cudaErrorInvalidValue;
-    int64_t grid = (g.n_nodes + 127) / 128;
-    if (grid > 8 * n_sm) grid = 8 * n_sm;
+    int64_t grid = (g.n_nodes + 7) / 8;
+    if (grid > 32 * n_sm) grid = 32 * n_sm;
     if (grid < 1) return cudaSuccess;
-    k_gnn_agg_bwd<kHidden><<<(int)grid, 512, 0, st>>>(g, da, dh_in);
+    k_gnn_agg_bwd<kHidden><<<(int)grid, 256, 0, st>>>(g, da, dh_in);
     return cudaGetLastError();
 }
 
@@ -1049,7 +1049,7 @@ namespace dagrt {
 // as one 64-bit key each (a delta is not negative, so its bits order like it); the CTA merges
 // them by argmin over the threads' heads; one thread walks. A row is written as two 16-byte
 // stores, and only rows of the few nodes that some assignment changes look at the masks.
-// Bound by latency: 300 DAGs of 100-1,000 nodes, 857 -> XXT us (a warp per DAG, sorted lists in
+// Bound by latency: 300 DAGs of 100-1,000 nodes, 857 -> 53 us (a warp per DAG, sorted lists in
 // local memory, a test of every change for every byte).
 constexpr int kTopkMax = 16;
 constexpr int kTopkThreads = 128;
