@@ -366,9 +366,10 @@ int dagrt_realise(dagrt_ctx *ctx, int32_t V, const int32_t *row_ptr, const int32
  *               groups (Theorem 1's sum splits at group ends), as many as fit in this many
  *               rows (a longer group alone); 8 .. 256. Default 64.
  *   item_warps  candidate bounds: warps per CTA of the work-item kernel, 1 .. 8. Default 4.
- *   cta_smem    scheduler: k in 1 .. 4 = CTA teams keep their workspace in shared memory
- *               while it takes at most 1/k of a CTA's shared memory (smallest large DAGs
- *               first; k teams then fit per SM), 0 = always in global memory. Default 2. */
+ *   cta_smem    scheduler: k in 1 .. 4 = CTA teams keep their workspace in shared memory,
+ *               one class of DAGs while it takes at most 1/k of a CTA's shared memory
+ *               (smallest large DAGs first; k teams then fit per SM) and another while it
+ *               fits at all, 0 = always in global memory. Default 2. */
 typedef struct {
     int32_t warp_max_v;
     int32_t chunk_rows;

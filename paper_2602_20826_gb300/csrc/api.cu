@@ -63,7 +63,7 @@ struct dagrt_ctx {
     DevicePool pool;
     // side streams: the scheduler's size-class kernels run concurrently, forked from and
     // joined back into `stream` with events
-    static constexpr int kSide = 18;  // one per scheduler size class
+    static constexpr int kSide = 19;  // one per scheduler size class
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork = nullptr, join[kSide] = {};
     bool side_ready = false;
@@ -124,9 +124,11 @@ namespace {
 // with the edge capacity of its densest DAG (finer classes than powers of two keep the
 // workspaces close to the DAGs' sizes, so more teams fit an SM)
 constexpr int kNumWarpClasses = 256 / kWarpClassStep;
-// classes after the warp classes: CTA teams with a shared-memory workspace, then CTA teams
-// with global workspaces
-constexpr int kClsCtaSmem = kNumWarpClasses, kClsCtaGlobal = kNumWarpClasses + 1, kNumClasses = kNumWarpClasses + 2;
+// classes after the warp classes: CTA teams with a shared-memory workspace (of at most
+// 1/cta_smem, then of at most all of a CTA's), then CTA teams with global workspaces
+constexpr int kNumSmemClasses = 2;
+constexpr int kClsCtaSmem = kNumWarpClasses, kClsCtaGlobal = kClsCtaSmem + kNumSmemClasses,
+              kNumClasses = kClsCtaGlobal + 1;
 static_assert(dagrt_ctx::kSide >= kNumClasses, "a side stream per size class");
 
 struct Plan {
@@ -159,7 +161,7 @@ struct dagrt_batch {
     int32_t *counters = nullptr;  // [kNumClasses] work-stealing counters of the size classes
     int class_off[kNumClasses + 1] = {0};
     int max_v = 0, big_vcap = 0, big_ecap = 0, big_grid = 0;
-    int smem_vcap = 0, smem_ecap = 0;  // capacity of the shared-memory CTA class
+    int smem_vcap[kNumSmemClasses] = {0}, smem_ecap[kNumSmemClasses] = {0};  // capacities of the shared-memory CTA classes
     int wcap_v[kNumWarpClasses] = {0}, wcap_e[kNumWarpClasses] = {0};  // capacities of the warp classes
     unsigned char *gws = nullptr;  // pooled, gws_cap bytes
     int64_t gws_stride = 0;
@@ -329,9 +331,9 @@ void dagrt_batch_free(dagrt_batch *b) {
 
 // Size classes for the scheduler: a DAG goes to the smallest warp class whose shared-memory
 // workspace holds its V nodes and E edges, among the classes of at most tune.warp_max_v
-// nodes; the rest go to CTA teams -- with a shared-memory workspace while the class's
+// nodes; the rest go to CTA teams -- with a shared-memory workspace while a class's
 // capacity (largest V and E so far, smallest DAGs first) still fits 1/tune.cta_smem of a
-// CTA's shared memory (cta_smem = 0: never), else with global workspaces. Each class is ordered by
+// CTA's shared memory, or all of it (cta_smem = 0: never), else with global workspaces. Each class is ordered by
 // descending node count (longest work first). Host work plus one list upload.
 static int partition_classes(dagrt_batch *b) {
     dagrt_ctx *ctx = b->ctx;
@@ -358,33 +360,31 @@ static int partition_classes(dagrt_batch *b) {
     }
     std::stable_sort(big.begin(), big.end(),
                      [&](int x, int y) { return hn[x + 1] - hn[x] > hn[y + 1] - hn[y]; });  // descending V
-    // cta_smem = k: a workspace takes at most 1/k of the shared memory, so k teams fit per SM
-    const int64_t limit = b->tune.cta_smem > 0 ? sched_smem_limit() / b->tune.cta_smem : 0;
-    int sv = 0, gv = 0;
-    int64_t se = 0, ge = 0;
-    std::vector<char> in_smem(big.size(), 0);
+    const int64_t whole = b->tune.cta_smem > 0 ? sched_smem_limit() : 0;
+    const int64_t limit[kNumSmemClasses] = {b->tune.cta_smem > 0 ? whole / b->tune.cta_smem : 0, whole};
+    int sv[kNumSmemClasses] = {0}, gv = 0;
+    int64_t se[kNumSmemClasses] = {0}, ge = 0;
+    std::vector<int32_t> big_cls(big.size());
     for (int i = (int)big.size() - 1; i >= 0; i--) {  // smallest first
         const int d = big[i];
         const int v = (int)(hn[d + 1] - hn[d]);
         const int64_t ed = he[d + 1] - he[d];
-        const int nv = std::max(sv, v);
-        const int64_t ne = std::max(se, ed);
-        if (ne < (1ll << 30) && sched_ws_bytes(nv, (int)ne) <= limit) {
-            sv = nv;
-            se = ne;
-            in_smem[i] = 1;
+        int c = kClsCtaGlobal;
+        for (int k = 0; k < kNumSmemClasses && c == kClsCtaGlobal; k++) {
+            const int nv = std::max(sv[k], v);
+            const int64_t ne = std::max(se[k], ed);
+            if (ne < (1ll << 30) && sched_smem_ws_bytes(nv, (int)ne) <= limit[k]) {
+                sv[k] = nv;
+                se[k] = ne;
+                c = kClsCtaSmem + k;
+            }
         }
-    }
-    std::vector<int32_t> big_cls(big.size());
-    for (size_t i = 0; i < big.size(); i++) {
-        const int d = big[i];
-        const int c = in_smem[i] ? kClsCtaSmem : kClsCtaGlobal;
+        if (c == kClsCtaGlobal) {
+            gv = std::max(gv, v);
+            ge = std::max(ge, ed);
+        }
         big_cls[i] = c;
         count[c]++;
-        if (!in_smem[i]) {
-            gv = std::max(gv, (int)(hn[d + 1] - hn[d]));
-            ge = std::max(ge, he[d + 1] - he[d]);
-        }
     }
     // the class lists, each in descending V (equal V: ascending DAG id), in pinned memory
     int off = 0, pos[kNumClasses];
@@ -412,8 +412,10 @@ static int partition_classes(dagrt_batch *b) {
         b->wcap_v[c] = (c + 1) * kWarpClassStep;
         b->wcap_e[c] = (int)std::max<int64_t>(wecap[c], 1);
     }
-    b->smem_vcap = sv;
-    b->smem_ecap = (int)se;
+    for (int k = 0; k < kNumSmemClasses; k++) {
+        b->smem_vcap[k] = sv[k];
+        b->smem_ecap[k] = (int)se[k];
+    }
     b->big_vcap = gv;
     b->big_ecap = (int)ge;
     if (n_dags > 0) {
@@ -740,9 +742,9 @@ extern "C" int dagrt_schedule(dagrt_batch *b, int32_t variant, const dagrt_sched
                 a.vcap = b->wcap_v[c];
                 a.ecap = b->wcap_e[c];
                 CK(sched_launch_warp(a, ctx->n_sm, st), "launch scheduler (warp teams)");
-            } else if (c == kClsCtaSmem) {
-                a.vcap = b->smem_vcap;
-                a.ecap = b->smem_ecap;
+            } else if (c < kClsCtaGlobal) {
+                a.vcap = b->smem_vcap[c - kClsCtaSmem];
+                a.ecap = b->smem_ecap[c - kClsCtaSmem];
                 CK(sched_launch_cta_smem(a, ctx->n_sm, st), "launch scheduler (CTA teams, shared memory)");
             } else {
                 a.gws = b->gws;

@@ -9,7 +9,7 @@
 namespace dagrt {
 
 constexpr int kWarpsPerCta = 4;    // independent warp teams per CTA (small DAGs; 4 measured 3% faster than 2 on the 10,000-DAG batch)
-constexpr int kCtaThreads = 256;   // threads of a CTA team with a shared-memory workspace
+constexpr int kCtaThreads = 128;   // threads of a CTA team with a shared-memory workspace
 constexpr int kCtaThreadsGlobal = 384;  // threads of a CTA team with a global workspace (DAGs too large for shared
                                        // memory; 384 measured 13% faster than 256 on 200 DAGs of 2,000-20,000 nodes)
 constexpr int kEdgesPerNode = 12;  // warp teams take DAGs of at most this many edges per node of warp_max_v
@@ -51,13 +51,14 @@ struct SchedArgs {
     int32_t vcap, ecap;
 };
 
-int64_t sched_ws_bytes(int vc, int ec);
+int64_t sched_ws_bytes(int vc, int ec);       // a global workspace for DAGs of up to vc nodes and ec edges
+int64_t sched_smem_ws_bytes(int vc, int ec);  // one in shared memory
 // warp teams: the workspace (a.vcap, a.ecap) of kWarpsPerCta teams must fit sched_smem_limit()
 cudaError_t sched_launch_warp(const SchedArgs &a, int n_sm, cudaStream_t st);
 int sched_cta_grid(int n_sm);
 cudaError_t sched_launch_cta(const SchedArgs &a, int grid, cudaStream_t st);
-// CTA teams with the workspace (a.vcap, a.ecap) in shared memory: sched_ws_bytes of the
-// class must not exceed sched_smem_limit()
+// CTA teams with the workspace (a.vcap, a.ecap) in shared memory: sched_smem_ws_bytes of
+// the class must not exceed sched_smem_limit()
 int64_t sched_smem_limit();
 cudaError_t sched_launch_cta_smem(const SchedArgs &a, int n_sm, cudaStream_t st);
 
