@@ -369,10 +369,42 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
     uint64_t bound = 0;
     int64_t nextra = 0;
     int nrows = 0, nseg = 0, nrel = acc.nrel;
-    // The scalar part is stored by all lanes alike (one transaction, and no divergent branch).
+    // The scalar part is stored by all lanes alike (one transaction, and no divergent branch);
+    // the optional outputs of one row, segment or node by a lane per field: lanes 0 .. 4 hold
+    // {id, group, SMs, load's two halves} and where they go, so five stores are one.
+    struct Field {
+        int32_t *p;  // NULL: not wanted, or no field of this lane
+        int step;
+    };
+    auto field = [&](int32_t *id, int32_t *group, int32_t *m, int64_t *load) {
+        Field f;
+        f.p = lane == 0 ? id : lane == 1 ? group : lane == 2 ? m : nullptr;
+        f.step = 1;
+        if (load && (lane == 3 || lane == 4)) {
+            f.p = (int32_t *)load + (lane - 3);
+            f.step = 2;
+        }
+        return f;
+    };
+    auto store = [&](const Field &f, int i, int id, int j, uint32_t m, uint32_t load) {
+        if (f.p) f.p[(int64_t)i * f.step] = lane == 0 ? id : lane == 1 ? j : lane == 2 ? (int)m : lane == 3 ? (int)load : 0;
+    };
+    auto at = [](auto *p, int64_t i) { return p ? p + i : nullptr; };
+    Field f_row = {nullptr, 1}, f_seg = {nullptr, 1};
+    if constexpr (FULL_OUT) {
+        f_row = field(at(a.o.row_id, g.rbase), at(a.o.row_group, g.rbase), at(a.o.row_m0, g.rbase), at(a.o.row_load, g.rbase));
+        f_seg = field(at(a.o.seg_parent, g.n0), at(a.o.seg_group, g.n0), at(a.o.seg_m, g.n0), at(a.o.seg_load, g.n0));
+    }
+    Field f_node = {nullptr, 1};
+    if constexpr (FULL_OUT) f_node = field(nullptr, at(a.o.exec_group, g.n0), at(a.o.m, g.n0), nullptr);
     // Plan row i runs `id` (a segment: >= V) of node `owner` with `load`; z = m | k << 16
     auto write_row = [&](int i, int id, int owner, int j, uint32_t load, uint32_t z, uint32_t c, bool last) {
         if (!FULL_OUT || plan) plan[i] = make_uint4(load, c, z | (last ? 1u << 24 : 0u), (uint32_t)owner);
+        if constexpr (FULL_OUT) store(f_row, i, id, j, z & 0xffffu, load);
+    };
+    // ... a different row in every lane
+    auto write_own_row = [&](int i, int id, int j, uint32_t load, uint32_t z, uint32_t c, bool last) {
+        if (!FULL_OUT || plan) plan[i] = make_uint4(load, c, z | (last ? 1u << 24 : 0u), (uint32_t)id);
         if constexpr (FULL_OUT) {
             if (a.o.row_id) a.o.row_id[g.rbase + i] = id;
             if (a.o.row_group) a.o.row_group[g.rbase + i] = j;
@@ -382,6 +414,16 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
     };
     // node r finishes with group j on m SMs
     auto finish = [&](uint32_t r, int id, int j, uint32_t m) {
+        w.left(r) = 0;
+        if constexpr (FULL_OUT) {
+            store(f_node, id, id, j, m, 0u);
+        } else if (node_out) {
+            if (a.o.exec_group) a.o.exec_group[g.n0 + id] = j;
+            if (a.o.m) a.o.m[g.n0 + id] = (int32_t)m;
+        }
+    };
+    // ... a different node in every lane
+    auto finish_own = [&](uint32_t r, int id, int j, uint32_t m) {
         w.left(r) = 0;
         if (node_out) {
             if (a.o.exec_group) a.o.exec_group[g.n0 + id] = j;
@@ -572,13 +614,7 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                     seg = nseg++;
                     *(uint2 *)&w.rc(u) = make_uint2(x - p, 0u);
                     write_row(row, g.V + seg, id, j, p, lastz, cu, true);
-                    if constexpr (FULL_OUT)
-                        if (a.o.seg_parent) {
-                            a.o.seg_parent[g.n0 + seg] = id;
-                            a.o.seg_load[g.n0 + seg] = (int64_t)p;
-                            a.o.seg_m[g.n0 + seg] = (int32_t)mu;
-                            a.o.seg_group[g.n0 + seg] = j;
-                        }
+                    if constexpr (FULL_OUT) store(f_seg, seg, id, j, mu, p);
                     break;
                 }
                 const uint32_t ub = qu.z, ud = qu.w & 0xffffu;
@@ -645,8 +681,8 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
         } else if (n <= 32) {
             if (q.x) {
                 const int i = __popc(live & ((1u << lane) - 1)), idm = w.byrank(r);
-                write_row(nrows + i, idm, idm, j, q.x, m | (q.w & 0xffff0000u), c, nl == 0 && i == np - 1);
-                finish(r, idm, j, m);
+                write_own_row(nrows + i, idm, j, q.x, m | (q.w & 0xffff0000u), c, nl == 0 && i == np - 1);
+                finish_own(r, idm, j, m);
             }
             release_lanes();
         } else {
@@ -661,8 +697,8 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                 if (q.x) {
                     const int x = i + __popc(live & ((1u << lane) - 1)), idm = w.byrank(r);
                     const uint32_t mr = w.mm(i0 + lane);
-                    write_row(nrows + x, idm, idm, j, q.x, mr | (q.w & 0xffff0000u), q.y, nl == 0 && x == np - 1);
-                    finish(r, idm, j, mr);
+                    write_own_row(nrows + x, idm, j, q.x, mr | (q.w & 0xffff0000u), q.y, nl == 0 && x == np - 1);
+                    finish_own(r, idm, j, mr);
                 }
                 i += __popc(live);
                 release_lanes();

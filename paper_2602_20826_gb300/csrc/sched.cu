@@ -424,34 +424,10 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
         if (ids)
             for (int v = tm.t; v < V; v += NT) ws.lvl_off[v] = 0;  // levels, until they are written out
         tm.sync();
-        const int cw = (W + NWP - 1) / NWP, w0 = min(W, wp * cw), w1 = min(W, w0 + cw);  // this warp's columns
-        auto push = [&](int u, int eb, int end) {
-            for (int w = w0; w < w1; w++) {
-                const uint64_t row = ws.anc[u * W + w];
-                for (int e = eb + lane; e < end; e += 32) ws.anc[col[e] * W + w] |= row;
-            }
-        };
-        if (ids) {
-            uint16_t *lev = ws.lvl_off;
-            int end = 0, top = 0;
-            for (int u = 0; u < V; u++) {
-                const int eb = end;
-                end = (int)rp[u + 1];
-                if (wp == NWP - 1) {  // the last warp has the fewest columns
-                    const uint32_t l = lev[u] + 1u;
-                    top = max(top, (int)l);
-                    for (int e = eb + lane; e < end; e += 32) lev[col[e]] = (uint16_t)max((uint32_t)lev[col[e]], l);
-                }
-                push(u, eb, end);
-                __syncwarp();
-            }
-            if (tm.t == NT - 1) sc[1] = top;
-            tm.sync();
-            nlev = sc[1];
-            if (a.o.level)
-                for (int v = tm.t; v < V; v += NT) a.o.level[n0 + v] = lev[v];
-            for (int v = tm.t; v < V; v += NT) ws.topo[v] = (uint16_t)v;
-        } else {
+        const int cw = (W + NWP - 1) / NWP;
+        int w0 = min(W, wp * cw);  // this warp's columns, w0 .. w1 - 1
+        const int w1 = min(W, w0 + cw);
+        if (!ids) {
             if (wp == 0) {
                 int head = 0, tail = sc[0], lend = tail, L = 0;
                 for (int i = lane; i < tail; i += 32)
@@ -487,11 +463,68 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                 if (lead) write_failure(a, d, DAGRT_E_CYCLE);
                 return;
             }
+        }
+        uint16_t *lev = ws.lvl_off;
+        int top = 0;
+        // the warp's columns w0 .. w0 + CW - 1 of the closure; a step's first 32 successors are
+        // loaded a node ahead, and all its rows before any is stored
+        auto columns = [&](auto cwc, bool levels) {
+            constexpr int CW = decltype(cwc)::value;
+            int u = ids ? 0 : ws.topo[0];
+            int eb = (int)rp[u], end = (int)rp[u + 1];
+            int s0 = eb + lane < end ? col[eb + lane] : -1;
             for (int i = 0; i < V; i++) {
-                const int u = ws.topo[i];
-                push(u, (int)rp[u], (int)rp[u + 1]);
+                const int un = i + 1 < V ? (ids ? i + 1 : ws.topo[i + 1]) : u;
+                const int ebn = (int)rp[un], endn = (int)rp[un + 1];
+                const int sn = ebn + lane < endn ? col[ebn + lane] : -1;
+                const uint64_t *ru = ws.anc + u * W + w0;
+                uint64_t row[CW > 0 ? CW : 1];
+#pragma unroll
+                for (int c = 0; c < CW; c++) row[c] = ru[c];
+                const uint32_t l = levels ? lev[u] + 1u : 0u;
+                top = max(top, (int)l);
+                int s = s0;
+                for (int e = eb; e < end; e += 32) {
+                    if (e > eb) s = e + lane < end ? col[e + lane] : -1;
+                    if (s >= 0) {
+                        uint64_t *rs = ws.anc + s * W + w0;
+                        uint64_t x[CW > 0 ? CW : 1];
+#pragma unroll
+                        for (int c = 0; c < CW; c++) x[c] = rs[c];
+#pragma unroll
+                        for (int c = 0; c < CW; c++) rs[c] = x[c] | row[c];
+                        if (levels) lev[s] = (uint16_t)max((uint32_t)lev[s], l);
+                    }
+                }
                 __syncwarp();
+                u = un;
+                eb = ebn;
+                end = endn;
+                s0 = sn;
             }
+        };
+        // (every warp has cw columns but for the last ones; the last warp also pushes levels)
+        const bool levels = ids && wp == NWP - 1;
+        for (int c = w1 - w0, at = w0;; ) {
+            w0 = at;
+            const int n = min(c, 4);
+            const bool lv = levels && at + n == w1;
+            if (n == 4) columns(std::integral_constant<int, 4>(), lv);
+            else if (n == 3) columns(std::integral_constant<int, 3>(), lv);
+            else if (n == 2) columns(std::integral_constant<int, 2>(), lv);
+            else if (n == 1) columns(std::integral_constant<int, 1>(), lv);
+            else if (lv) columns(std::integral_constant<int, 0>(), true);
+            c -= n;
+            at += n;
+            if (c == 0) break;
+        }
+        if (ids) {
+            if (tm.t == NT - 1) sc[1] = top;
+            tm.sync();
+            nlev = sc[1];
+            if (a.o.level)
+                for (int v = tm.t; v < V; v += NT) a.o.level[n0 + v] = lev[v];
+            for (int v = tm.t; v < V; v += NT) ws.topo[v] = (uint16_t)v;
         }
         tm.sync();
         // ---- Eq.2: W^anc(v) = sum of C^ over v and its ancestors, by bit planes of C^
@@ -912,17 +945,15 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
         }
         work = tm.sum(work);
         tm.sync();
-        auto longest = [&](int v, uint64_t dv, int e0, int step) {
-            for (int e = rp[v] + e0; e < (int)rp[v + 1]; e += step)
-                atomicMax((unsigned long long *)&ws.cpM[ws.byrank[col[e]]], (unsigned long long)dv);
-        };
-        if constexpr (SH) {  // one warp in topological order
+        if constexpr (SH) {  // one warp in topological order: a node's successors are distinct
             for (int i = 0; tm.warp() == 0 && i < V; i++) {
                 const int v = ws.topo[i];
                 const uint64_t dv = ws.cpT[v] + ws.cpM[v];
-                __syncwarp();
                 ws.cpT[v] = dv;
-                longest(v, dv, tm.lane(), 32);
+                for (int e = (int)rp[v] + tm.lane(); e < (int)rp[v + 1]; e += 32) {
+                    const int s = ws.byrank[col[e]];
+                    if (dv > ws.cpM[s]) ws.cpM[s] = dv;
+                }
                 __syncwarp();
             }
             tm.sync();
@@ -933,7 +964,8 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                     const int v = ws.topo[i];
                     const uint64_t dv = ws.cpT[v] + ws.cpM[v];
                     ws.cpT[v] = dv;
-                    longest(v, dv, 0, 1);
+                    for (int e = rp[v]; e < (int)rp[v + 1]; e++)
+                        atomicMax((unsigned long long *)&ws.cpM[ws.byrank[col[e]]], (unsigned long long)dv);
                 }
                 tm.sync();
             }
@@ -953,8 +985,10 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
 // Warp teams for small DAGs: kWarpsPerCta teams per CTA, each with a shared-memory workspace
 // sized for (a.vcap, a.ecap), the largest V and E of the launch's size class.
 // Five CTAs an SM (96 registers): at four (128) the 10,000-DAG batch is latency-bound on 16 warps.
+// The variants with every output keep four: at 96 registers they spill (1,000 DAGs of 50-500 nodes
+// with the plan written out: 1.27 ms at four, 1.35 ms at five).
 template <bool FULL_OUT>
-__global__ void __launch_bounds__(32 * kWarpsPerCta, 5) k_sched_warp(SchedArgs a) {
+__global__ void __launch_bounds__(32 * kWarpsPerCta, FULL_OUT ? 4 : 5) k_sched_warp(SchedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const WarpWs ws = warp_carve(a.vcap, a.ecap);
