@@ -72,13 +72,23 @@ struct dagrt_ctx {
     int64_t capture_launch0 = 0;
     cudaStream_t cap_stream = nullptr;  // captures run here; `stream` is restored at the end
     cudaStream_t saved_stream = nullptr;
-    // pinned host staging of dagrt_load_csr (offsets down, class lists up); pin_ev marks the
-    // end of the last asynchronous copy out of it, waited for before the next reuse
+    // pinned host staging of dagrt_load_csr (offsets down; class lists and small host arrays
+    // up); pin_ev marks the end of the last asynchronous copy out of it, waited for before the
+    // next reuse
     void *pin = nullptr;
     size_t pin_cap = 0;
     cudaEvent_t pin_ev = nullptr;
     bool pin_pending = false;
+    void *pin_out = nullptr;  // kPinOut bytes of pinned memory: small host outputs of dagrt_schedule
 };
+
+// Small host arrays travel together. A copy from or to pageable memory costs the host 6-8 us
+// whatever its size, so arrays of up to kPinArray bytes go up in one copy out of the pinned
+// staging buffer (from there on the caller's arrays are free, without a synchronisation), and
+// outputs of up to kPinOut bytes altogether are written by the kernels straight to pinned host
+// memory. Loading, scheduling and freeing one DAG of 20 nodes takes 57 us, with a copy per array
+// (and a side stream for its only size class) it was 100.
+constexpr size_t kPinArray = 64 << 10, kPinOut = 256 << 10;
 
 // The context's pinned staging buffer, at least `bytes` long, once its last asynchronous
 // copy has completed.
@@ -269,6 +279,11 @@ int dagrt_create(dagrt_ctx **out, int device, void *cuda_stream) {
 int dagrt_set_stream(dagrt_ctx *ctx, void *cuda_stream) {
     if (!ctx) return DAGRT_E_INVAL;
     if (ctx->capturing) return fail(ctx, DAGRT_E_INVAL, "dagrt_set_stream: not allowed while capturing a graph");
+    if (ctx->pin_pending && (cudaStream_t)cuda_stream != ctx->stream) {  // a batch may be on its way on the old stream
+        CK(cudaSetDevice(ctx->device), "cudaSetDevice");
+        CK(cudaEventSynchronize(ctx->pin_ev), "synchronize");
+        ctx->pin_pending = false;
+    }
     ctx->stream = (cudaStream_t)cuda_stream;
     return DAGRT_OK;
 }
@@ -294,6 +309,7 @@ static void ctx_release(dagrt_ctx *ctx) {
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->pin_ev) cudaEventDestroy(ctx->pin_ev);
     if (ctx->pin) cudaFreeHost(ctx->pin);
+    if (ctx->pin_out) cudaFreeHost(ctx->pin_out);
     delete ctx;
 }
 
@@ -334,8 +350,9 @@ void dagrt_batch_free(dagrt_batch *b) {
 // nodes; the rest go to CTA teams -- with a shared-memory workspace while a class's
 // capacity (largest V and E so far, smallest DAGs first) still fits 1/tune.cta_smem of a
 // CTA's shared memory, or all of it (cta_smem = 0: never), else with global workspaces. Each class is ordered by
-// descending node count (longest work first). Host work plus one list upload.
-static int partition_classes(dagrt_batch *b) {
+// descending node count (longest work first). Host work: the lists go to lists[n_dags], which
+// the caller uploads.
+static int partition_classes(dagrt_batch *b, int32_t *lists) {
     dagrt_ctx *ctx = b->ctx;
     const int n_dags = b->n_dags, max_v = b->max_v;
     const std::vector<int64_t> &hn = b->h_node_off, &he = b->h_edge_off;
@@ -386,7 +403,7 @@ static int partition_classes(dagrt_batch *b) {
         big_cls[i] = c;
         count[c]++;
     }
-    // the class lists, each in descending V (equal V: ascending DAG id), in pinned memory
+    // the class lists, each in descending V (equal V: ascending DAG id)
     int off = 0, pos[kNumClasses];
     for (int c = 0; c < kNumClasses; c++) {
         b->class_off[c] = pos[c] = off;
@@ -401,8 +418,6 @@ static int partition_classes(dagrt_batch *b) {
             p += cnt_v[v];
         }
     }
-    int32_t *lists = nullptr;
-    CK(pinned(ctx, 4 * (size_t)std::max(n_dags, 1), (void **)&lists), "pinned staging");
     for (int d = 0; d < n_dags; d++) {
         const int v = (int)(hn[d + 1] - hn[d]);
         if (v <= wmax && he[d + 1] - he[d] <= (int64_t)kEdgesPerNode * wmax) lists[start_v[v]++] = d;
@@ -418,11 +433,6 @@ static int partition_classes(dagrt_batch *b) {
     }
     b->big_vcap = gv;
     b->big_ecap = (int)ge;
-    if (n_dags > 0) {
-        CK(cudaMemcpyAsync(b->lists, lists, 4 * n_dags, cudaMemcpyHostToDevice, ctx->stream), "copy class lists");
-        CK(cudaEventRecord(ctx->pin_ev, ctx->stream), "record staging event");
-        ctx->pin_pending = true;
-    }
     const int n_big = b->class_off[kClsCtaGlobal + 1] - b->class_off[kClsCtaGlobal];
     if (n_big > 0) {
         b->big_grid = std::min(sched_cta_grid(ctx->n_sm), n_big);
@@ -496,46 +506,60 @@ int dagrt_load_csr(dagrt_ctx *ctx, int32_t n_dags, const int64_t *node_off, cons
         delete b;
         return code;
     };
-    cudaError_t e;
-    if (dev) {
-        b->node_off = node_off;
-        b->edge_off = edge_off;
-        b->row_ptr = row_ptr;
-        b->col = col;
-        b->wcet = wcet;
-        b->k64 = k64;
-    } else {
-        int64_t *dn, *de, *dw;
-        int32_t *dr, *dc;
-        uint8_t *dk;
-        if ((e = batch_alloc(b, &dn, n_dags + 1)) != cudaSuccess || (e = batch_alloc(b, &de, n_dags + 1)) != cudaSuccess ||
-            (e = batch_alloc(b, &dr, tn + n_dags)) != cudaSuccess || (e = batch_alloc(b, &dc, te)) != cudaSuccess ||
-            (e = batch_alloc(b, &dw, tn)) != cudaSuccess || (e = batch_alloc(b, &dk, tn)) != cudaSuccess)
-            return bail(cuda_fail(ctx, e, "allocate batch copy"));
-        cudaStream_t st = ctx->stream;
-        if ((e = cudaMemcpyAsync(dn, node_off, 8 * (n_dags + 1), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(de, edge_off, 8 * (n_dags + 1), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(dr, row_ptr, 4 * (tn + n_dags), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (te > 0 && (e = cudaMemcpyAsync(dc, col, 4 * te, cudaMemcpyHostToDevice, st)) != cudaSuccess) ||
-            (e = cudaMemcpyAsync(dw, wcet, 8 * tn, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(dk, k64, tn, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-            return bail(cuda_fail(ctx, e, "copy batch to device"));
-        b->node_off = dn;
-        b->edge_off = de;
-        b->row_ptr = dr;
-        b->col = dc;
-        b->wcet = dw;
-        b->k64 = dk;
-    }
-
     b->h_edge_off = std::move(he);
-    if ((e = batch_alloc(b, &b->lists, n_dags)) != cudaSuccess ||
-        (e = batch_alloc(b, &b->counters, kNumClasses)) != cudaSuccess || (e = batch_alloc(b, &b->err, 1)) != cudaSuccess ||
-        (e = cudaMemsetAsync(b->err, 0, sizeof(int32_t), ctx->stream)) != cudaSuccess)
-        return bail(cuda_fail(ctx, e, "allocate class lists"));
-    if (int rc = partition_classes(b)) return bail(rc);
-    // host copies must be complete before the caller may reuse its buffers
-    if (!dev && (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return bail(cuda_fail(ctx, e, "synchronize"));
+    // One device block, filled by one copy from the pinned staging buffer: the class lists, the
+    // counters and the error word (zero), and the host arrays of up to kPinArray bytes.
+    struct Array {
+        const void *src;
+        size_t bytes;
+        const void **slot;
+    };
+    const Array arrays[] = {
+        {node_off, 8 * ((size_t)n_dags + 1), (const void **)&b->node_off},
+        {edge_off, 8 * ((size_t)n_dags + 1), (const void **)&b->edge_off},
+        {row_ptr, 4 * (size_t)(tn + n_dags), (const void **)&b->row_ptr},
+        {col, 4 * (size_t)te, (const void **)&b->col},
+        {wcet, 8 * (size_t)tn, (const void **)&b->wcet},
+        {k64, (size_t)tn, (const void **)&b->k64},
+    };
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t o_cnt = up(4 * (size_t)n_dags), o_err = o_cnt + up(kNumClasses * sizeof(int32_t));
+    size_t block_bytes = o_err + 256;
+    for (const Array &x : arrays)
+        if (!dev && x.bytes <= kPinArray) block_bytes += up(x.bytes);
+    unsigned char *block = nullptr, *pin = nullptr;
+    cudaError_t e = batch_alloc(b, &block, block_bytes);
+    if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "allocate batch"));
+    if ((e = pinned(ctx, block_bytes, (void **)&pin)) != cudaSuccess) return bail(cuda_fail(ctx, e, "pinned staging"));
+    b->lists = (int32_t *)block;
+    b->counters = (int32_t *)(block + o_cnt);
+    b->err = (int32_t *)(block + o_err);
+    std::memset(pin + o_cnt, 0, o_err + 256 - o_cnt);
+    bool direct = false;  // some array is copied from the caller's memory
+    size_t at = o_err + 256;
+    for (const Array &x : arrays) {
+        if (dev) {
+            *x.slot = x.src;
+        } else if (x.bytes <= kPinArray) {
+            if (x.bytes > 0) std::memcpy(pin + at, x.src, x.bytes);
+            *x.slot = block + at;
+            at += up(x.bytes);
+        } else {
+            unsigned char *q = nullptr;
+            if ((e = batch_alloc(b, &q, x.bytes)) != cudaSuccess) return bail(cuda_fail(ctx, e, "allocate batch copy"));
+            if ((e = cudaMemcpyAsync(q, x.src, x.bytes, cudaMemcpyHostToDevice, ctx->stream)) != cudaSuccess)
+                return bail(cuda_fail(ctx, e, "copy batch to device"));
+            *x.slot = q;
+            direct = true;
+        }
+    }
+    if (int rc = partition_classes(b, (int32_t *)pin)) return bail(rc);
+    if ((e = cudaMemcpyAsync(block, pin, block_bytes, cudaMemcpyHostToDevice, ctx->stream)) != cudaSuccess ||
+        (e = cudaEventRecord(ctx->pin_ev, ctx->stream)) != cudaSuccess)
+        return bail(cuda_fail(ctx, e, "copy batch to device"));
+    ctx->pin_pending = true;
+    // copies of the caller's arrays must be complete before it may reuse them
+    if (direct && (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return bail(cuda_fail(ctx, e, "synchronize"));
     ctx->n_batches++;
     ctx->live++;
     *out = b;
@@ -685,17 +709,30 @@ extern "C" int dagrt_schedule(dagrt_batch *b, int32_t variant, const dagrt_sched
     if ((o.seg_parent || o.seg_load || o.seg_m || o.seg_group) &&
         !(o.seg_parent && o.seg_load && o.seg_m && o.seg_group))
         return fail(ctx, DAGRT_E_INVAL, "dagrt_schedule: segment outputs go together");
-    if (!dev) {  // stage every requested host output through one device scratch block
+    bool mapped = false;  // the kernels write the outputs to pinned host memory
+    const int32_t *h_status = nullptr;
+    if (!dev) {  // every requested host output in one block: of pinned memory if small, else of device scratch
+        auto up = [](size_t x) { return (x + 255) / 256 * 256; };
         size_t total = 0;
         for (auto &f : fields)
-            if (f.user) total += (f.bytes + 255) / 256 * 256;
-        rc = ensure_tmp(b, total > 0 ? total : 256);
-        if (rc) return rc;
+            if (f.user) total += up(f.bytes);
+        mapped = !o.extra_off && total + up(4 * nd) <= kPinOut;
+        if (mapped) {
+            if (!ctx->pin_out) CK(cudaHostAlloc(&ctx->pin_out, kPinOut, cudaHostAllocDefault), "pinned outputs");
+        } else {
+            rc = ensure_tmp(b, total > 0 ? total : 256);
+            if (rc) return rc;
+        }
+        char *block = (char *)(mapped ? ctx->pin_out : b->tmp);
         size_t off = 0;
         for (auto &f : fields) {
             if (!f.user) continue;
-            *f.slot = (char *)b->tmp + off;
-            off += (f.bytes + 255) / 256 * 256;
+            *f.slot = block + off;
+            off += up(f.bytes);
+        }
+        if (mapped) {
+            if (!o.status) dv.status = (int32_t *)(block + off);
+            h_status = dv.status;
         }
         if (o.extra_off)
             CK(cudaMemcpyAsync(dv.extra_off, o.extra_off, 8 * (nd + 1), cudaMemcpyHostToDevice, ctx->stream),
@@ -722,22 +759,36 @@ extern "C" int dagrt_schedule(dagrt_batch *b, int32_t variant, const dagrt_sched
     a.plan = p.rows;
     a.o = dv;
     if (nd > 0) {
-        CK(cudaMemsetAsync(b->counters, 0, kNumClasses * sizeof(int32_t), ctx->stream), "reset counters");
-        CK(ensure_side_streams(ctx), "create side streams");
+        int n_classes = 0;
+        int64_t ctas = 0;  // that take one DAG per team
+        for (int c = 0; c < kNumClasses; c++) {
+            const int n = b->class_off[c + 1] - b->class_off[c];
+            n_classes += n > 0;
+            ctas += c < kNumWarpClasses ? (n + kWarpsPerCta - 1) / kWarpsPerCta : n;
+        }
+        // with an SM for every CTA there is nothing to steal: team i takes the list's DAG i, and
+        // the counters stay out of it (a memset and an atomic less in the chain of a small call)
+        const bool steal = ctas > ctx->n_sm;
+        if (steal) CK(cudaMemsetAsync(b->counters, 0, kNumClasses * sizeof(int32_t), ctx->stream), "reset counters");
         // size classes run concurrently: fork from the context stream, join back into it.
         // Largest class first, so that the longest DAGs start at once and the short ones
         // fill in around them (with classes of 16 nodes and four teams per CTA this measured
-        // 1-4% faster than smallest first on the 10,000-DAG batch)
-        CK(cudaEventRecord(ctx->fork, ctx->stream), "record fork");
+        // 1-4% faster than smallest first on the 10,000-DAG batch). A single class runs on the
+        // context stream itself.
+        const bool side = n_classes > 1;
+        if (side) {
+            CK(ensure_side_streams(ctx), "create side streams");
+            CK(cudaEventRecord(ctx->fork, ctx->stream), "record fork");
+        }
         int used[dagrt_ctx::kSide], nused = 0;
         for (int c = kNumClasses - 1; c >= 0; c--) {
             const int n = b->class_off[c + 1] - b->class_off[c];
             if (n == 0) continue;
-            cudaStream_t st = ctx->side[c];
-            CK(cudaStreamWaitEvent(st, ctx->fork, 0), "fork");
+            cudaStream_t st = side ? ctx->side[c] : ctx->stream;
+            if (side) CK(cudaStreamWaitEvent(st, ctx->fork, 0), "fork");
             a.list = b->lists + b->class_off[c];
             a.n_list = n;
-            a.counter = b->counters + c;
+            a.counter = steal ? b->counters + c : nullptr;
             if (c < kNumWarpClasses) {
                 a.vcap = b->wcap_v[c];
                 a.ecap = b->wcap_e[c];
@@ -754,6 +805,7 @@ extern "C" int dagrt_schedule(dagrt_batch *b, int32_t variant, const dagrt_sched
                 CK(sched_launch_cta(a, b->big_grid, st), "launch scheduler (CTA teams)");
             }
             ctx->launches++;
+            if (!side) continue;
             CK(cudaEventRecord(ctx->join[c], st), "record join");
             used[nused++] = c;
         }
@@ -763,16 +815,23 @@ extern "C" int dagrt_schedule(dagrt_batch *b, int32_t variant, const dagrt_sched
     p.chunked = false;
     if (dev) return DAGRT_OK;
 
-    for (auto &f : fields) {
-        if (!f.user || f.user == (void *)o.extra_off) continue;
-        if (f.bytes) CK(cudaMemcpyAsync(f.user, *f.slot, f.bytes, cudaMemcpyDeviceToHost, ctx->stream), "copy output");
+    std::vector<int32_t> st;
+    if (!mapped) {
+        for (auto &f : fields) {
+            if (!f.user || f.user == (void *)o.extra_off) continue;
+            if (f.bytes) CK(cudaMemcpyAsync(f.user, *f.slot, f.bytes, cudaMemcpyDeviceToHost, ctx->stream), "copy output");
+        }
+        st.resize(nd);
+        if (nd) CK(cudaMemcpyAsync(st.data(), p.status, 4 * nd, cudaMemcpyDeviceToHost, ctx->stream), "copy status");
+        h_status = st.data();
     }
-    std::vector<int32_t> st(nd);
-    if (nd) CK(cudaMemcpyAsync(st.data(), p.status, 4 * nd, cudaMemcpyDeviceToHost, ctx->stream), "copy status");
     CK(cudaStreamSynchronize(ctx->stream), "synchronize");
+    if (mapped)
+        for (auto &f : fields)
+            if (f.user && f.bytes) std::memcpy(f.user, *f.slot, f.bytes);
     for (size_t d = 0; d < nd; d++)
-        if (st[d] != DAGRT_OK)
-            return fail(ctx, st[d], "dagrt_schedule: DAG %zu failed with status %d", d, st[d]);
+        if (h_status[d] != DAGRT_OK)
+            return fail(ctx, h_status[d], "dagrt_schedule: DAG %zu failed with status %d", d, h_status[d]);
     return DAGRT_OK;
 }
 
@@ -1421,7 +1480,12 @@ extern "C" int dagrt_set_tuning(dagrt_batch *b, const dagrt_tuning *t) {
     b->tune = *t;
     if (repart) {
         CK(cudaStreamSynchronize(ctx->stream), "synchronize");  // the lists may be in use
-        return partition_classes(b);
+        std::vector<int32_t> lists(b->n_dags);
+        if (int rc = partition_classes(b, lists.data())) return rc;
+        if (b->n_dags > 0) {
+            CK(cudaMemcpyAsync(b->lists, lists.data(), 4 * lists.size(), cudaMemcpyHostToDevice, ctx->stream), "copy class lists");
+            CK(cudaStreamSynchronize(ctx->stream), "synchronize");
+        }
     }
     return DAGRT_OK;
 }

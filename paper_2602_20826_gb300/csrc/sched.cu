@@ -993,12 +993,14 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta, FULL_OUT ? 4 : 5) k_sched_w
     const int lane = threadIdx.x & 31;
     const WarpWs ws = warp_carve(a.vcap, a.ecap);
     const uint32_t base = (threadIdx.x >> 5) * ws.bytes;
-    for (;;) {
-        int idx = 0;
-        if (lane == 0) idx = atomicAdd(a.counter, 1);
-        idx = __shfl_sync(FULL, idx, 0);
+    for (int idx = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);;) {
+        if (a.counter) {
+            if (lane == 0) idx = atomicAdd(a.counter, 1);
+            idx = __shfl_sync(FULL, idx, 0);
+        }
         if (idx >= a.n_list) break;
         schedule_warp<FULL_OUT>(ws, base, a, a.list[idx], lane);
+        if (!a.counter) break;
         __syncwarp();
     }
 }
@@ -1018,12 +1020,13 @@ __global__ void __launch_bounds__(NT, SMEM ? 512 / NT : 1) k_sched_cta(SchedArgs
     }
     Team<NT> tm{(int)threadIdx.x, red};
     for (;;) {
-        if (threadIdx.x == 0) idx_s = atomicAdd(a.counter, 1);
+        if (threadIdx.x == 0) idx_s = a.counter ? atomicAdd(a.counter, 1) : (int)blockIdx.x;
         __syncthreads();
         const int idx = idx_s;
         __syncthreads();
         if (idx >= a.n_list) break;
         schedule_one<NT, SMEM, FULL_OUT>(tm, ws, a, a.list ? a.list[idx] : idx, a.vcap, a.ecap);
+        if (!a.counter) break;
         __syncthreads();
     }
 }

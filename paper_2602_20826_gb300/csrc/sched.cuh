@@ -26,7 +26,7 @@ struct SchedArgs {
     int32_t M;
     int32_t variant;
     // DAGs of this size class (NULL: DAGs 0 .. n_list-1 in order) and the work-stealing
-    // counter over them
+    // counter over them (NULL: the grid covers the list, team i takes its DAG i)
     const int32_t *list;
     int32_t n_list;
     int32_t *counter;
