@@ -128,19 +128,68 @@ __device__ void team_scan_inplace(const Team<NT> &tm, T *arr, int n, Op op, bool
     }
 }
 
-// Bitonic sort of keys[0..P) ascending, P a power of two.
+// Bitonic network, strides j, j / 2, ..., jmin of the merge of runs of k, over keys[0..n) (n a
+// power of two), which are the keys from `base` on of the sequence that is sorted. Two strides a
+// pass: a thread takes four keys through both.
 template <int NT>
-__device__ void team_bitonic_sort(const Team<NT> &tm, uint64_t *keys, int P) {
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tm.t; i < P; i += NT) {
-                int l = i ^ j;
-                if (l > i) {
-                    uint64_t a = keys[i], b = keys[l];
-                    bool up = (i & k) == 0;
-                    if (up ? (a > b) : (a < b)) { keys[i] = b; keys[l] = a; }
-                }
+__device__ __forceinline__ void team_bitonic_merge(const Team<NT> &tm, uint64_t *keys, int n, int base, int k, int j, int jmin) {
+    auto order = [](uint64_t &x, uint64_t &y, bool up) {
+        const uint64_t lo = x < y ? x : y, hi = x < y ? y : x;
+        x = up ? lo : hi;
+        y = up ? hi : lo;
+    };
+    while (j >= jmin) {
+        const int h = j >> 1;
+        if (h >= jmin) {
+            for (int t = tm.t; t < n >> 2; t += NT) {
+                const int i = (t & ~(h - 1)) << 2 | (t & (h - 1));
+                const bool up = ((base + i) & k) == 0;
+                uint64_t x0 = keys[i], x1 = keys[i + h], x2 = keys[i + 2 * h], x3 = keys[i + 3 * h];
+                order(x0, x2, up);
+                order(x1, x3, up);
+                order(x0, x1, up);
+                order(x2, x3, up);
+                keys[i] = x0;
+                keys[i + h] = x1;
+                keys[i + 2 * h] = x2;
+                keys[i + 3 * h] = x3;
             }
+            j >>= 2;
+        } else {
+            for (int t = tm.t; t < n >> 1; t += NT) {
+                const int i = (t & ~(j - 1)) << 1 | (t & (j - 1));
+                uint64_t x0 = keys[i], x1 = keys[i + j];
+                order(x0, x1, ((base + i) & k) == 0);
+                keys[i] = x0;
+                keys[i + j] = x1;
+            }
+            j >>= 1;
+        }
+        tm.sync();
+    }
+}
+
+// Sorts keys[0..P) ascending, P a power of two. `buf`: shared memory for C keys (C a power of
+// two; 0: the keys are in shared memory themselves), which takes every stride below C: what
+// bounds the sort is the barrier and the latency of a pass, so passes over global memory are
+// the few strides of C and above (32,768 keys by 384 threads: @@).
+template <int NT>
+__device__ void team_bitonic_sort(const Team<NT> &tm, uint64_t *keys, int P, uint64_t *buf = nullptr, int C = 0) {
+    if (C == 0) {
+        for (int k = 2; k <= P; k <<= 1) team_bitonic_merge(tm, keys, P, 0, k, k >> 1, 1);
+        return;
+    }
+    C = min(C, P);
+    for (int k0 = C; k0 <= P; k0 <<= 1) {
+        if (k0 > C) team_bitonic_merge(tm, keys, P, 0, k0, k0 >> 1, C);
+        for (int b = 0; b < P; b += C) {
+            for (int i = tm.t; i < C; i += NT) buf[i] = keys[b + i];
+            tm.sync();
+            if (k0 == C)
+                for (int k = 2; k <= C; k <<= 1) team_bitonic_merge(tm, buf, C, b, k, k >> 1, 1);
+            else
+                team_bitonic_merge(tm, buf, C, b, k0, C >> 1, 1);
+            for (int i = tm.t; i < C; i += NT) keys[b + i] = buf[i];
             tm.sync();
         }
     }

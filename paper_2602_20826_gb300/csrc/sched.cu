@@ -623,7 +623,9 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
 
     // ---- ... then the ancestor closure and Eq.2 level by level, a warp per node: the rows of
     //      the predecessors and the predecessors themselves, 64-bit words over the lanes, and
-    //      the row's share of W^anc by bit planes of C^ (in shared memory while they fit)
+    //      W^anc as one predecessor's plus the loads of the ancestors that only others have, by
+    //      bit planes of C^ (in shared memory while they fit). Most words add nothing: counting
+    //      the bits of every word was two thirds of this phase (20,000 nodes: @@).
     uint64_t *planes = nb * W <= kPlaneWords ? (uint64_t *)(dyn + kRelBytes) : ws.planes;
     for (int i = tm.t; i < nb * W; i += NT) {
         const int b = i / W, w = i - b * W;
@@ -643,43 +645,91 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     tm.sync();
     for (int l = 0; l < nlev; l++) {
         const int lb = ws.lvl_off[l], lend = (l + 1 < nlev) ? ws.lvl_off[l + 1] : V;
-        for (int i = lb + tm.warp(); i < lend; i += NT / 32) {
-            const int v = ws.topo[i];
-            const int pe = ws.poff[v], pb = pe - ws.indeg[v];
-            uint64_t acc = 0;
-            for (int c = 0; c < W; c += 4 * 32) {  // four words per lane in flight
-                uint64_t x[4] = {0, 0, 0, 0};
-                for (int k = pb; k < pe; k++) {
-                    const int p = ws.pid[k];
-                    const uint64_t *row = ws.anc + (int64_t)p * W;
+        const int ln = tm.lane(), stride = NT / 32;
+        for (int i0 = lb + tm.warp(); i0 < lend; i0 += 32 * stride) {
+            // the warp's next 32 nodes, one per lane; their predecessor lists are fetched two
+            // nodes ahead and the predecessors' W^anc one node ahead
+            const int mine = i0 + ln * stride, nq = min(32, (lend - i0 + stride - 1) / stride);
+            const int vq = mine < lend ? ws.topo[mine] : 0;
+            const int peq = mine < lend ? ws.poff[vq] : 0, npq = mine < lend ? ws.indeg[vq] : 0;
+            auto preds = [&](int q) {  // the q-th node's first 32 predecessors, one per lane
+                const int n = __shfl_sync(FULL, npq, q), b = __shfl_sync(FULL, peq, q) - n;
+                return q < nq && ln < n ? (int)ws.pid[b + ln] : -1;
+            };
+            auto weight = [&](int p) { return p >= 0 ? ws.wanc[p] : 0ull; };
+            int p0 = preds(0), p1 = preds(1);
+            uint64_t w0 = weight(p0);
+            for (int q = 0; q < nq; q++) {
+                const int v = __shfl_sync(FULL, vq, q), np = __shfl_sync(FULL, npq, q);
+                const int pb = __shfl_sync(FULL, peq, q) - np;
+                const int p2 = preds(min(q + 2, 31));
+                const uint64_t w1 = weight(p1);
+                // the predecessor of largest W^anc (about: any would do) and two others
+                const uint32_t key = p0 >= 0 ? __float_as_uint((float)w0) : 0u;
+                const int kb = __ffs(__ballot_sync(FULL, key == __reduce_max_sync(FULL, key))) - 1;
+                uint32_t rest = (np < 32 ? (1u << np) - 1u : FULL) & ~(1u << kb);
+                const int pa = __shfl_sync(FULL, p0, kb);
+                const int pc = __shfl_sync(FULL, p0, (__ffs(rest) - 1) & 31);
+                rest &= rest - 1;
+                const int pd = __shfl_sync(FULL, p0, (__ffs(rest) - 1) & 31);
+                rest &= rest - 1;
+                uint64_t acc = 0;
+                for (int c = 0; c < W; c += 4 * 32) {  // four words of three rows per lane in flight
+                    uint64_t x0[4] = {0, 0, 0, 0}, x[4] = {0, 0, 0, 0}, y[4] = {0, 0, 0, 0};
+                    auto load = [&](uint64_t(&r)[4], int p) {
+                        const uint64_t *row = ws.anc + (int64_t)p * W;
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            if (c + 32 * j + ln < W) r[j] = row[c + 32 * j + ln];
+                    };
+                    auto self = [&](uint64_t(&r)[4], int p) {
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            if (c + 32 * j + ln == p >> 6) r[j] |= 1ull << (p & 63);
+                    };
+                    if (np > 0) load(x0, pa);
+                    if (np > 1) load(x, pc);
+                    if (np > 2) load(y, pd);
+                    if (np > 0) self(x0, pa);
+                    if (np > 1) self(x, pc);
+                    if (np > 2) self(y, pd);
+                    uint32_t more = rest;
+                    for (int k = 3; k < np; k++) {
+                        const int l = (__ffs(more) - 1) & 31;
+                        const int p = k < 32 ? __shfl_sync(FULL, p0, l) : (int)ws.pid[pb + k];
+                        more &= more - 1;
+                        uint64_t z[4] = {0, 0, 0, 0};
+                        load(z, p);
+                        self(z, p);
+#pragma unroll
+                        for (int j = 0; j < 4; j++) x[j] |= z[j];
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
-                        const int w = c + 32 * j + tm.lane();
-                        if (w < W) x[j] |= row[w];
-                        if (w == p >> 6) x[j] |= 1ull << (p & 63);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const int w = c + 32 * j + tm.lane();
-                    if (w >= W) break;
-                    ws.anc[(int64_t)v * W + w] = x[j];
-                    if (x[j]) {
-                        if (nb <= 24) {  // 64 * 2^24 fits: the word's sum in 32 bits
-                            uint32_t s = 0;
-                            for (int b = 0; b < nb; b++) s += (uint32_t)__popcll(x[j] & planes[b * W + w]) << b;
-                            acc += s;
-                        } else {
-                            for (int b = 0; b < nb; b++) acc += (uint64_t)__popcll(x[j] & planes[b * W + w]) << b;
+                        const int w = c + 32 * j + ln;
+                        x[j] |= y[j];
+                        if (w < W) ws.anc[(int64_t)v * W + w] = x0[j] | x[j];
+                        const uint64_t add = x[j] & ~x0[j];  // zero beyond W
+                        if (add) {
+                            if (nb <= 24) {  // 64 * 2^24 fits: the word's sum in 32 bits
+                                uint32_t t = 0;
+                                for (int b = 0; b < nb; b++) t += (uint32_t)__popcll(add & planes[b * W + w]) << b;
+                                acc += t;
+                            } else {
+                                for (int b = 0; b < nb; b++) acc += (uint64_t)__popcll(add & planes[b * W + w]) << b;
+                            }
                         }
                     }
                 }
-            }
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-            acc += ws.load[v];
-            if (tm.lane() == 0) {
-                ws.wanc[v] = acc;
-                if (a.o.wanc) a.o.wanc[n0 + v] = (int64_t)acc;
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+                acc += ws.load[v] + __shfl_sync(FULL, w0, kb);  // (no predecessor: 0)
+                if (ln == 0) {
+                    ws.wanc[v] = acc;
+                    if (a.o.wanc) a.o.wanc[n0 + v] = (int64_t)acc;
+                }
+                p0 = p1;
+                p1 = p2;
+                w0 = w1;
             }
         }
         tm.sync();
@@ -693,7 +743,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     uint64_t *skey = ws.wanc;  // the keys take the weights' place
     for (int i = tm.t; i < P; i += NT) skey[i] = i < V ? ((ws.wanc[i] << 16) | (uint64_t)i) : KEY_INF;
     tm.sync();
-    team_bitonic_sort(tm, skey, P);
+    team_bitonic_sort(tm, skey, P, SH ? nullptr : (uint64_t *)(dyn + kRelBytes), SH ? 0 : kPlaneWords);
     // per sorted position: join flag (-> Theta index), start and end of its W^anc run
     for (int i = tm.t; i < V; i += NT) {
         const int v = (int)(skey[i] & 0xffff);
