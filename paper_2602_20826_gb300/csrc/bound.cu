@@ -697,15 +697,8 @@ size_t bound_chunk_scratch(int32_t n_dags, int64_t total_nodes, int32_t n_varian
     return 256 + (size_t)n_dags * n_variants * n_alloc * 8;
 }
 
-// Programmatic dependent launch: the work-item kernel lets k_bound_finish start early;
-// k_bound_finish reads what earlier kernels wrote, then waits for the work items to
-// complete (and their stores to be visible) before it touches their partial sums.
-__device__ __forceinline__ void griddep_launch_dependents() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// After the work items, one warp per DAG: the items have added their partial bounds into
+// After the work items (programmatic launch: they let this kernel start early, and it waits for
+// them before it touches their partial sums), one warp per DAG: the items have added their partial bounds into
 // the DAG's per-candidate accumulators; lane l reads candidates 2l and 2l + 1 of four
 // 64-candidate blocks at a time, writes the bounds (-1 for a variant whose schedule
 // failed), clears the accumulators for the next call and takes the argmin by shuffles. The

@@ -195,6 +195,15 @@ __device__ void team_bitonic_sort(const Team<NT> &tm, uint64_t *keys, int P, uin
     }
 }
 
+// ------------------------------------------------------------------ programmatic launches
+// A kernel launched with programmatic stream serialization starts once every CTA of the kernel
+// before it has called the first of these or ended; the second waits until that kernel has
+// completed and its stores are visible. Both do nothing in an ordinary launch.
+__device__ __forceinline__ void griddep_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ Eq.1
 // Execution time of a kernel with load x (ticks on one SM) and parallel fraction k/64 on m
 // of M SMs: max(1, ceil(ceil(m/M) * x * (64m - k(m-1)) / (64m))). Products stay below

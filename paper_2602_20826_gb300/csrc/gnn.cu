@@ -310,21 +310,40 @@ __device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const
 // 165,000 nodes, 2.8 M edges, 128 features: 116 us, and the product 52, where one kernel for
 // both took 190 (the rows of a CTA's nodes from a chunk next to its SM's other CTAs: 127, the
 // chunks' degrees then differ by SM); 16 features: 97 -> 31 and 24.
+//
+// SMALL (no SM has a second tile of the product): latency is what counts, so a warp takes the
+// predecessors or the successors of its nodes, a CTA one pass of them, and the layer's kernels
+// start early (programmatic launches): three layers and the head on 9,000 nodes of degree 55 took
+// 85 us in the other form, 58 in this. With all nodes of a large batch the two
+// kinds of lists apart cost the L1 cache more than they gain: 447 -> 473 us for the whole
+// network on 165,000 nodes.
 constexpr int kAggThreads = 512;
-template <int KIN>
+template <int KIN, bool SMALL>
 __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *__restrict__ h,
                                                          uint16_t *__restrict__ agg) {
-    constexpr int LPN = KIN / 8, NODES = kAggThreads / LPN;  // lanes per node, nodes per CTA pass
-    const int sub = threadIdx.x % LPN;
-    constexpr int CHUNK = NODES < 128 ? 128 : NODES;         // neighbouring nodes that a CTA takes together
-    for (int64_t c0 = (int64_t)blockIdx.x * CHUNK; c0 < g.n_nodes; c0 += (int64_t)gridDim.x * CHUNK)
-        for (int i = 0; i < CHUNK / NODES; i++) {
-            const int64_t v = c0 + i * NODES + threadIdx.x / LPN;
-            if (v >= g.n_nodes) break;
-            uint4 *dst = (uint4 *)(agg + v * 2 * KIN);
-            dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred_off[v], g.pred_off[v + 1], sub);
-            dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ_off[v], g.succ_off[v + 1], sub);
-        }
+    constexpr int LPN = KIN / 8;  // lanes per node
+    if constexpr (SMALL) {
+        griddep_wait();
+        griddep_launch_dependents();
+        constexpr int NODES = kAggThreads / 2 / LPN;
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % LPN, succ = w & 1;
+        const int32_t *off = succ ? g.succ_off : g.pred_off, *idx = succ ? g.succ_idx : g.pred_idx;
+        for (int64_t v = (int64_t)blockIdx.x * NODES + (w >> 1) * (32 / LPN) + lane / LPN; v < g.n_nodes;
+             v += (int64_t)gridDim.x * NODES)
+            ((uint4 *)(agg + v * 2 * KIN))[succ * LPN + sub] = mean_rows<KIN>(h, idx, off[v], off[v + 1], sub);
+    } else {
+        constexpr int NODES = kAggThreads / LPN;          // nodes per CTA pass
+        constexpr int CHUNK = NODES < 128 ? 128 : NODES;  // neighbouring nodes that a CTA takes together
+        const int sub = threadIdx.x % LPN;
+        for (int64_t c0 = (int64_t)blockIdx.x * CHUNK; c0 < g.n_nodes; c0 += (int64_t)gridDim.x * CHUNK)
+            for (int i = 0; i < CHUNK / NODES; i++) {
+                const int64_t v = c0 + i * NODES + threadIdx.x / LPN;
+                if (v >= g.n_nodes) break;
+                uint4 *dst = (uint4 *)(agg + v * 2 * KIN);
+                dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred_off[v], g.pred_off[v + 1], sub);
+                dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ_off[v], g.succ_off[v + 1], sub);
+            }
+    }
 }
 
 // 16-byte piece i of warp w's share of a [128 rows x 8 C columns] tile in the layout of
@@ -358,7 +377,7 @@ __global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint1
                                                          const uint16_t *__restrict__ agg,
                                                          const uint16_t *__restrict__ wt,
                                                          const float *__restrict__ bias,
-                                                         uint16_t *__restrict__ h_out, int32_t *err) {
+                                                         uint16_t *__restrict__ h_out, int32_t *err, bool early) {
     constexpr int K = 3 * KIN, C = K / 8, N_IT = (128 * C + kFwdThreads - 1) / kFwdThreads;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar;
@@ -379,7 +398,7 @@ __global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint1
                                    : __ldg((const uint4 *)(agg + v * 2 * KIN) + c - KIN / 8);
         }
     };
-    load(blockIdx.x);
+    if (!early) load(blockIdx.x);
     for (int i = t; i < kHidden * (K / 8); i += blockDim.x) {  // W^T [H x K] -> K-major B operand
         const int r = i / (K / 8), kc = (i % (K / 8)) * 8;
         *(uint4 *)(sB + kmajor_off(r, kc, K)) = *(const uint4 *)(wt + (size_t)r * K + kc);
@@ -387,6 +406,11 @@ __global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint1
     if (t < kHidden) sbias[t] = bias[t];
     if (w == 0) tmem_alloc(&tslot, 128);
     if (t == 0) mbar_init1(&bar);
+    if (early) {  // the weights are older than the aggregation that this launch may overlap
+        griddep_wait();
+        griddep_launch_dependents();
+        load(blockIdx.x);
+    }
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
@@ -439,19 +463,41 @@ __global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint1
     if (w == 0) tmem_dealloc(taddr, 128);
 }
 
+// one launch of the forward chain, early: it may start before the kernel before it has ended
+template <class... P, class... A>
+static cudaError_t launch_chain(bool early, void (*kern)(P...), int64_t grid, int block, int smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// a batch of at most one 128-node tile per SM (see k_gnn_agg)
+static bool small_batch(int64_t n_nodes, int n_sm) { return n_nodes <= 128ll * n_sm; }
+
 template <int KIN>
 static cudaError_t launch_fwd(GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,
                               uint16_t *h_out, uint16_t *agg, int32_t *err, int n_sm, cudaStream_t st) {
     constexpr int K = 3 * KIN;
     const int64_t n_tiles = (g.n_nodes + 127) / 128;
     if (n_tiles < 1) return cudaSuccess;
+    const bool small = small_batch(g.n_nodes, n_sm);
+    const auto agg_kern = small ? k_gnn_agg<KIN, true> : k_gnn_agg<KIN, false>;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gnn_agg<KIN>, kAggThreads, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, agg_kern, kAggThreads, 0);
     if (e != cudaSuccess) return e;
-    constexpr int chunk = kAggThreads * 8 / KIN < 128 ? 128 : kAggThreads * 8 / KIN;
-    const int64_t n_chunks = (g.n_nodes + chunk - 1) / chunk, most = (int64_t)n_sm * (per_sm < 1 ? 1 : per_sm);
-    k_gnn_agg<KIN><<<(int)(n_chunks < most ? n_chunks : most), kAggThreads, 0, st>>>(g, h_in, agg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    constexpr int pass = kAggThreads * 8 / KIN, chunk = pass < 128 ? 128 : pass;
+    const int64_t per_cta = small ? pass / 2 : chunk;
+    const int64_t n_chunks = (g.n_nodes + per_cta - 1) / per_cta, most = (int64_t)n_sm * (per_sm < 1 ? 1 : per_sm);
+    e = launch_chain(small, agg_kern, n_chunks < most ? n_chunks : most, kAggThreads, 0, st, g, h_in, agg);
+    if (e != cudaSuccess) return e;
     const int smem = 2 * 128 * K * 2;
     e = cudaFuncSetAttribute(k_gnn_fwd<KIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -459,9 +505,9 @@ static cudaError_t launch_fwd(GnnGraph g, const uint16_t *h_in, const uint16_t *
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     if (per_sm > 4) per_sm = 4;  // 4 x 128 TMEM columns per SM
-    int grid = (int)(n_tiles < (int64_t)n_sm * per_sm ? n_tiles : (int64_t)n_sm * per_sm);
-    k_gnn_fwd<KIN><<<grid, kFwdThreads, smem, st>>>(g, h_in, agg, wt, bias, h_out, err);
-    return cudaGetLastError();
+    const int64_t grid = n_tiles < (int64_t)n_sm * per_sm ? n_tiles : (int64_t)n_sm * per_sm;
+    return launch_chain(small, k_gnn_fwd<KIN>, grid, kFwdThreads, smem, st, g, h_in, (const uint16_t *)agg, wt, bias, h_out,
+                        err, small);
 }
 
 cudaError_t gnn_layer_fwd(int kin, GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,
@@ -491,6 +537,7 @@ __global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uin
     __shared__ float sout[kHeadThreads / 32][32 * kMaxLevels];
     for (int i = threadIdx.x; i < kHidden * kMaxLevels; i += blockDim.x) swh[i] = wh[i];
     if (threadIdx.x < kMaxLevels) sbh[threadIdx.x] = bh[threadIdx.x];
+    griddep_wait();  // (in a small batch this launch overlaps the last layer's)
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *so = sout[w];
@@ -604,9 +651,8 @@ cudaError_t gnn_head(GnnGraph g, const uint16_t *h3, const float *wh, const floa
                      float *loss_part, int n_sm, cudaStream_t st) {
     if (g.n_nodes == 0) return cudaSuccess;
     // the loss is reduced per CTA: a fixed grid keeps the summation order fixed
-    k_gnn_head<<<gnn_head_ctas(g.n_nodes, n_sm), kHeadThreads, 0, st>>>(g, h3, wh, bh, n_levels, labels, scale, logits,
-                                                                        dlogits, dh3, loss_part);
-    return cudaGetLastError();
+    return launch_chain(small_batch(g.n_nodes, n_sm), k_gnn_head, gnn_head_ctas(g.n_nodes, n_sm), kHeadThreads, 0, st, g, h3,
+                        wh, bh, n_levels, labels, scale, logits, dlogits, dh3, loss_part);
 }
 
 // dWh = h3^T dlogits, dbh = sum dlogits: CTA c reduces a fixed node range in tiles of

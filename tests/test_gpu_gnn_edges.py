@@ -65,3 +65,24 @@ def test_logits_gradient_and_topk(ctx, sizes, n_levels):
             assert np.allclose(got, want, atol=1e-4 * (1 + max(want)))
     model.free()
     lb.free()
+
+
+@pytest.mark.parametrize("extra", [0, 1, 200])
+def test_forward_around_one_tile_per_sm(ctx, extra):
+    """Up to 128 nodes per SM the forward pass takes its small-batch form. A node's logits do not
+    depend on the rest of the batch, so a batch on either side of the line gives bit for bit what
+    its parts give (which the test above compares with the oracle)."""
+    import torch
+    from paper_2602_20826_gb300.dagrt import Model
+    total = 128 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    rng = np.random.default_rng(90 + extra)
+    sizes = [400] * (total // 400) + [total % 400]
+    dags = [random_small_dag(rng, V, 0.02, 5000, kmin=1) for V in sizes if V]
+    model = Model(ctx, list(range(1, 16)), seed=3)
+    z = []
+    for part in (dags, dags[:9], dags[9:]):
+        lb = ctx.load(wl.from_dags(part, 148))
+        z.append(model.logits(lb).copy())
+        lb.free()
+    model.free()
+    assert len(z[0]) == total and np.array_equal(z[0], np.concatenate(z[1:]))
