@@ -311,12 +311,12 @@ __device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const
 // both took 190 (the rows of a CTA's nodes from a chunk next to its SM's other CTAs: 127, the
 // chunks' degrees then differ by SM); 16 features: 97 -> 31 and 24.
 //
-// SMALL (no SM has a second tile of the product): latency is what counts, so a warp takes the
-// predecessors or the successors of its nodes, a CTA one pass of them, and the layer's kernels
-// start early (programmatic launches): three layers and the head on 9,000 nodes of degree 55 took
-// 85 us in the other form, 58 in this. With all nodes of a large batch the two
-// kinds of lists apart cost the L1 cache more than they gain: 447 -> 473 us for the whole
-// network on 165,000 nodes.
+// SMALL (up to four 128-node tiles of the product per SM): latency is what counts, so a warp
+// takes the predecessors or the successors of its nodes, a CTA one pass of them, and the
+// layer's kernels start early (programmatic launches). Three layers and the head, in this form
+// and in the other: 9,000 nodes of degree 55 58 and 85 us, 25,000 of degree 20 81 and 101,
+// 42,000 of degree 70 150 and 175. On 165,000 nodes the two kinds of lists apart cost the L1
+// cache more than they gain (447 -> 473).
 constexpr int kAggThreads = 512;
 template <int KIN, bool SMALL>
 __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *__restrict__ h,
@@ -479,8 +479,8 @@ static cudaError_t launch_chain(bool early, void (*kern)(P...), int64_t grid, in
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// a batch of at most one 128-node tile per SM (see k_gnn_agg)
-static bool small_batch(int64_t n_nodes, int n_sm) { return n_nodes <= 128ll * n_sm; }
+// a batch of at most four 128-node tiles per SM (see k_gnn_agg)
+static bool small_batch(int64_t n_nodes, int n_sm) { return n_nodes <= 512ll * n_sm; }
 
 template <int KIN>
 static cudaError_t launch_fwd(GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,

@@ -643,9 +643,78 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
             ws.pid[ws.poff[s] - ws.indeg[s] + atomicAdd(&ws.cnt[s], 1)] = (uint16_t)u;
         }
     tm.sync();
+    // the bits of word w of a row that `planes` weigh
+    auto weigh = [&](uint64_t x, int w) {
+        uint64_t s = 0;
+        if (nb <= 24) {  // 64 * 2^24 fits: the word's sum in 32 bits
+            uint32_t t = 0;
+            for (int b = 0; b < nb; b++) t += (uint32_t)__popcll(x & planes[b * W + w]) << b;
+            s = t;
+        } else {
+            for (int b = 0; b < nb; b++) s += (uint64_t)__popcll(x & planes[b * W + w]) << b;
+        }
+        return s;
+    };
+    // Rows of up to 32 words (2,048 nodes), and any node of more than 16 predecessors: what takes
+    // the time is the latency of their rows, so a warp reads 32 / LW rows at once, one or two words
+    // per lane, and eight deep. (Dense graphs, whose levels are narrow: 100 DAGs of 300-900 nodes with
+    // 35% of the edges 10 ms, 10 of 1,500-2,500 with 30% 81; with the rows one after another 18
+    // and 121.)
+    const int LW = W <= 4 ? 4 : W <= 8 ? 8 : W <= 16 ? 16 : 32;
+    auto store_wanc = [&](int v, uint64_t w) {
+        if (tm.lane() == 0) {
+            ws.wanc[v] = w;
+            if (a.o.wanc) a.o.wanc[n0 + v] = (int64_t)w;
+        }
+    };
+    auto wide = [&](auto twoc, int v, int pb, int np) {
+        constexpr bool TWO = decltype(twoc)::value;  // rows of more than 32 words
+        const int ln = tm.lane(), step = 32 / LW;
+        uint64_t acc = 0;
+        for (int c = 0; c < W; c += 64) {
+            const int wi = c + (ln & (LW - 1)), w2 = c + 32 + ln;
+            uint64_t x = 0, x2 = 0;
+            for (int k0 = ln / LW; k0 < np; k0 += 8 * step) {
+                int p[8];
+                uint64_t z[8], z2[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) p[j] = k0 + j * step < np ? (int)ws.pid[pb + k0 + j * step] : -1;
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    z[j] = p[j] >= 0 && wi < W ? ws.anc[(int64_t)p[j] * W + wi] : 0ull;
+                    if constexpr (TWO) z2[j] = p[j] >= 0 && w2 < W ? ws.anc[(int64_t)p[j] * W + w2] : 0ull;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    x |= z[j] | (p[j] >= 0 && wi == p[j] >> 6 ? 1ull << (p[j] & 63) : 0ull);
+                    if constexpr (TWO) x2 |= z2[j] | (p[j] >= 0 && w2 == p[j] >> 6 ? 1ull << (p[j] & 63) : 0ull);
+                }
+            }
+            __syncwarp();
+            for (int o = LW; o < 32; o <<= 1) x |= __shfl_xor_sync(FULL, x, o);
+            if (c + ln < W) {  // (LW < 32: the lanes of the first row)
+                ws.anc[(int64_t)v * W + c + ln] = x;
+                acc += weigh(x, c + ln);
+            }
+            if (TWO && w2 < W) {
+                ws.anc[(int64_t)v * W + w2] = x2;
+                acc += weigh(x2, w2);
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+        store_wanc(v, acc + ws.load[v]);
+    };
     for (int l = 0; l < nlev; l++) {
         const int lb = ws.lvl_off[l], lend = (l + 1 < nlev) ? ws.lvl_off[l + 1] : V;
         const int ln = tm.lane(), stride = NT / 32;
+        if (W <= 32) {
+            for (int i = lb + tm.warp(); i < lend; i += stride) {
+                const int v = ws.topo[i], np = ws.indeg[v];
+                wide(std::false_type(), v, ws.poff[v] - np, np);
+            }
+            tm.sync();
+            continue;
+        }
         for (int i0 = lb + tm.warp(); i0 < lend; i0 += 32 * stride) {
             // the warp's next 32 nodes, one per lane; their predecessor lists are fetched two
             // nodes ahead and the predecessors' W^anc one node ahead
@@ -664,10 +733,17 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                 const int pb = __shfl_sync(FULL, peq, q) - np;
                 const int p2 = preds(min(q + 2, 31));
                 const uint64_t w1 = weight(p1);
+                if (np > 16) {
+                    wide(std::true_type(), v, pb, np);
+                    p0 = p1;
+                    p1 = p2;
+                    w0 = w1;
+                    continue;
+                }
                 // the predecessor of largest W^anc (about: any would do) and two others
                 const uint32_t key = p0 >= 0 ? __float_as_uint((float)w0) : 0u;
                 const int kb = __ffs(__ballot_sync(FULL, key == __reduce_max_sync(FULL, key))) - 1;
-                uint32_t rest = (np < 32 ? (1u << np) - 1u : FULL) & ~(1u << kb);
+                uint32_t rest = ((1u << np) - 1u) & ~(1u << kb);
                 const int pa = __shfl_sync(FULL, p0, kb);
                 const int pc = __shfl_sync(FULL, p0, (__ffs(rest) - 1) & 31);
                 rest &= rest - 1;
@@ -694,15 +770,20 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                     if (np > 1) self(x, pc);
                     if (np > 2) self(y, pd);
                     uint32_t more = rest;
-                    for (int k = 3; k < np; k++) {
-                        const int l = (__ffs(more) - 1) & 31;
-                        const int p = k < 32 ? __shfl_sync(FULL, p0, l) : (int)ws.pid[pb + k];
+                    auto other = [&]() {
+                        const int p = __shfl_sync(FULL, p0, (__ffs(more) - 1) & 31);
                         more &= more - 1;
-                        uint64_t z[4] = {0, 0, 0, 0};
+                        return p;
+                    };
+                    for (int k = 3; k < np; k += 2) {
+                        uint64_t z[4] = {0, 0, 0, 0}, z2[4] = {0, 0, 0, 0};
+                        const int p = other(), p3 = k + 1 < np ? other() : -1;
                         load(z, p);
+                        if (p3 >= 0) load(z2, p3);
                         self(z, p);
+                        if (p3 >= 0) self(z2, p3);
 #pragma unroll
-                        for (int j = 0; j < 4; j++) x[j] |= z[j];
+                        for (int j = 0; j < 4; j++) x[j] |= z[j] | z2[j];
                     }
 #pragma unroll
                     for (int j = 0; j < 4; j++) {
@@ -710,23 +791,11 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                         x[j] |= y[j];
                         if (w < W) ws.anc[(int64_t)v * W + w] = x0[j] | x[j];
                         const uint64_t add = x[j] & ~x0[j];  // zero beyond W
-                        if (add) {
-                            if (nb <= 24) {  // 64 * 2^24 fits: the word's sum in 32 bits
-                                uint32_t t = 0;
-                                for (int b = 0; b < nb; b++) t += (uint32_t)__popcll(add & planes[b * W + w]) << b;
-                                acc += t;
-                            } else {
-                                for (int b = 0; b < nb; b++) acc += (uint64_t)__popcll(add & planes[b * W + w]) << b;
-                            }
-                        }
+                        if (add) acc += weigh(add, w);
                     }
                 }
                 for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
-                acc += ws.load[v] + __shfl_sync(FULL, w0, kb);  // (no predecessor: 0)
-                if (ln == 0) {
-                    ws.wanc[v] = acc;
-                    if (a.o.wanc) a.o.wanc[n0 + v] = (int64_t)acc;
-                }
+                store_wanc(v, acc + ws.load[v] + __shfl_sync(FULL, w0, kb));  // (no predecessor: 0)
                 p0 = p1;
                 p1 = p2;
                 w0 = w1;
