@@ -187,7 +187,8 @@ struct dagrt_batch {
     // learned proposer: message-passing graph, features, activations (allocated on first use)
     struct Gnn {
         bool graph = false, train = false;
-        int32_t *pred_off, *pred_idx, *succ_off, *succ_idx, *cursor, *level, *m;
+        int2 *pred, *succ;
+        int32_t *pred_idx, *succ_idx, *cursor, *level, *m;
         int64_t *wanc;
         uint16_t *x, *h[3], *agg[3];  // agg: the layers' aggregated inputs; agg[1] alone serves
                                        // every layer of a forward pass, training keeps all
@@ -1108,9 +1109,9 @@ GnnGraph graph_of(dagrt_batch *b) {
     GnnGraph g;
     g.n_nodes = b->total_nodes;
     g.n_edges = b->total_edges;
-    g.pred_off = b->gnn.pred_off;
+    g.pred = b->gnn.pred;
     g.pred_idx = b->gnn.pred_idx;
-    g.succ_off = b->gnn.succ_off;
+    g.succ = b->gnn.succ;
     g.succ_idx = b->gnn.succ_idx;
     return g;
 }
@@ -1124,7 +1125,7 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
     const size_t N = (size_t)b->total_nodes, E = (size_t)b->total_edges;
     cudaError_t e;
     if (!G.graph) {
-        if ((e = batch_alloc(b, &G.pred_off, N + 1)) != cudaSuccess || (e = batch_alloc(b, &G.succ_off, N + 1)) != cudaSuccess ||
+        if ((e = batch_alloc(b, &G.pred, N)) != cudaSuccess || (e = batch_alloc(b, &G.succ, N)) != cudaSuccess ||
             (e = batch_alloc(b, &G.pred_idx, E)) != cudaSuccess || (e = batch_alloc(b, &G.succ_idx, E)) != cudaSuccess ||
             (e = batch_alloc(b, &G.cursor, N)) != cudaSuccess || (e = batch_alloc(b, &G.level, N)) != cudaSuccess ||
             (e = batch_alloc(b, &G.m, N)) != cudaSuccess || (e = batch_alloc(b, &G.wanc, N)) != cudaSuccess ||
@@ -1143,8 +1144,8 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
         int rc = dagrt_schedule(b, DAGRT_VAR_PAPER, &o, DAGRT_PTR_DEVICE);
         if (rc) return rc;
         const int32_t *st0 = b->plan[DAGRT_VAR_PAPER].status;
-        CK(gnn_build_graph(b->n_dags, b->node_off, b->edge_off, b->row_ptr, b->col, st0, G.pred_off, G.pred_idx,
-                           G.succ_off, G.succ_idx, G.cursor, b->max_v, ctx->n_sm, ctx->stream), "build message-passing graph");
+        CK(gnn_build_graph(b->n_dags, b->node_off, b->edge_off, b->row_ptr, b->col, st0, G.pred, G.pred_idx,
+                           G.succ, G.succ_idx, G.cursor, b->max_v, ctx->n_sm, ctx->stream), "build message-passing graph");
         CK(gnn_features(b->n_dags, b->node_off, b->wcet, b->k64, G.level, G.wanc, G.m, st0, graph_of(b), G.x,
                         ctx->n_sm, ctx->stream), "node features");
         ctx->launches += 3;

@@ -41,7 +41,7 @@ static int graph_smem(int v) { return 4 * ((kGraphWarps + 2) * v + 1); }
 // take 300 DAGs of 100-1,000 nodes from 725 to 110 us.
 __global__ void __launch_bounds__(kGraphThreads)
     k_gnn_graph(int32_t n_dags, const int64_t *node_off, const int64_t *edge_off, const int32_t *row_ptr,
-                const int32_t *col, const int32_t *status, int32_t *pred_off, int32_t *pred_idx, int32_t *succ_off,
+                const int32_t *col, const int32_t *status, int2 *pred, int32_t *pred_idx, int2 *succ,
                 int32_t *succ_idx, int32_t *cursor, int vcap) {
     extern __shared__ int32_t s_graph[];
     __shared__ uint64_t red[kGraphWarps];
@@ -53,15 +53,9 @@ __global__ void __launch_bounds__(kGraphThreads)
     for (int d = blockIdx.x; d < n_dags; d += gridDim.x) {
         const int64_t n0 = node_off[d], e0 = edge_off[d];
         const int V = (int)(node_off[d + 1] - n0);
-        if (tid == 0 && d == n_dags - 1) {
-            pred_off[node_off[n_dags]] = (int32_t)edge_off[n_dags];
-            succ_off[node_off[n_dags]] = (int32_t)edge_off[n_dags];
-        }
         if (status[d] != DAGRT_OK) {  // a DAG the scheduler rejected: its CSR is not trusted
-            for (int v = tid; v < V; v += kGraphThreads) {
-                succ_off[n0 + v] = (int32_t)e0;
-                pred_off[n0 + v] = (int32_t)e0;
-            }
+            for (int v = tid; v < V; v += kGraphThreads)
+                succ[n0 + v] = pred[n0 + v] = make_int2((int32_t)e0, (int32_t)e0);
             continue;
         }
         const int32_t *rp = row_ptr + n0 + d;
@@ -71,7 +65,7 @@ __global__ void __launch_bounds__(kGraphThreads)
             for (int v = tid; v <= V; v += kGraphThreads) {
                 const int x = rp[v];
                 rps[v] = x;
-                if (v < V) succ_off[n0 + v] = (int32_t)(e0 + x);
+                if (v < V) succ[n0 + v] = make_int2((int32_t)(e0 + x), (int32_t)(e0 + rp[v + 1]));
             }
             for (int i = tid; i < kGraphWarps * V; i += kGraphThreads) cur[i] = 0;
             __syncthreads();
@@ -97,7 +91,7 @@ __global__ void __launch_bounds__(kGraphThreads)
             team_scan_inplace(tm, off, V, [](uint64_t x, uint64_t y) { return x + y; }, false);
             for (int v = tid; v < V; v += kGraphThreads) {
                 const int x = v ? off[v - 1] : 0;
-                pred_off[n0 + v] = (int32_t)(e0 + x);
+                pred[n0 + v] = make_int2((int32_t)(e0 + x), (int32_t)(e0 + off[v]));
                 for (int i = 0; i < kGraphWarps; i++) cur[i * V + v] += x;
             }
             __syncthreads();
@@ -132,7 +126,7 @@ __global__ void __launch_bounds__(kGraphThreads)
             continue;
         }
         for (int v = tid; v < V; v += kGraphThreads) {
-            succ_off[n0 + v] = (int32_t)(e0 + rp[v]);
+            succ[n0 + v] = make_int2((int32_t)(e0 + rp[v]), (int32_t)(e0 + rp[v + 1]));
             cursor[n0 + v] = 0;
         }
         for (int e = tid; e < E; e += kGraphThreads) succ_idx[e0 + e] = (int32_t)(n0 + cl[e]);
@@ -140,18 +134,19 @@ __global__ void __launch_bounds__(kGraphThreads)
         for (int e = tid; e < E; e += kGraphThreads) atomicAdd(&cursor[n0 + cl[e]], 1);
         __syncthreads();
         team_scan_inplace(tm, cursor + n0, V, [](uint64_t x, uint64_t y) { return x + y; }, false);
-        for (int v = tid; v < V; v += kGraphThreads) pred_off[n0 + v] = (int32_t)(e0 + (v ? cursor[n0 + v - 1] : 0));
+        for (int v = tid; v < V; v += kGraphThreads)
+            pred[n0 + v] = make_int2((int32_t)(e0 + (v ? cursor[n0 + v - 1] : 0)), (int32_t)(e0 + cursor[n0 + v]));
         __syncthreads();
         for (int v = tid; v < V; v += kGraphThreads) cursor[n0 + v] = 0;
         __syncthreads();
         for (int u = tid; u < V; u += kGraphThreads)  // fill in any order ...
             for (int e = rp[u]; e < rp[u + 1]; e++) {
                 const int s = cl[e];
-                pred_idx[pred_off[n0 + s] + atomicAdd(&cursor[n0 + s], 1)] = (int32_t)(n0 + u);
+                pred_idx[pred[n0 + s].x + atomicAdd(&cursor[n0 + s], 1)] = (int32_t)(n0 + u);
             }
         __syncthreads();
         for (int v = tid; v < V; v += kGraphThreads) {  // ... then sort each list (increasing predecessor id)
-            int32_t *p = pred_idx + pred_off[n0 + v];
+            int32_t *p = pred_idx + pred[n0 + v].x;
             const int n = cursor[n0 + v];
             for (int i = 1; i < n; i++) {
                 const int32_t x = p[i];
@@ -168,8 +163,8 @@ __global__ void __launch_bounds__(kGraphThreads)
 }
 
 cudaError_t gnn_build_graph(int32_t n_dags, const int64_t *node_off, const int64_t *edge_off, const int32_t *row_ptr,
-                            const int32_t *col, const int32_t *status, int32_t *pred_off, int32_t *pred_idx,
-                            int32_t *succ_off, int32_t *succ_idx, int32_t *cursor, int max_v, int n_sm,
+                            const int32_t *col, const int32_t *status, int2 *pred, int32_t *pred_idx,
+                            int2 *succ, int32_t *succ_idx, int32_t *cursor, int max_v, int n_sm,
                             cudaStream_t st) {
     if (n_dags == 0) return cudaSuccess;
     const int vcap = max_v < kGraphSmemV ? max_v : kGraphSmemV;
@@ -177,7 +172,7 @@ cudaError_t gnn_build_graph(int32_t n_dags, const int64_t *node_off, const int64
     if (e != cudaSuccess) return e;
     const int grid = n_dags < 32 * n_sm ? n_dags : 32 * n_sm;
     k_gnn_graph<<<grid, kGraphThreads, graph_smem(vcap), st>>>(n_dags, node_off, edge_off, row_ptr, col, status,
-                                                               pred_off, pred_idx, succ_off, succ_idx, cursor, vcap);
+                                                               pred, pred_idx, succ, succ_idx, cursor, vcap);
     return cudaGetLastError();
 }
 
@@ -230,8 +225,9 @@ __global__ void __launch_bounds__(kFeatThreads) k_gnn_features(int32_t n_dags, c
             for (int q = 0; q < kFeat; q++) f[q] = 0.f;
             f[0] = log2f((float)wcet[i]) / 32.f;
             f[1] = (float)k64[i] / 64.f;
-            f[2] = log2f(1.f + (float)(g.pred_off[i + 1] - g.pred_off[i])) / 8.f;
-            f[3] = log2f(1.f + (float)(g.succ_off[i + 1] - g.succ_off[i])) / 8.f;
+            const int2 pl = g.pred[i], sl = g.succ[i];
+            f[2] = log2f(1.f + (float)(pl.y - pl.x)) / 8.f;
+            f[3] = log2f(1.f + (float)(sl.y - sl.x)) / 8.f;
             f[4] = depth > 0 ? (float)level[i] / (float)depth : 0.f;
             f[5] = tot > 0 ? (float)((double)wanc[i] / tot) : 0.f;
             f[6] = log2f((float)max(m[i], 1)) / 12.f;
@@ -272,11 +268,12 @@ __device__ __forceinline__ void acc8(uint64_t *acc, uint4 u) {
     }
 }
 
-// bf16 mean over the rows idx[b .. e) of h, features [8 sub, 8 sub + 8): fp32 sums in list
+// bf16 mean over the rows idx[list.x .. list.y) of h, features [8 sub, 8 sub + 8): fp32 sums in list
 // order, one rounding; four rows in flight
 template <int KIN>
-__device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const int32_t *__restrict__ idx, int b,
-                                           int e, int sub) {
+__device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const int32_t *__restrict__ idx, int2 list,
+                                           int sub) {
+    const int b = list.x, e = list.y;
     uint64_t acc[4] = {0, 0, 0, 0};
     const uint4 *hs = (const uint4 *)h + sub;
     int i = b;
@@ -327,10 +324,11 @@ __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const ui
         griddep_launch_dependents();
         constexpr int NODES = kAggThreads / 2 / LPN;
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane % LPN, succ = w & 1;
-        const int32_t *off = succ ? g.succ_off : g.pred_off, *idx = succ ? g.succ_idx : g.pred_idx;
+        const int2 *list = succ ? g.succ : g.pred;
+        const int32_t *idx = succ ? g.succ_idx : g.pred_idx;
         for (int64_t v = (int64_t)blockIdx.x * NODES + (w >> 1) * (32 / LPN) + lane / LPN; v < g.n_nodes;
              v += (int64_t)gridDim.x * NODES)
-            ((uint4 *)(agg + v * 2 * KIN))[succ * LPN + sub] = mean_rows<KIN>(h, idx, off[v], off[v + 1], sub);
+            ((uint4 *)(agg + v * 2 * KIN))[succ * LPN + sub] = mean_rows<KIN>(h, idx, list[v], sub);
     } else {
         constexpr int NODES = kAggThreads / LPN;          // nodes per CTA pass
         constexpr int CHUNK = NODES < 128 ? 128 : NODES;  // neighbouring nodes that a CTA takes together
@@ -340,8 +338,8 @@ __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const ui
                 const int64_t v = c0 + i * NODES + threadIdx.x / LPN;
                 if (v >= g.n_nodes) break;
                 uint4 *dst = (uint4 *)(agg + v * 2 * KIN);
-                dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred_off[v], g.pred_off[v + 1], sub);
-                dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ_off[v], g.succ_off[v + 1], sub);
+                dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred[v], sub);
+                dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ[v], sub);
             }
     }
 }
@@ -994,9 +992,9 @@ __global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < g.n_nodes; u += warps) {
         float4 s = __ldg((const float4 *)(da + u * K) + lane);
-        auto gather = [&](const int32_t *__restrict__ off, const int32_t *__restrict__ idx,
-                          const int32_t *__restrict__ noff, int third) {
-            const int b = off[u], e = off[u + 1];
+        auto gather = [&](const int2 *__restrict__ list, const int32_t *__restrict__ idx,
+                          const int2 *__restrict__ nlist, int third) {
+            const int b = list[u].x, e = list[u].y;
             for (int i = b; i < e; i += 4) {
                 float4 x[4];
                 float n[4];
@@ -1004,7 +1002,8 @@ __global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__
                 for (int j = 0; j < 4; j++) {
                     if (i + j >= e) break;
                     const int64_t v = __ldg(idx + i + j);
-                    n[j] = (float)(__ldg(noff + v + 1) - __ldg(noff + v));
+                    const int2 nl = __ldg(nlist + v);
+                    n[j] = (float)(nl.y - nl.x);
                     x[j] = __ldg((const float4 *)(da + v * K + third * KIN) + lane);
                 }
 #pragma unroll
@@ -1014,8 +1013,8 @@ __global__ void __launch_bounds__(256) k_gnn_agg_bwd(GnnGraph g, const float *__
                 }
             }
         };
-        gather(g.succ_off, g.succ_idx, g.pred_off, 1);
-        gather(g.pred_off, g.pred_idx, g.succ_off, 2);
+        gather(g.succ, g.succ_idx, g.pred, 1);
+        gather(g.pred, g.pred_idx, g.succ, 2);
         *((float4 *)(dh_in + u * KIN) + lane) = s;
     }
 }

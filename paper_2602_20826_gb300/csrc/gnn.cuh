@@ -32,8 +32,10 @@ struct ParamLayout {
 // the batch's graph for message passing (global node ids)
 struct GnnGraph {
     int64_t n_nodes, n_edges;
-    const int32_t *pred_off, *pred_idx;  // [N+1], [E]
-    const int32_t *succ_off, *succ_idx;
+    // {first, end} of each node's list in pred_idx / succ_idx [E]. Ends are kept apart from the next
+    // list's start: a DAG the scheduler rejected leaves its edges out, a gap behind the node before.
+    const int2 *pred, *succ;
+    const int32_t *pred_idx, *succ_idx;
 };
 
 struct GnnParams {
@@ -46,8 +48,8 @@ struct GnnParams {
 // graph build: per-DAG CSRs -> global pred/succ CSRs (deterministic order); DAGs whose
 // paper schedule failed (status != DAGRT_OK) get no edges
 cudaError_t gnn_build_graph(int32_t n_dags, const int64_t *node_off, const int64_t *edge_off, const int32_t *row_ptr,
-                            const int32_t *col, const int32_t *status, int32_t *pred_off, int32_t *pred_idx,
-                            int32_t *succ_off, int32_t *succ_idx, int32_t *cursor, int max_v, int n_sm,
+                            const int32_t *col, const int32_t *status, int2 *pred, int32_t *pred_idx,
+                            int2 *succ, int32_t *succ_idx, int32_t *cursor, int max_v, int n_sm,
                             cudaStream_t st);
 // features from the batch and the paper schedule's outputs (zero for failed DAGs)
 cudaError_t gnn_features(int32_t n_dags, const int64_t *node_off, const int64_t *wcet, const uint8_t *k64,
