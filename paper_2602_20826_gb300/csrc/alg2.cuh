@@ -346,6 +346,10 @@ __device__ __noinline__ int members_large(const A2<SH, ID> w, int variant, uint3
 // its way. Ranks instead of ids take the lookups out of the chain: the released set is one
 // 32-bit word per lane (up to 1,024 nodes) or a mask with a summary word per lane (SUM).
 //
+// Where all lanes store alike, each has read what it needs from there first: a warp barrier (the
+// one that ends release_succ, or one of its own) stands between the records' loads and the stores
+// that change them, and between a plan row and the store that marks it the last of its group.
+//
 // A segment p is the largest load that finishes within R on min(p, S) SMs, and adding one
 // tick of load adds at most one tick of time: the part takes exactly R.
 //
@@ -560,8 +564,10 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                         sbits &= sbits - 1;
                         cw = sl * 64 + b;
                         bits = ((const uint64_t *)w.rel())[cw];
-                        if (!bits && lane == 0)  // emptied since it was marked
-                            atomicAnd(w.sum() + 2 * sl + (b >> 5), ~(1u << (b & 31)));
+                        if (!bits) {  // emptied since it was marked
+                            if (lane == 0) atomicAnd(w.sum() + 2 * sl + (b >> 5), ~(1u << (b & 31)));
+                            __syncwarp();  // before a release marks it again
+                        }
                     }
                     const int b = __ffsll((long long)bits) - 1;
                     bits &= bits - 1;
@@ -574,9 +580,12 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
             if (early) {  // every lane has its copy of the released set
                 __syncwarp();
                 nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
+            } else if constexpr (!FULL_OUT) {
+                __syncwarp();  // (from here on every release ends with one)
             }
             T WS = R * (T)S;  // Eq.6 (literal variant)
             while (u >= 0) {
+                if constexpr (FULL_OUT) __syncwarp();  // (not every round has a release)
                 const uint32_t x = qu.x, k = qu.w >> 16;
                 uint32_t mu = min(x, S), p = 0, cu;
                 bool fits;
@@ -637,10 +646,12 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                 if (!defer) nrel += release_succ<SUM, FULL_OUT>(w, ub, ud, su, lane);
                 u = u1;
             }
+            if constexpr (FULL_OUT) __syncwarp();
             // the last launch ends the group
             if (nwhole && seg < 0 && (!FULL_OUT || plan)) plan[row - 1].z = lastz | (1u << 24);
-        } else if (early) {
-            nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
+        } else {
+            __syncwarp();  // every lane has its copy of the member's record
+            if (early) nrel += release_succ<SUM, FULL_OUT>(w, q.z, deg, s0, lane);
         }
         const int nl = nwhole + (seg >= 0);
         if constexpr (FULL_OUT) {

@@ -1081,6 +1081,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
             for (int i = 0; tm.warp() == 0 && i < V; i++) {
                 const int v = ws.topo[i];
                 const uint64_t dv = ws.cpT[v] + ws.cpM[v];
+                __syncwarp();  // every lane has read cpT[v]
                 ws.cpT[v] = dv;
                 for (int e = (int)rp[v] + tm.lane(); e < (int)rp[v + 1]; e += 32) {
                     const int s = ws.byrank[col[e]];
