@@ -962,6 +962,7 @@ extern "C" int dagrt_bound(dagrt_batch *b, int32_t n_variants, const int32_t *va
         int rc = ensure_bscr(b, bound_chunk_scratch(b->n_dags, b->total_nodes, n_variants, n_alloc, b->tune.chunk_rows));
         if (rc) return rc;
         char *t = (char *)b->bscr;
+        ch.counter = (uint32_t *)t;  // the first 256 bytes
         ch.acc = (unsigned long long *)(t + 256);
         ch.warps = b->tune.item_warps;
         ch.alloc_rows = 2 * b->total_nodes;

@@ -702,13 +702,15 @@ size_t bound_chunk_scratch(int32_t n_dags, int64_t total_nodes, int32_t n_varian
 // the DAG's per-candidate accumulators; lane l reads candidates 2l and 2l + 1 of four
 // 64-candidate blocks at a time, writes the bounds (-1 for a variant whose schedule
 // failed), clears the accumulators for the next call and takes the argmin by shuffles. The
-// statuses are read before the wait on the work items.
+// statuses are read before the wait on the work items. Block 0 also resets the work-item
+// counter.
 __global__ void __launch_bounds__(32) k_bound_finish(BoundArgs a, ChunkArgs ch) {
     const int nv = a.n_variants, ncb = a.n_alloc / 64, n_cand = nv * a.n_alloc, nblk = nv * ncb;
     const int lane = threadIdx.x;
     int32_t st = 0;
     if (lane < nv && (int)blockIdx.x < a.n_dags) st = a.status[lane][blockIdx.x];
     griddep_wait();
+    if (blockIdx.x == 0 && lane == 0) *ch.counter = 0u;
     for (int d = blockIdx.x; d < a.n_dags; d += gridDim.x) {
         if (d != (int)blockIdx.x && lane < nv) st = a.status[lane][d];
         unsigned long long *acc = ch.acc + (int64_t)d * n_cand;
@@ -866,34 +868,19 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
     __syncthreads();
     const uint32_t total = (uint32_t)s_cum[nv];
 
-    // This warp's run of items [first, first + count): as many as the others' or one more (one at
-    // a time off a counter: 62.2 us for 1,000 DAGs of 50-500 nodes x 256 candidates, now 61.6). Lane k
-    // holds the k-th record {d, first row, end row, flags}, variant slot and candidate block of
-    // the current 32.
-    const uint32_t nw = gridDim.x * (blockDim.x >> 5), me = blockIdx.x * (blockDim.x >> 5) + w;
-    const uint32_t share = total / nw, more = total % nw;
-    const uint32_t first = me * share + min(me, more), count = share + (me < more);
-    int4 l_rec = make_int4(0, 0, 0, 0);
-    int l_vi = 0, l_cb = 0;
-    auto fetch = [&](uint32_t k0) {
-        if (k0 + lane >= count) return;
-        const uint32_t j = first + k0 + lane;
-        l_vi = 0;
-        while ((int64_t)j >= s_cum[l_vi + 1]) l_vi++;
-        const uint32_t jj = j - (uint32_t)s_cum[l_vi];
-        const uint32_t q = ncb == 1 ? jj : jj / (uint32_t)ncb;
-        l_cb = (int)(jj - q * (uint32_t)ncb);
-        l_rec = ch.item[l_vi][q];
+    auto grab = [&]() -> uint32_t {
+        uint32_t v = 0;
+        if (lane == 0) v = atomicAdd(ch.counter, 1u);
+        return __shfl_sync(FULL, v, 0);
     };
-    auto locate = [&](uint32_t k, int &vi, int &cb, int4 &rec) {  // item k of the run
-        if (k > 0 && (k & 31u) == 0) fetch(k);
-        const int l = (int)(k & 31u);
-        vi = __shfl_sync(FULL, l_vi, l);
-        cb = __shfl_sync(FULL, l_cb, l);
-        rec.x = __shfl_sync(FULL, l_rec.x, l);
-        rec.y = __shfl_sync(FULL, l_rec.y, l);
-        rec.z = __shfl_sync(FULL, l_rec.z, l);
-        rec.w = __shfl_sync(FULL, l_rec.w, l);
+    // variant slot, 64-candidate block and record of item j
+    auto locate = [&](uint32_t j, int &vi, int &cb, int4 &rec) {
+        vi = 0;
+        while ((int64_t)j >= s_cum[vi + 1]) vi++;
+        const uint32_t jj = j - (uint32_t)s_cum[vi];
+        const uint32_t q = ncb == 1 ? jj : jj / (uint32_t)ncb;
+        cb = (int)(jj - q * (uint32_t)ncb);
+        rec = ch.item[vi][q];
     };
     uint32_t parity = 0u;    // bit b: parity of the next wait on buffer b
     uint32_t inflight = 0u;  // bit b: a copy issued into buffer b and not yet waited for
@@ -920,20 +907,19 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
         return ok;
     };
 
-    uint32_t j = 0;
+    uint32_t j = grab();
     int vi = 0, cb = 0, buf = 0;
     int4 rec = make_int4(0, 0, 0, 0);
-    fetch(0);
-    if (count > 0) {
-        locate(0, vi, cb, rec);
+    if (j < total) {
+        locate(j, vi, cb, rec);
         stage(0, vi, cb, rec.y, min(rec.z, rec.y + kSubRows));
     }
     bool failed = false;
-    while (j < count && !failed) {
-        const uint32_t jn = j + 1;
+    while (j < total && !failed) {
+        const uint32_t jn = grab();
         int vn = 0, cbn = 0;
         int4 recn = make_int4(0, 0, 0, 0);
-        if (jn < count) locate(jn, vn, cbn, recn);
+        if (jn < total) locate(jn, vn, cbn, recn);
         // the item's phases; FIT: 32-bit table path, else 64-bit sums with exec_time
         auto run_item = [&](auto fitc) {
             constexpr bool FIT = decltype(fitc)::value;
@@ -951,7 +937,7 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
                 // item's next rows, or the first rows of the next item
                 if (g0 + kSubRows < rec.z)
                     stage(buf ^ 1, vi, cb, g0 + kSubRows, min(rec.z, g0 + 2 * kSubRows));
-                else if (jn < count)
+                else if (jn < total)
                     stage(buf ^ 1, vn, cbn, recn.y, min(recn.z, recn.y + kSubRows));
                 const unsigned char *cbuf = wbase + buf * kStageBytes;
                 const uint4 *pbuf = (const uint4 *)(cbuf + kSubRows * 64);
@@ -1100,6 +1086,8 @@ cudaError_t bound_launch(const BoundArgs &a, const ChunkArgs *ch, int n_sm, cuda
     const int n_cand = a.n_variants * a.n_alloc;
     const bool items = ch != nullptr;
     if (items) {
+        // the item counter is zero here: set when the scratch was allocated, and reset by
+        // k_bound_finish at the end of every call
         cudaError_t e;
         CUtensorMap tmap;
         if ((e = encode_alloc_map(a, ch->alloc_rows, &tmap)) != cudaSuccess) return e;

@@ -92,12 +92,13 @@ cudaError_t bound_build_chunks(int32_t n_dags, const int64_t *node_off, const ui
 struct ChunkArgs {
     const int32_t *chunk[kMaxVariantsPerCall], *nchunk[kMaxVariantsPerCall], *cpre[kMaxVariantsPerCall];
     const int4 *item[kMaxVariantsPerCall];
+    uint32_t *counter;            // work-item counter
     unsigned long long *acc;      // [n_dags * n_cand] bound accumulators; zero between calls
     int32_t warps;                // warps per CTA of the work-item kernel
     int64_t alloc_rows;           // rows of the candidate-byte array (2 * total nodes)
 };
 
-// scratch bytes the balanced path needs for a call (the accumulators behind 256 bytes); all of it must
+// scratch bytes the balanced path needs for a call (counter, accumulators); all of it must
 // be zero before the first call, and every call leaves it zero
 size_t bound_chunk_scratch(int32_t n_dags, int64_t total_nodes, int32_t n_variants, int32_t n_alloc, int chunk_rows);
 // the call can take the balanced path (materialised candidates, n_alloc % 64 == 0, and few
