@@ -128,7 +128,8 @@ constexpr int kSoloNodes = 32;
 // bytes in two registers, so a round of Rule 2 costs two warp reductions, a look at the lane's own
 // heads and a byte comparison, however many nodes wait. A forest with loads above M has a round per
 // node: rounds that scan all nodes, with one 64-bit atomic maximum per head, took 10,000 cycles each
-// for 256 isolated nodes. `mask`: 8 words, zero before and after.
+// for 256 isolated nodes (600 binary trees of 256 nodes, loads up to 10,000: 1,245 -> 300 us).
+// `mask`: 8 words, zero before and after.
 __device__ __forceinline__ uint32_t peel_solo(uint32_t b, uint32_t n, uint32_t M, int V, int NC, const uint32_t *load,
                                            const uint8_t *rank, const uint8_t *byrank, const uint8_t *blk,
                                            const uint8_t *lpred, uint16_t *rnd, uint32_t *mask, int lane) {
@@ -529,9 +530,10 @@ __device__ __forceinline__ void schedule_warp(const WarpWs &ws, uint32_t base, c
 
     // ---- Alg.1: peel every block's out-forest round by round; a round of a block takes Top_M
     //      of its heads by W^anc (Rule 1), or a single head with C^ >= M (Rule 2). Blocks of more
-    //      than kSoloNodes nodes are peeled one after another (they may have a round per node),
-    //      then all others advance together. A node has an in-block predecessor only if it has a single
-    //      predecessor (a join's ancestors are in blocks up to its own, it is in a later one).
+    //      than kSoloNodes nodes (they may have a round per node) or than M (more than M heads) are
+    //      peeled one after another, then all others advance together. A node has an in-block
+    //      predecessor only if it has a single predecessor (a join's ancestors are in blocks up to
+    //      its own, it is in a later one).
     uint16_t *rnd = (uint16_t *)(smem + base + ws.rnd), *nround = (uint16_t *)(smem + base + ws.nround);
     unsigned long long *bigk = (unsigned long long *)(smem + base + ws.bigk);
     uint32_t *fcnt = (uint32_t *)(smem + base + ws.fcnt);
@@ -545,88 +547,39 @@ __device__ __forceinline__ void schedule_warp(const WarpWs &ws, uint32_t base, c
         lpred[v] = (uint8_t)(blk[p] == blk[v] ? p : (uint32_t)v);
     }
     __syncwarp();
-    bool bigblk = false;  // a block of more than M nodes may have more than M heads
     if (V > kSoloNodes || V > (int)M) {
         for (int v = lane; v < V; v += 32) atomicAdd(&fcnt[blk[v]], 1u);
         __syncwarp();
         for (int c = 0; c < NC; c++) {
-            const int b0 = 32 * c + lane;
-            const uint32_t n = b0 < V ? fcnt[b0] : 0u;  // the block's nodes
-            for (uint32_t m = __ballot_sync(FULL, n > (uint32_t)kSoloNodes); m; m &= m - 1) {
+            const uint32_t n = 32 * c + lane < V ? fcnt[32 * c + lane] : 0u;  // the block's nodes
+            for (uint32_t m = __ballot_sync(FULL, n > min((uint32_t)kSoloNodes, M)); m; m &= m - 1) {
                 const int b = 32 * c + __ffs(m) - 1;
-                const uint32_t rounds =
-                    peel_solo(b, __shfl_sync(FULL, n, __ffs(m) - 1), M, V, NC, load, rank, byrank, blk, lpred, rnd, (uint32_t *)bigk, lane);
+                const uint32_t rounds = peel_solo(b, __shfl_sync(FULL, n, __ffs(m) - 1), M, V, NC, load, rank, byrank, blk,
+                                                  lpred, rnd, (uint32_t *)bigk, lane);
                 if (lane == 0) nround[b] = (uint16_t)rounds;
             }
-            bigblk |= n > M && n <= (uint32_t)kSoloNodes;
-            if (b0 < V) fcnt[b0] = 0;
         }
-        bigblk = __any_sync(FULL, bigblk);
         __syncwarp();
     }
     // the key of a head that Rule 2 may take alone: the largest load, then the lowest rank
     auto big_key = [&](uint32_t v) { return ((unsigned long long)load[v] << 16) | (0xffffu - rank[v]); };
     for (uint32_t round = 0;; round++) {
-        uint32_t hm = 0, take = 0;  // this lane's heads by chunk, and those in Top_M
+        uint32_t hm = 0;  // this lane's heads by chunk: all of them are in Top_M
         for (int c = 0; c < NC; c++) {
             const int v = 32 * c + lane;
             if (v < V && rnd[v] == kNone) {
                 const uint32_t p = lpred[v];
                 if (p == (uint32_t)v || rnd[p] < round) {
                     hm |= 1u << c;
-                    if (bigblk) atomicAdd(&fcnt[blk[v]], 1u);
-                    else if (load[v] >= M) atomicMax(&bigk[blk[v]], big_key(v));
+                    if (load[v] >= M) atomicMax(&bigk[blk[v]], big_key(v));
                 }
             }
         }
         if (!__any_sync(FULL, hm != 0)) break;
-        take = hm;
         __syncwarp();
-        if (bigblk) {
-            // over-full blocks keep the heads up to the rank of their M-th: fcnt becomes
-            // that rank | 2^31. Each lane shows its heads by rank, 32 ranks at a time.
-            for (int c = 0; c < NC; c++) {
-                const int v = 32 * c + lane;
-                const bool h = (hm >> c) & 1u;
-                for (;;) {
-                    const uint32_t f = h ? fcnt[blk[v]] : 0u;
-                    const uint32_t ob = __ballot_sync(FULL, f > M && !(f >> 31));
-                    if (!ob) break;
-                    const uint32_t b = __shfl_sync(FULL, h ? (uint32_t)blk[v] : 0u, __ffs(ob) - 1);
-                    uint32_t seen = 0, th = 0;
-                    for (int r0 = 0; r0 < V; r0 += 32) {
-                        const int r = r0 + lane;
-                        bool in = false;
-                        if (r < V) {
-                            const uint32_t w = byrank[r];
-                            const uint32_t p = lpred[w];
-                            in = blk[w] == b && rnd[w] == kNone && (p == w || rnd[p] < round);
-                        }
-                        uint32_t mb = __ballot_sync(FULL, in);
-                        const uint32_t n = __popc(mb);
-                        if (seen + n >= M) {  // the M-th head is among these ranks
-                            for (uint32_t i = 1; i < M - seen; i++) mb &= mb - 1;
-                            th = r0 + __ffs(mb) - 1;
-                            break;
-                        }
-                        seen += n;
-                    }
-                    if (lane == 0) fcnt[b] = th | (1u << 31);
-                    __syncwarp();
-                }
-            }
-            for (int c = 0; c < NC; c++) {
-                const int v = 32 * c + lane;
-                if (!((hm >> c) & 1u)) continue;
-                const uint32_t f = fcnt[blk[v]];
-                if ((f >> 31) && rank[v] > (f & 0xffffu)) take &= ~(1u << c);
-                else if (load[v] >= M) atomicMax(&bigk[blk[v]], big_key(v));
-            }
-            __syncwarp();
-        }
         for (int c = 0; c < NC; c++) {
             const int v = 32 * c + lane;
-            if (!((take >> c) & 1u)) continue;
+            if (!((hm >> c) & 1u)) continue;
             const unsigned long long bg = bigk[blk[v]];
             if (bg == 0 || (uint32_t)(bg & 0xffffu) == 0xffffu - rank[v]) {
                 rnd[v] = (uint16_t)round;
@@ -635,11 +588,7 @@ __device__ __forceinline__ void schedule_warp(const WarpWs &ws, uint32_t base, c
         }
         __syncwarp();
         for (int c = 0; c < NC; c++)
-            if ((hm >> c) & 1u) {
-                const uint32_t b = blk[32 * c + lane];
-                bigk[b] = 0;
-                fcnt[b] = 0;
-            }
+            if ((hm >> c) & 1u) bigk[blk[32 * c + lane]] = 0;
         __syncwarp();
     }
 
