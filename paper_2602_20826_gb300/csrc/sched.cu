@@ -414,7 +414,8 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
     const int nb = 64 - __clzll((long long)mx);
     if constexpr (SH) {
         // ---- Shared memory: levels by one warp, node by node in topological order -- the ids,
-        //      where every edge leads to a larger one, else Kahn's queue. Then (with the ids as
+        //      where every edge leads to a larger one, else Kahn's queue; nodes without successors
+        //      are left out (1,000 isolated ones waited for 1,000 steps). Then (with the ids as
         //      order: meanwhile) the closure: its 64-bit columns are independent, so every warp
         //      carries its own columns through all nodes, a lane per successor (they are
         //      distinct: no atomics), without a barrier between levels. Column by column in
@@ -426,6 +427,19 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
             for (int v = tm.t; v < V; v += NT) ws.anc[w * V + v] = v >> 6 == w ? 1ull << (v & 63) : 0ull;
         if (ids)
             for (int v = tm.t; v < V; v += NT) ws.lvl_off[v] = 0;  // levels, until they are written out
+        uint16_t *list = ws.byrank;  // the nodes with successors, in topological order
+        auto collect = [&](auto ith) {  // one warp; their number in sc[4]
+            int n = 0;
+            for (int i0 = 0; i0 < V; i0 += 32) {
+                const int u = i0 + lane < V ? ith(i0 + lane) : 0;
+                const bool has = i0 + lane < V && rp[u + 1] > rp[u];
+                const uint32_t hb = __ballot_sync(FULL, has);
+                if (has) list[n + __popc(hb & ((1u << lane) - 1))] = (uint16_t)u;
+                n += __popc(hb);
+            }
+            if (lane == 0) sc[4] = n;
+        };
+        if (ids && wp == 0) collect([](int i) { return i; });
         tm.sync();
         const int cw = (W + NWP - 1) / NWP;
         int w0 = min(W, wp * cw);  // this warp's columns, w0 .. w1 - 1
@@ -459,6 +473,7 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                     __syncwarp();
                 }
                 if (lane == 0) sc[1] = tail == V ? L + 1 : 0;
+                if (tail == V) collect([&](int i) { return (int)ws.topo[i]; });
             }
             tm.sync();
             nlev = sc[1];
@@ -468,19 +483,20 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
             }
         }
         uint16_t *lev = ws.lvl_off;
-        int top = 0;
+        const int nlist = sc[4];
         // the warp's columns w0 .. w0 + CW - 1 of the closure. A node takes one load's latency:
         // its edges' bounds are loaded two nodes ahead, its first 32 successors one node ahead,
         // and all rows before any is stored (440 -> 300 cycles a node at 500 nodes)
         auto columns = [&](auto cwc, auto lvc) {
             constexpr int CW = decltype(cwc)::value;
             constexpr bool LV = decltype(lvc)::value;
-            auto node = [&](int i) { return ids ? min(i, V - 1) : (int)ws.topo[min(i, V - 1)]; };
+            auto node = [&](int i) { return (int)list[min(i, nlist - 1)]; };
             uint64_t *anc = ws.anc + w0 * V;
+            if (nlist == 0) return;
             int u = node(0), u1 = node(1);
             int eb = (int)rp[u], end = (int)rp[u + 1], eb1 = (int)rp[u1], end1 = (int)rp[u1 + 1];
             int s = eb + lane < end ? col[eb + lane] : 0;
-            for (int i = 0; i < V; i++) {
+            for (int i = 0; i < nlist; i++) {
                 const int u2 = node(i + 2);
                 const int eb2 = (int)rp[u2], end2 = (int)rp[u2 + 1];
                 const int s1 = eb1 + lane < end1 ? col[eb1 + lane] : 0;
@@ -502,7 +518,6 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
                         if constexpr (LV) lev[s] = (uint16_t)max(ls, l);
                     }
                 }
-                if constexpr (LV) top = max(top, (int)l);
                 __syncwarp();
                 u = u1;
                 u1 = u2;
@@ -532,12 +547,14 @@ __device__ void schedule_one(const Team<NT> &tm, const Ws &ws, const SchedArgs &
             if (c == 0) break;
         }
         if (ids) {
-            if (tm.t == NT - 1) sc[1] = top;
             tm.sync();
-            nlev = sc[1];
-            if (a.o.level)
-                for (int v = tm.t; v < V; v += NT) a.o.level[n0 + v] = lev[v];
-            for (int v = tm.t; v < V; v += NT) ws.topo[v] = (uint16_t)v;
+            uint64_t top = 0;
+            for (int v = tm.t; v < V; v += NT) {
+                top = max(top, (uint64_t)lev[v]);
+                if (a.o.level) a.o.level[n0 + v] = lev[v];
+                ws.topo[v] = (uint16_t)v;
+            }
+            nlev = (int)tm.maxu(top) + 1;
         }
         tm.sync();
         // ---- Eq.2: W^anc(v) = sum of C^ over v and its ancestors, by bit planes of C^
