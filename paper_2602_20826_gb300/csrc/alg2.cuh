@@ -673,10 +673,11 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
             }
         }
         // ---- the members' rows; members finish with pi_j and release their successors
-        auto release_lanes = [&]() {  // lane by lane: targets of different members may coincide
-            for (uint32_t b = live; b; b &= b - 1) {
+        auto release_lanes = [&](uint32_t b) {  // lane by lane: targets of different members may coincide
+            for (; b; b &= b - 1) {
                 const int l = __ffs(b) - 1;
                 const uint32_t eb = __shfl_sync(FULL, q.z, l), dl = __shfl_sync(FULL, q.w, l) & 0xffffu;
+                if (!dl) continue;
                 const uint32_t s = (uint32_t)lane < dl ? w.col(eb + lane) : 0u;
                 nrel += release_succ<SUM, FULL_OUT>(w, eb, dl, s, lane);
             }
@@ -695,7 +696,7 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                 write_own_row(nrows + i, idm, j, q.x, m | (q.w & 0xffff0000u), c, nl == 0 && i == np - 1);
                 finish_own(r, idm, j, m);
             }
-            release_lanes();
+            release_lanes(live);
         } else {
             int i = 0;  // rows written
             for (int i0 = 0; i0 < n; i0 += 32) {
@@ -712,7 +713,7 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                     finish_own(r, idm, j, mr);
                 }
                 i += __popc(live);
-                release_lanes();
+                release_lanes(__ballot_sync(FULL, q.x && (q.w & 0xffffu)));
             }
         }
         if constexpr (FULL_OUT) {
