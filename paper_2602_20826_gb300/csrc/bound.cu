@@ -123,7 +123,7 @@ __device__ __forceinline__ uint32_t gen_alloc(const BoundArgs &a, int d, int c, 
 // a lane above 32 allocations (one: 359 us instead of 279 below). Windows of 32 rows: 64 and
 // 128 take 65 and 92 us instead of 58 on the second workload, the first does not care.
 // 500 DAGs of 100-1,000 nodes x 256 perturbations: 3.06 -> 0.28 ms; 1,000 DAGs of 20-200 nodes
-// x 74 allocations: 116 -> 63 us a call.
+// x 74 allocations: 116 -> 53 us a call; 5,000 DAGs of 3-6 nodes x 100 allocations: 31 -> 29.
 constexpr int kRowWindow = 32;
 constexpr int kRowTile = 2048;   // candidates of one pass over the DAG (shared-memory sums)
 enum { SRC_BYTES = 0, SRC_RANDOM = 1, SRC_PERTURB = 2 };
@@ -147,12 +147,15 @@ struct Div64m {
 };
 __device__ constexpr Div64m kDiv64m;
 
+// Registers: where a lane's loads wait for bytes, warps in flight count (118 registers: 1,000 DAGs of
+// 20-200 nodes x 1,000 allocations 408 us, 80: 326); generated candidates do not care for more.
 template <int CPT, int SRC>
-__global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
+__global__ void __maxnreg__(CPT == 1 ? 64 : SRC == SRC_BYTES ? 80 : 104) k_bound_rows(BoundArgs a, int entries) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint8_t s_lev[16];
     __shared__ int64_t s_bb[16];
     __shared__ int32_t s_bc[16];
+    __shared__ bool s_ok[kMaxVariantsPerCall];
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -180,23 +183,26 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
             for (int vi = t0 / a.n_alloc; vi * a.n_alloc < t1; vi++) {
                 // allocations of this variant in this pass
                 const int a0 = max(t0 - vi * a.n_alloc, 0), a1 = min(t1 - vi * a.n_alloc, a.n_alloc);
-                const int rows = a.status[vi][d] == DAGRT_OK ? a.nrows[vi][d] : 0;
-                const bool fit = rows && (a.pflag[vi][d] & 1);
+                const int st = a.status[vi][d], nr = a.nrows[vi][d], pf = a.pflag[vi][d];  // (together: one latency)
+                const int rows = st == DAGRT_OK ? nr : 0;
+                if (tid == 0) s_ok[vi] = st == DAGRT_OK;
+                const bool fit = rows && (pf & 1);
                 const int nwin = (rows + kRowWindow - 1) / kRowWindow;
                 const int nblk = (a1 - a0 + 32 * CPT - 1) / (32 * CPT);
                 const uint4 *plan = a.plan[vi] + rbase;
-                for (; task < nwin * nblk; task += NW) {
+                // FIT: 32-bit sums, else 64-bit ones (apart, so that neither holds the other's registers)
+                auto run = [&](auto fitc) {
+                    constexpr bool FIT = decltype(fitc)::value;
                     const int win = task / nblk, al0 = a0 + (task - win * nblk) * 32 * CPT + lane;
                     const int wend = (win + 1) * kRowWindow;  // groups that start before it
                     bool on[CPT];
 #pragma unroll
                     for (int q = 0; q < CPT; q++) on[q] = al0 + 32 * q < a1;
-                    uint64_t total[CPT];
-                    uint32_t b[CPT], gmax[CPT], gsum[CPT], gm[CPT];
-                    uint64_t wmax[CPT], wsum[CPT];  // 64-bit sums
+                    using S = typename std::conditional<FIT, uint32_t, uint64_t>::type;
+                    S b[CPT], gmax[CPT], gsum[CPT];
+                    uint32_t gm[CPT];
 #pragma unroll
-                    for (int q = 0; q < CPT; q++)
-                        total[q] = 0, b[q] = gmax[q] = gsum[q] = gm[q] = 0, wmax[q] = wsum[q] = 0;
+                    for (int q = 0; q < CPT; q++) b[q] = gmax[q] = gsum[q] = 0, gm[q] = 0;
                     // is row `base` the start of a group?
                     bool prev = win == 0 || (plan[win * kRowWindow - 1].z >> 24) != 0, open = false;
                     for (int base = win * kRowWindow; base < rows && (open || base < wend); base += 32) {
@@ -219,18 +225,21 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
                         if (later && inwin < 32) rb = __ffs(later) - 1;
                         open = rb == 32 && !(endm >> 31);
                         __syncwarp();
-                        if (SRC == SRC_BYTES) {
+                        if constexpr (!FIT) {
+                        } else if (SRC == SRC_BYTES) {
                             ((uint4 *)tab)[lane] = make_uint4(x.x * (64u - k), x.x * k - 1u, x.y, m0);
-                        } else if (fit && lane < rn) {
-                            uint2 *t = tab + lane * entries;
-                            t[0] = make_uint2(x.y, m0);  // keep
-                            for (int e = 1; e < entries; e++) {
-                                const uint32_t m = SRC == SRC_PERTURB ? perturb_m(m0, e) : s_lev[e - 1];
-                                t[e] = make_uint2((uint32_t)exec_time(x.x, k, m, M), m);
+                        } else {  // 2^l lanes for the rows, the rest of the bits for a row's choices
+                            const int l = 32 - __clz(rn - 1), row = lane & ((1 << l) - 1), part = lane >> l;
+                            const uint32_t tx = __shfl_sync(FULL, x.x, row), tz = __shfl_sync(FULL, x.z, row);
+                            uint2 *t = tab + row * entries;
+                            if (lane < rn) t[0] = make_uint2(x.y, m0);  // keep
+                            for (int e = 1 + part; row < rn && e < entries; e += 32 >> l) {
+                                const uint32_t m = SRC == SRC_PERTURB ? perturb_m(tz & 0xffffu, e) : s_lev[e - 1];
+                                t[e] = make_uint2((uint32_t)exec_time(tx, (tz >> 16) & 0xffu, m, M), m);
                             }
                         }
                         __syncwarp();
-                        if (fit) {
+                        if constexpr (FIT) {
                             const uint8_t *src = a.m_alloc + (rbase + base) * a.stride + vi * a.n_alloc + al0;
                             constexpr int U = SRC == SRC_BYTES ? 8 : 2;  // rows in flight together
                             for (int rr = ra; rr < rb; rr += U) {
@@ -255,11 +264,11 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
                                             const uint2 dv = s_div[m];
                                             cm[q].x = (__umulhi(y.x * m + y.y, dv.x) >> dv.y) + 1u;
                                             cm[q].y = m;
-                                            if (m > M) {
+                                            if (m - 1u >= M) {  // the schedule's own SMs (0), or more than M
                                                 const uint4 z = plan[base + r];
-                                                cm[q].x = (uint32_t)exec_time(z.x, (z.z >> 16) & 0xffu, m, M);
+                                                cm[q] = m ? make_uint2((uint32_t)exec_time(z.x, (z.z >> 16) & 0xffu, m, M), m)
+                                                          : make_uint2(y.z, y.w);
                                             }
-                                            if (m == 0) cm[q] = make_uint2(y.z, y.w);
                                         }
                                     } else {
 #pragma unroll
@@ -297,10 +306,10 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
                                     if (SRC != SRC_BYTES) m = gen_alloc(a, d, vi * a.n_alloc + al, base + r, y.w, my, s_lev);
                                     else if (on[q]) m = a.m_alloc[(rbase + base + r) * a.stride + vi * a.n_alloc + al];
                                     const uint64_t c = m ? exec_time(y.x, ky, m, M) : (uint64_t)y.y;
-                                    wmax[q] = first || c > wmax[q] ? c : wmax[q];
-                                    wsum[q] = first ? c : wsum[q] + c;
+                                    gmax[q] = first || c > gmax[q] ? c : gmax[q];
+                                    gsum[q] = first ? c : gsum[q] + c;
                                     gm[q] = (first ? 0u : gm[q]) + (m ? m : my);
-                                    if (last) total[q] += gm[q] <= M ? wmax[q] : wsum[q];
+                                    if (last) b[q] += gm[q] <= M ? gmax[q] : gsum[q];
                                 }
                             }
                         }
@@ -308,7 +317,11 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
 #pragma unroll
                     for (int q = 0; q < CPT; q++)
                         if (on[q] && rows)
-                            atomicAdd(&s_acc[vi * a.n_alloc + al0 + 32 * q - t0], (unsigned long long)(total[q] + b[q]));
+                            atomicAdd(&s_acc[vi * a.n_alloc + al0 + 32 * q - t0], (unsigned long long)b[q]);
+                };
+                for (; task < nwin * nblk; task += NW) {
+                    if (fit) run(std::true_type());
+                    else run(std::false_type());
                 }
                 task -= nwin * nblk;
             }
@@ -324,7 +337,7 @@ __global__ void __launch_bounds__(512) k_bound_rows(BoundArgs a, int entries) {
             }
             for (int i = tid; rank == 0 && t0 + i < t1; i += blockDim.x) {
                 const int c = t0 + i;
-                const bool ok = a.status[c / a.n_alloc][d] == DAGRT_OK;
+                const bool ok = s_ok[nv == 1 ? 0 : c / a.n_alloc];
                 const int64_t v = ok ? (int64_t)s_acc[i] : -1;
                 if (a.out) a.out[(int64_t)d * n_cand + c] = v;
                 if (ok) better(best_b, best_c, v, c);
