@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(kHidden * kHgParts) k_gnn_head_grad(GnnGraph g
         const int oo = i / kMaxLevels, l = i % kMaxLevels;
         float s = 0.f;
         for (int k = 0; k < kHgParts; k++) s += s_hg[(k * kMaxLevels + l) * kHidden + oo];
-        pp[ParamLayout::Wh + i] = s;  // (levels from L on: zeros)
+        pp[ParamLayout::Wh + i] = l < L ? s : 0.f;  // (beyond L, an infinite h3 times 0 is a NaN)
     }
     if (tid < kMaxLevels) pp[ParamLayout::bh + tid] = bacc;
 }

@@ -49,3 +49,11 @@ def test_infinite_input_gradient(ctx):
     loss, g, f = _grad(ctx, 1e-37)
     assert np.isfinite(loss)
     assert np.isinf(g[B2 + f])
+
+
+def test_levels_beyond_the_models(ctx):
+    """h2 = 2: h3 is infinite, the gradient of the model's two levels not a number; the other 14
+    columns of the head stay zero."""
+    _, g, _ = _grad(ctx, 2.0)
+    assert not np.isfinite(g[WH:BH].reshape(H, LEVELS)[:, :2]).any()
+    assert (g[WH:BH].reshape(H, LEVELS)[:, 2:] == 0).all() and (g[BH + 2:BH + LEVELS] == 0).all()
