@@ -271,24 +271,28 @@ __device__ __forceinline__ void acc8(uint64_t *acc, uint4 u) {
 }
 
 // bf16 mean over the rows idx[list.x .. list.y) of h, features [8 sub, 8 sub + 8): fp32 sums in list
-// order, one rounding; four rows in flight
-template <int KIN>
-__device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const int32_t *__restrict__ idx, int2 list,
-                                           int sub) {
+// order, one rounding; four rows in flight. OVERLAP: the launch may start while the kernel that
+// writes h still runs, so h is not read-only for its whole life (what ld.global.nc asks for).
+template <int KIN, bool OVERLAP>
+__device__ __forceinline__ uint4 mean_rows(const uint16_t *h, const int32_t *__restrict__ idx, int2 list, int sub) {
+    auto ld = [](const uint4 *p) {
+        if constexpr (OVERLAP) return *p;
+        else return __ldg(p);
+    };
     const int b = list.x, e = list.y;
     uint64_t acc[4] = {0, 0, 0, 0};
     const uint4 *hs = (const uint4 *)h + sub;
     int i = b;
     for (; i + 4 <= e; i += 4) {
         const int32_t j0 = __ldg(idx + i), j1 = __ldg(idx + i + 1), j2 = __ldg(idx + i + 2), j3 = __ldg(idx + i + 3);
-        const uint4 u0 = __ldg(hs + (int64_t)j0 * (KIN / 8)), u1 = __ldg(hs + (int64_t)j1 * (KIN / 8));
-        const uint4 u2 = __ldg(hs + (int64_t)j2 * (KIN / 8)), u3 = __ldg(hs + (int64_t)j3 * (KIN / 8));
+        const uint4 u0 = ld(hs + (int64_t)j0 * (KIN / 8)), u1 = ld(hs + (int64_t)j1 * (KIN / 8));
+        const uint4 u2 = ld(hs + (int64_t)j2 * (KIN / 8)), u3 = ld(hs + (int64_t)j3 * (KIN / 8));
         acc8(acc, u0);
         acc8(acc, u1);
         acc8(acc, u2);
         acc8(acc, u3);
     }
-    for (; i < e; i++) acc8(acc, __ldg(hs + (int64_t)__ldg(idx + i) * (KIN / 8)));
+    for (; i < e; i++) acc8(acc, ld(hs + (int64_t)__ldg(idx + i) * (KIN / 8)));
     const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
     float m[8];
 #pragma unroll
@@ -318,8 +322,7 @@ __device__ __forceinline__ uint4 mean_rows(const uint16_t *__restrict__ h, const
 // cache more than they gain (447 -> 473).
 constexpr int kAggThreads = 512;
 template <int KIN, bool SMALL>
-__global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *__restrict__ h,
-                                                         uint16_t *__restrict__ agg) {
+__global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const uint16_t *h, uint16_t *agg) {
     constexpr int LPN = KIN / 8;  // lanes per node
     if constexpr (SMALL) {
         griddep_wait();
@@ -330,7 +333,7 @@ __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const ui
         const int32_t *idx = succ ? g.succ_idx : g.pred_idx;
         for (int64_t v = (int64_t)blockIdx.x * NODES + (w >> 1) * (32 / LPN) + lane / LPN; v < g.n_nodes;
              v += (int64_t)gridDim.x * NODES)
-            ((uint4 *)(agg + v * 2 * KIN))[succ * LPN + sub] = mean_rows<KIN>(h, idx, list[v], sub);
+            ((uint4 *)(agg + v * 2 * KIN))[succ * LPN + sub] = mean_rows<KIN, true>(h, idx, list[v], sub);
     } else {
         constexpr int NODES = kAggThreads / LPN;          // nodes per CTA pass
         constexpr int CHUNK = NODES < 128 ? 128 : NODES;  // neighbouring nodes that a CTA takes together
@@ -340,8 +343,8 @@ __global__ void __launch_bounds__(kAggThreads, 3) k_gnn_agg(GnnGraph g, const ui
                 const int64_t v = c0 + i * NODES + threadIdx.x / LPN;
                 if (v >= g.n_nodes) break;
                 uint4 *dst = (uint4 *)(agg + v * 2 * KIN);
-                dst[sub] = mean_rows<KIN>(h, g.pred_idx, g.pred[v], sub);
-                dst[LPN + sub] = mean_rows<KIN>(h, g.succ_idx, g.succ[v], sub);
+                dst[sub] = mean_rows<KIN, false>(h, g.pred_idx, g.pred[v], sub);
+                dst[LPN + sub] = mean_rows<KIN, false>(h, g.succ_idx, g.succ[v], sub);
             }
     }
 }
@@ -373,11 +376,10 @@ __device__ __forceinline__ void st32(void *p, const uint32_t *x) {
 constexpr int kFwdThreads = 512;
 
 template <int KIN>
-__global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint16_t *__restrict__ h_in,
-                                                         const uint16_t *__restrict__ agg,
+__global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint16_t *h_in, const uint16_t *agg,
                                                          const uint16_t *__restrict__ wt,
-                                                         const float *__restrict__ bias,
-                                                         uint16_t *__restrict__ h_out, int32_t *err, bool early) {
+                                                         const float *__restrict__ bias, uint16_t *h_out,
+                                                         int32_t *err, bool early) {
     constexpr int K = 3 * KIN, C = K / 8, N_IT = (128 * C + kFwdThreads - 1) / kFwdThreads;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(8) uint64_t bar;
@@ -394,8 +396,8 @@ __global__ void __launch_bounds__(kFwdThreads) k_gnn_fwd(GnnGraph g, const uint1
             const int64_t v = tile * 128 + r;
             x[i] = make_uint4(0, 0, 0, 0);
             if (r < 128 && v < g.n_nodes)
-                x[i] = c < KIN / 8 ? __ldg((const uint4 *)(h_in + v * KIN) + c)
-                                   : __ldg((const uint4 *)(agg + v * 2 * KIN) + c - KIN / 8);
+                x[i] = c < KIN / 8 ? *((const uint4 *)(h_in + v * KIN) + c)
+                                   : *((const uint4 *)(agg + v * 2 * KIN) + c - KIN / 8);
         }
     };
     if (!early) load(blockIdx.x);
@@ -527,7 +529,8 @@ cudaError_t gnn_layer_fwd(int kin, GnnGraph g, const uint16_t *h_in, const uint1
 // nodes took 285 us (now 89), 165,000 without labels 77 (now 39).
 constexpr int kHeadThreads = 128;
 constexpr int kHeadMaxCtas = 1024;  // partial losses
-__global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uint16_t *__restrict__ h3,
+template <bool OVERLAP>
+__global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uint16_t *h3,
                                                   const float *__restrict__ wh, const float *__restrict__ bh,
                                                   int L, const int8_t *__restrict__ labels, float scale,
                                                   float *logits, float *dlogits, float *dh3, float *loss_part) {
@@ -537,7 +540,7 @@ __global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uin
     __shared__ float sout[kHeadThreads / 32][32 * kMaxLevels];
     for (int i = threadIdx.x; i < kHidden * kMaxLevels; i += blockDim.x) swh[i] = wh[i];
     if (threadIdx.x < kMaxLevels) sbh[threadIdx.x] = bh[threadIdx.x];
-    griddep_wait();  // (in a small batch this launch overlaps the last layer's)
+    if constexpr (OVERLAP) griddep_wait();  // (in a small batch this launch overlaps the last layer's)
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float *so = sout[w];
@@ -553,7 +556,9 @@ __global__ void __launch_bounds__(kHeadThreads) k_gnn_head(GnnGraph g, const uin
             const uint4 *row = (const uint4 *)(h3 + v * kHidden);
 #pragma unroll 2
             for (int c = 0; c < kHidden / 8; c++) {
-                const uint4 q = __ldg(row + c);
+                uint4 q;
+                if constexpr (OVERLAP) q = row[c];
+                else q = __ldg(row + c);
                 const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
@@ -651,8 +656,9 @@ cudaError_t gnn_head(GnnGraph g, const uint16_t *h3, const float *wh, const floa
                      float *loss_part, int n_sm, cudaStream_t st) {
     if (g.n_nodes == 0) return cudaSuccess;
     // the loss is reduced per CTA: a fixed grid keeps the summation order fixed
-    return launch_chain(small_batch(g.n_nodes, n_sm), k_gnn_head, gnn_head_ctas(g.n_nodes, n_sm), kHeadThreads, 0, st, g, h3,
-                        wh, bh, n_levels, labels, scale, logits, dlogits, dh3, loss_part);
+    const bool small = small_batch(g.n_nodes, n_sm);
+    return launch_chain(small, small ? k_gnn_head<true> : k_gnn_head<false>, gnn_head_ctas(g.n_nodes, n_sm), kHeadThreads, 0,
+                        st, g, h3, wh, bh, n_levels, labels, scale, logits, dlogits, dh3, loss_part);
 }
 
 // dWh = h3^T dlogits, dbh = sum dlogits: CTA c reduces a fixed node range in tiles of
