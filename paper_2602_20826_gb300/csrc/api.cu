@@ -190,8 +190,11 @@ struct dagrt_batch {
         int2 *pred, *succ;
         int32_t *pred_idx, *succ_idx, *cursor, *level, *m;
         int64_t *wanc;
-        uint16_t *x, *h[3], *agg[3];  // agg: the layers' aggregated inputs; agg[1] alone serves
-                                       // every layer of a forward pass, training keeps all
+        // h: the layers' outputs, in one block. A forward pass alone runs in place in h[0] and
+        // keeps the aggregated input of the current layer in h[1] and h[2]; training keeps all
+        // three of both, the aggregated ones where the backward pass puts something only once they
+        // are used: agg[0] in cand, agg[1] and agg[2] in dh[0] and dh[1]
+        uint16_t *x, *h[3], *agg[3];
         float *logits, *dlogits, *dh[3], *da, *loss_part;
         int8_t *labels;
         uint8_t *best_level, *cand;
@@ -1130,13 +1133,12 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
             (e = batch_alloc(b, &G.pred_idx, E)) != cudaSuccess || (e = batch_alloc(b, &G.succ_idx, E)) != cudaSuccess ||
             (e = batch_alloc(b, &G.cursor, N)) != cudaSuccess || (e = batch_alloc(b, &G.level, N)) != cudaSuccess ||
             (e = batch_alloc(b, &G.m, N)) != cudaSuccess || (e = batch_alloc(b, &G.wanc, N)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.x, N * kFeat)) != cudaSuccess || (e = batch_alloc(b, &G.h[0], N * kHidden)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.h[1], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.h[2], N * kHidden)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.agg[1], N * 2 * kHidden)) != cudaSuccess ||
+            (e = batch_alloc(b, &G.x, N * kFeat)) != cudaSuccess || (e = batch_alloc(b, &G.h[0], 3 * N * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.logits, N * kMaxLevels)) != cudaSuccess ||
             (e = batch_alloc(b, &G.best_level, N)) != cudaSuccess || (e = batch_alloc(b, &G.cand, 2 * N * kPropStride)) != cudaSuccess ||
             (e = batch_alloc(b, &G.cbest, b->n_dags)) != cudaSuccess || (e = batch_alloc(b, &G.bbest, b->n_dags)) != cudaSuccess)
             return cuda_fail(ctx, e, "allocate proposer state");
+        for (int l = 1; l < 3; l++) G.h[l] = G.h[0] + l * N * kHidden;
         dagrt_schedule_out o;
         std::memset(&o, 0, sizeof o);
         o.level = G.level;
@@ -1156,26 +1158,31 @@ static int gnn_prepare(dagrt_batch *b, bool train) {
         if ((e = batch_alloc(b, &G.dlogits, N * kMaxLevels)) != cudaSuccess ||
             (e = batch_alloc(b, &G.dh[0], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.dh[1], N * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.dh[2], N * kHidden)) != cudaSuccess || (e = batch_alloc(b, &G.da, N * 3 * kHidden)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.agg[0], N * 2 * kFeat)) != cudaSuccess ||
-            (e = batch_alloc(b, &G.agg[2], N * 2 * kHidden)) != cudaSuccess ||
             (e = batch_alloc(b, &G.labels, N)) != cudaSuccess || (e = batch_alloc(b, &G.loss_part, 1024)) != cudaSuccess)
             return cuda_fail(ctx, e, "allocate training state");
+        static_assert(2 * kPropStride == 2 * kFeat * sizeof(uint16_t), "agg[0] takes cand's bytes");
+        G.agg[0] = (uint16_t *)G.cand;
+        G.agg[1] = (uint16_t *)G.dh[0];
+        G.agg[2] = (uint16_t *)G.dh[1];
         G.train = true;
     }
     return DAGRT_OK;
 }
 
-static int gnn_forward(dagrt_batch *b, dagrt_model *md, bool train = false) {
+// *h3: where the last layer's output is
+static int gnn_forward(dagrt_batch *b, dagrt_model *md, const uint16_t **h3, bool train = false) {
     dagrt_ctx *ctx = b->ctx;
     auto &G = b->gnn;
     const GnnGraph g = graph_of(b);
     const int64_t boff[3] = {ParamLayout::b1, ParamLayout::b2, ParamLayout::b3};
     const uint16_t *in = G.x;
     for (int l = 0; l < 3; l++) {
-        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], G.h[l], G.agg[train ? l : 1], b->err, ctx->n_sm,
+        uint16_t *out = G.h[train ? l : 0], *agg = train ? G.agg[l] : G.h[1];
+        CK(gnn_layer_fwd(l == 0 ? kFeat : kHidden, g, in, md->wt[l], md->p + boff[l], out, agg, b->err, ctx->n_sm,
                          ctx->stream), "layer forward");
-        in = G.h[l];
+        in = out;
     }
+    *h3 = in;
     ctx->launches += 6;
     return DAGRT_OK;
 }
@@ -1292,10 +1299,11 @@ extern "C" int dagrt_model_logits(dagrt_batch *b, dagrt_model *md, float *logits
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     int rc = gnn_prepare(b, false);
     if (rc) return rc;
-    if ((rc = gnn_forward(b, md))) return rc;
+    const uint16_t *h3;
+    if ((rc = gnn_forward(b, md, &h3))) return rc;
     const GnnGraph g = graph_of(b);
     float *dst = (flags & DAGRT_PTR_DEVICE) ? logits : b->gnn.logits;
-    CK(gnn_head(g, b->gnn.h[2], md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, nullptr, 0.f, dst, nullptr,
+    CK(gnn_head(g, h3, md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, nullptr, 0.f, dst, nullptr,
                 nullptr, nullptr, ctx->n_sm, ctx->stream), "head");
     ctx->launches++;
     if (flags & DAGRT_PTR_DEVICE) return DAGRT_OK;
@@ -1318,11 +1326,12 @@ static int gnn_grad(dagrt_batch *b, dagrt_model *md, const int8_t *labels, float
     const float scale = nl ? 1.f / (float)nl : 0.f;
     cudaStream_t st = ctx->stream;
     if (N) CK(cudaMemcpyAsync(G.labels, labels, N, cudaMemcpyHostToDevice, st), "copy labels");
-    if ((rc = gnn_forward(b, md, true))) return rc;
+    const uint16_t *h3;
+    if ((rc = gnn_forward(b, md, &h3, true))) return rc;
     const GnnGraph g = graph_of(b);
-    CK(gnn_head(g, G.h[2], md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, G.labels, scale, G.logits, G.dlogits,
+    CK(gnn_head(g, h3, md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, G.labels, scale, G.logits, G.dlogits,
                 G.dh[2], G.loss_part, ctx->n_sm, st), "head");
-    CK(gnn_head_grad(g, G.h[2], G.dlogits, md->L, md->part, md->n_parts, st), "head gradient");
+    CK(gnn_head_grad(g, h3, G.dlogits, md->L, md->part, md->n_parts, st), "head gradient");
     // layer 3 and 2: weight gradients, then the gradient of the layer input
     for (int l = 2; l >= 1; l--) {
         CK(gnn_layer_bwd_dw(kHidden, l, g, G.h[l - 1], G.agg[l], G.h[l], G.dh[l], md->part, md->n_parts, b->err, st), "dW");
@@ -1394,11 +1403,12 @@ extern "C" int dagrt_propose(dagrt_batch *b, dagrt_model *md, int32_t k, int64_t
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     int rc = gnn_prepare(b, false);
     if (rc) return rc;
-    if ((rc = gnn_forward(b, md))) return rc;
+    const uint16_t *h3;
+    if ((rc = gnn_forward(b, md, &h3))) return rc;
     auto &G = b->gnn;
     const GnnGraph g = graph_of(b);
     cudaStream_t st = ctx->stream;
-    CK(gnn_head(g, G.h[2], md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, nullptr, 0.f, G.logits, nullptr,
+    CK(gnn_head(g, h3, md->p + ParamLayout::Wh, md->p + ParamLayout::bh, md->L, nullptr, 0.f, G.logits, nullptr,
                 nullptr, nullptr, ctx->n_sm, st), "head");
     const Plan &pl = b->plan[DAGRT_VAR_PAPER];
     CK(gnn_topk(b->n_dags, b->node_off, G.logits, md->L, md->d_levels, k, pl.rows, pl.nrows, G.best_level, G.cand,

@@ -56,7 +56,7 @@ cudaError_t gnn_features(int32_t n_dags, const int64_t *node_off, const int64_t 
                          const int32_t *level, const int64_t *wanc, const int32_t *m, const int32_t *status,
                          GnnGraph g, uint16_t *x, int n_sm, cudaStream_t st);
 // one layer: h_out = ReLU([h_in | mean_pred h_in | mean_succ h_in] W + b); kin = 16 or 128;
-// agg receives the two means, bf16 [N x 2 kin] (the weight gradients read them)
+// agg receives the two means, bf16 [N x 2 kin] (the weight gradients read them); h_out may be h_in
 cudaError_t gnn_layer_fwd(int kin, GnnGraph g, const uint16_t *h_in, const uint16_t *wt, const float *bias,
                           uint16_t *h_out, uint16_t *agg, int32_t *err, int n_sm, cudaStream_t st);
 // head: logits (and, with labels, loss pieces and dlogits)
