@@ -337,6 +337,8 @@ __device__ __noinline__ int members_large(const A2<SH, ID> w, int variant, uint3
     return np;
 }
 
+constexpr uint32_t kOwnSucc = 8;  // successors that a lane releases by itself (groups of more than 32)
+
 // Alg.2 over all groups of a DAG with Lemma 1 and Theorem 1, by one warp. The group step is
 // a serial chain, so it is written for latency: every lane runs the scalar part on the same
 // values (no divergence, no hand-over between lanes), a node's record is one 16-byte load,
@@ -713,7 +715,24 @@ __device__ __forceinline__ void alg2_warp(const A2<SH, ID> &w, const SchedArgs &
                     finish_own(r, idm, j, mr);
                 }
                 i += __popc(live);
-                release_lanes(__ballot_sync(FULL, q.x && (q.w & 0xffffu)));
+                uint32_t dl = q.x ? q.w & 0xffffu : 0u;
+                if constexpr (sizeof(ID) == 2) {
+                    // members with few successors (leaves of wide graphs) each by their own lane, the
+                    // counts by atomics on their words: targets of different members may coincide
+                    uint32_t freed = 0;
+                    for (uint32_t e = 0; dl <= kOwnSucc && e < dl; e++) {
+                        const uint32_t t = w.col(q.z + e), sh = 16 * (t & 1);
+                        const uint32_t old = atomicSub(w.template at<uint32_t>(w.o_cnt) + (t >> 1), 1u << sh);
+                        if ((old >> sh & 0xffffu) != 1u) continue;
+                        freed++;
+                        atomicOr(w.rel() + (t >> 5), 1u << (t & 31));
+                        if constexpr (SUM) atomicOr(w.sum() + (t >> 11), 1u << ((t >> 6) & 31));
+                    }
+                    if constexpr (FULL_OUT) nrel += __reduce_add_sync(FULL, freed);
+                    if (dl <= kOwnSucc) dl = 0;
+                    __syncwarp();
+                }
+                release_lanes(__ballot_sync(FULL, dl > 0));
             }
         }
         if constexpr (FULL_OUT) {
