@@ -1,9 +1,8 @@
 // dagrt_internal.cuh -- device-side building blocks shared by the libdagrt kernels.
 //
-// A "team" is the set of threads that cooperates on one DAG: either one warp (NT == 32,
-// several independent teams per CTA, workspace in shared memory) or a whole CTA
-// (NT == blockDim.x, workspace in shared or global memory). Algorithms are written once
-// against Team<NT> and run unchanged on both.
+// A "team" is the set of threads that cooperates on one DAG: one warp (several independent teams
+// per CTA, sched_warp.cuh) or a whole CTA, here Team<NT>: NT == blockDim.x, workspace in shared or
+// global memory.
 #pragma once
 
 #include <cstdint>
@@ -22,32 +21,25 @@ __host__ __device__ constexpr int64_t align_up(int64_t x, int64_t a) { return (x
 // ------------------------------------------------------------------ team
 template <int NT>
 struct Team {
-    static constexpr int N = NT;
     static constexpr int NW = NT / 32;
     int t;              // rank in team
-    uint64_t *red;      // NW words of shared scratch (NT > 32 only)
+    uint64_t *red;      // NW words of shared scratch
 
     __device__ __forceinline__ int lane() const { return t & 31; }
     __device__ __forceinline__ int warp() const { return t >> 5; }
-    __device__ __forceinline__ void sync() const {
-        if constexpr (NT == 32) __syncwarp(); else __syncthreads();
-    }
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
 
     template <class Op>
     __device__ __forceinline__ uint64_t reduce(uint64_t v, Op op) const {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(FULL, v, o));
-        if constexpr (NT == 32) {
-            return v;
-        } else {
-            if (lane() == 0) red[warp()] = v;
-            __syncthreads();
-            uint64_t r = red[0];
+        if (lane() == 0) red[warp()] = v;
+        __syncthreads();
+        uint64_t r = red[0];
 #pragma unroll
-            for (int i = 1; i < NW; i++) r = op(r, red[i]);
-            __syncthreads();
-            return r;
-        }
+        for (int i = 1; i < NW; i++) r = op(r, red[i]);
+        __syncthreads();
+        return r;
     }
     __device__ __forceinline__ uint64_t sum(uint64_t v) const {
         return reduce(v, [](uint64_t a, uint64_t b) { return a + b; });
@@ -55,13 +47,7 @@ struct Team {
     __device__ __forceinline__ uint64_t maxu(uint64_t v) const {
         return reduce(v, [](uint64_t a, uint64_t b) { return a > b ? a : b; });
     }
-    __device__ __forceinline__ uint64_t minu(uint64_t v) const {
-        return reduce(v, [](uint64_t a, uint64_t b) { return a < b ? a : b; });
-    }
-    __device__ __forceinline__ bool any(bool p) const {
-        if constexpr (NT == 32) return __any_sync(FULL, p);
-        else return __syncthreads_or(p) != 0;
-    }
+    __device__ __forceinline__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
 
     // Inclusive scan of v across the team with an associative op; *total gets the
     // reduction of all values.
@@ -72,29 +58,17 @@ struct Team {
             uint64_t x = __shfl_up_sync(FULL, v, o);
             if (lane() >= o) v = op(v, x);
         }
-        if constexpr (NT == 32) {
-            *total = __shfl_sync(FULL, v, 31);
-            return v;
-        } else {
-            if (lane() == 31) red[warp()] = v;
-            __syncthreads();
-            uint64_t carry = 0, tot = 0;
-            bool have = false;
-            for (int i = 0; i < NW; i++) {
-                if (i == warp()) { carry = tot; have = i > 0; }
-                tot = i == 0 ? red[0] : op(tot, red[i]);
-            }
-            __syncthreads();
-            *total = tot;
-            return have ? op(carry, v) : v;
+        if (lane() == 31) red[warp()] = v;
+        __syncthreads();
+        uint64_t carry = 0, tot = 0;
+        bool have = false;
+        for (int i = 0; i < NW; i++) {
+            if (i == warp()) { carry = tot; have = i > 0; }
+            tot = i == 0 ? red[0] : op(tot, red[i]);
         }
-    }
-    // Exclusive prefix sum of non-negative counts.
-    __device__ __forceinline__ uint32_t excl_sum(uint32_t v, uint32_t *total) const {
-        uint64_t tot;
-        uint64_t inc = incl_scan(v, [](uint64_t a, uint64_t b) { return a + b; }, &tot);
-        *total = (uint32_t)tot;
-        return (uint32_t)(inc - v);
+        __syncthreads();
+        *total = tot;
+        return have ? op(carry, v) : v;
     }
 };
 
@@ -112,15 +86,10 @@ __device__ void team_scan_inplace(const Team<NT> &tm, T *arr, int n, Op op, bool
         uint64_t tot;
         uint64_t s = tm.incl_scan(v, op, &tot);
         int last = min(n - base, NT) - 1;
-        uint64_t chunk_tot;
-        if constexpr (NT == 32) {
-            chunk_tot = __shfl_sync(FULL, s, last);
-        } else {
-            if (tm.t == last) tm.red[0] = s;
-            __syncthreads();
-            chunk_tot = tm.red[0];
-            __syncthreads();
-        }
+        if (tm.t == last) tm.red[0] = s;
+        __syncthreads();
+        const uint64_t chunk_tot = tm.red[0];
+        __syncthreads();
         if (i < n) arr[idx] = (T)(have ? op(carry, s) : s);
         carry = have ? op(carry, chunk_tot) : chunk_tot;
         have = true;
@@ -225,25 +194,8 @@ __device__ __forceinline__ uint64_t exec_time(uint64_t x, uint32_t k, uint32_t m
     return c < 1 ? 1 : c;
 }
 
-// Largest load p in [1, L-1] that finishes within R ticks on min(p, S) SMs (S <= M):
-// closed form of the node-segmentation size (see the scheduler for the derivation).
 __device__ __forceinline__ uint64_t udiv(uint64_t n, uint64_t d) {  // 32-bit divide when both fit
     return (n >> 32) == 0 && (d >> 32) == 0 ? (uint64_t)((uint32_t)n / (uint32_t)d) : n / d;
-}
-
-__device__ __forceinline__ uint64_t split_size(uint64_t L, uint32_t k, uint32_t S, uint64_t R) {
-    uint64_t a = 64ull * S - (uint64_t)k * (S - 1);
-    uint64_t x2 = udiv(64ull * S * R, a);       // largest x >= S with x*a <= 64*S*R
-    uint64_t p;
-    if (x2 >= S) {
-        p = x2;
-    } else {                                    // k < 64 here; the answer is below S
-        uint64_t x1 = udiv(64ull * R - k, 64ull - k);
-        p = x1 < (uint64_t)S - 1 ? x1 : (uint64_t)S - 1;
-    }
-    if (p > L - 1) p = L - 1;
-    if (p < 1) p = 1;
-    return p;
 }
 
 // The largest dynamic shared memory a launch of `kern` may take on the current device: the
