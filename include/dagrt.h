@@ -19,8 +19,9 @@
  *  - Every call returns DAGRT_OK (0) or a negative DAGRT_E_* code and never aborts; the
  *    message of the last failure is available from dagrt_last_error().
  *  - All device work is enqueued on the context's stream in order. Calls given host
- *    pointers copy through device staging buffers and synchronise that stream before they
- *    return. Calls given device pointers (DAGRT_PTR_DEVICE) only enqueue work; their
+ *    pointers copy through staging buffers (small outputs are written straight to pinned
+ *    host memory) and synchronise that stream before they return; dagrt_load_csr is the
+ *    exception, see there. Calls given device pointers (DAGRT_PTR_DEVICE) only enqueue work; their
  *    outputs are valid once the caller synchronises the stream.
  *  - The caller owns every buffer it passes; the library owns the staging and scratch
  *    memory inside a context and a batch, and frees it in dagrt_destroy/dagrt_batch_free.
@@ -111,7 +112,11 @@ int64_t dagrt_launch_count(const dagrt_ctx *ctx);
  *   k64[total_nodes] uint8    k_i in [0, 64]
  * With DAGRT_PTR_DEVICE the arrays are device pointers that the batch reads in place and
  * that must stay valid and unchanged until dagrt_batch_free; otherwise they are host
- * pointers that are copied. The offsets are checked here (E_INVAL); per-DAG graph checks
+ * pointers that are copied: the arrays are the caller's again when the call returns. Arrays
+ * of at most 64 KB are copied to pinned memory first and only enqueued from there, so a
+ * call whose arrays are all that small does not wait for the stream, and an asynchronous
+ * error of its copy shows in a later call.
+ * The offsets are checked here (E_INVAL); per-DAG graph checks
  * run on the device inside dagrt_schedule and are reported there, per DAG. */
 int dagrt_load_csr(dagrt_ctx *ctx, int32_t n_dags, const int64_t *node_off,
                    const int64_t *edge_off, const int32_t *row_ptr, const int32_t *col,

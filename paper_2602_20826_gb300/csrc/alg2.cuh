@@ -356,9 +356,10 @@ constexpr uint32_t kOwnSucc = 8;  // successors that a lane releases by itself (
 // tick of load adds at most one tick of time: the part takes exactly R.
 //
 // What bounds it: the latency of one warp's dependent instructions (a third of the stalls are
-// shared-memory loads, the rest fixed-latency arithmetic). Against one lane walking id-indexed
-// arrays, a group went from 3,800 to 2,100-2,500 cycles and a call of 10,000 DAGs of 20-200
-// nodes from 1.80 to 1.42 ms; 300 DAGs of 100-1,000 nodes from 3.7 to 2.4 ms.
+// shared-memory loads, the rest fixed-latency arithmetic). One lane walking id-indexed arrays took
+// 3,800 cycles a group, this 1,500 in shared memory and 2,600 in a global workspace; by itself
+// that took a call of 10,000 DAGs of 20-200 nodes from 1.80 to 1.42 ms (now 0.67, by what
+// sched_warp.cuh changed).
 //
 // FULL_OUT: another variant than the paper's, no plan, or some of the outputs that few callers
 // ask for (rows, segments, group times, extra dependencies); without it the chain does not

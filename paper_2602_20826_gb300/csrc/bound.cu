@@ -116,10 +116,12 @@ __device__ __forceinline__ uint32_t gen_alloc(const BoundArgs &a, int d, int c, 
 // it: no chunk index is needed, nor scratch in global memory, and partial bounds add up in
 // shared memory (Theorem 1's sum splits at group ends).
 //
-// What bounds it is instruction issue. Eq.1's division is out of the inner loop: generated
-// candidates look {C, m} up in a table of the row's few possible choices (built by one lane
-// per row), and a byte m <= M divides by 64 m with a multiply and a shift. Per candidate and
-// row that leaves SplitMix64 (two 64-bit multiplications) or ten instructions. Two candidates
+// Eq.1's division is out of the inner loop: generated candidates look {C, m} up in a table of the
+// row's few possible choices, and a byte m <= M divides by 64 m with a multiply and a shift. Per
+// candidate and row that leaves SplitMix64 (two 64-bit multiplications) or ten instructions. What
+// bounds it: perturbations issue in 59% of the cycles with 16 warps an SM, between dependent
+// instructions for the most part; bytes of 74 candidates in 42% with 22 warps, which wait at the
+// DAGs' barriers (3.7 of 13 cycles between a warp's instructions) and for loads. Two candidates
 // a lane above 32 allocations (one: 359 us instead of 279 below). Windows of 32 rows: 64 and
 // 128 take 65 and 92 us instead of 58 on the second workload, the first does not care.
 // 500 DAGs of 100-1,000 nodes x 256 perturbations: 3.06 -> 0.28 ms; 1,000 DAGs of 20-200 nodes
@@ -1126,7 +1128,7 @@ cudaError_t bound_launch(const BoundArgs &a, const ChunkArgs *ch, int n_sm, cuda
         cfg.numAttrs = 1;
         if ((e = cudaLaunchKernelEx(&cfg, k_bound_finish, a, *ch)) != cudaSuccess) return e;
         *launches += 2;
-        return cudaSuccess;  // k_bound_finish evaluated the DAGs that need 64-bit sums
+        return cudaSuccess;  // (the items evaluate the DAGs that need 64-bit sums too)
     }
     using K = void (*)(BoundArgs, int);
     if (a.gen && a.gen_mode == DAGRT_SEARCH_EXHAUSTIVE) {

@@ -8,8 +8,9 @@
 // level barriers (176,000 -> 49,000 cycles at 200 nodes); the (W^anc, id) order is a bitonic
 // network in registers (45,000 -> 4,000); every lane reads the blocks of its own nodes off the
 // joins' rows (42,000 -> 10,000); a round of Alg.1 asks each node whether its only in-block
-// predecessor has been selected (77,000 -> 26,000). Alg.2 is then 65% of a DAG's 396,000 cycles.
-// 10,000 DAGs of 20-200 nodes, load and schedule: 1.42 -> 0.69 ms (four warps a CTA, five CTAs
+// predecessor has been selected (77,000 -> 26,000), large blocks apart (peel_solo). Alg.2 is then
+// 65% of a DAG's 396,000 cycles.
+// 10,000 DAGs of 20-200 nodes, load and schedule: 1.42 -> 0.67 ms (four warps a CTA, five CTAs
 // an SM; 6 CTAs at 80 registers 0.93, 2 warps 0.83, size classes of 32 nodes 0.85 against 0.83
 // when these were timed).
 #pragma once
